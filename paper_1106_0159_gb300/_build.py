@@ -16,7 +16,8 @@ CSRC = os.path.join(HERE, "csrc")
 LIBDIR = os.path.join(HERE, "_lib")
 LIB = os.path.join(LIBDIR, "libsht.so")
 LIBDIR_CHECK = os.path.join(HERE, "_lib_check")
-SOURCES = ["sht_plan.cu", "legendre.cu", "legendre_tc.cu", "legendre_df.cu", "ringfft.cu", "diag.cu", "noalloc.cu", "spin.cu", "batch.cu"]
+SOURCES = ["sht_plan.cu", "legendre.cu", "legendre_tc.cu", "legendre_tc_anal.cu",
+           "legendre_df.cu", "ringfft.cu", "diag.cu", "noalloc.cu", "spin.cu", "batch.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -484,6 +484,68 @@ __global__ void reduce_blocks_kernel(const double2 *__restrict__ partial, const 
     }
 }
 
+// ---------------------------------------------------------------- columns left by the tensor-core kernels
+//
+// The tensor-core kernels cut their operands into digits below one exponent, which cannot carry a
+// value that is not finite, subnormal or near the ends of the FP64 range.  They mark such (m, map)
+// columns in fix[m][16], and these kernels redo them with the sums above; without marks (every
+// ordinary input) each CTA reads its 16 marks and ends.
+
+__global__ void __launch_bounds__(SYN_T) legendre_synth_fix_kernel(SynArgs A, const int *__restrict__ fix, int nmaps)
+{
+    __shared__ Coef C;
+    __shared__ double2 s_a[1][CHL];
+    const int m = blockIdx.x;
+    const int64_t dstride = (int64_t)A.nrings * (A.mmax + 1);
+    for (int g = 0; g < nmaps; ++g) {
+        if (!fix[m * 16 + g]) continue;
+        SynArgs B = A;
+        B.alm += (int64_t)g * A.nalm;
+        B.delta += (int64_t)g * dstride;
+        for (int blk = 0; blk < A.nblk; ++blk) {
+            if (m <= A.mR && A.s[blk * SYN_T] < POLAR_SIN)
+                synth_body<1, true>(B, m, blk, C, s_a);
+            else
+                synth_body<1, false>(B, m, blk, C, s_a);
+        }
+    }
+}
+
+// A.partial: scratch of nblk x nalm_part coefficients from index idx0 on, each m its own part of it
+__global__ void __launch_bounds__(ANA_T) legendre_anal_fix_kernel(AnaArgs A, const int *__restrict__ fix, int nmaps,
+                                                                  int m0, double2 *__restrict__ alm)
+{
+    constexpr int NW = ANA_T / 32;
+    __shared__ Coef C;
+    __shared__ double s_red[NW][CHL][2];
+    const int m = m0 + blockIdx.x;
+    const int64_t dstride = (int64_t)A.nrings * (A.mmax + 1);
+    const int64_t base = (int64_t)m * (2 * A.lmax + 3 - m) / 2;
+    for (int g = 0; g < nmaps; ++g) {
+        if (!fix[m * 16 + g]) continue;
+        AnaArgs B = A;
+        B.delta += (int64_t)g * dstride;
+        for (int blk = 0; blk < A.nblk; ++blk) {
+            if (m <= A.mR && A.s[blk * ANA_T] < POLAR_SIN)
+                anal_body<1, 1, true>(B, m, blk, C, s_red);
+            else
+                anal_body<1, 1, false>(B, m, blk, C, s_red);
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i <= A.lmax - m; i += ANA_T) {
+            double re = 0.0, im = 0.0;
+            for (int blk = 0; blk < A.nblk; ++blk) {
+                const double2 v = A.partial[(int64_t)blk * A.part_blk_stride + base + i];
+                re += v.x;
+                im += v.y;
+            }
+            const double c = A.cfac[base + i];
+            alm[(int64_t)g * A.nalm + base + i] = make_double2(c * re, m == 0 ? 0.0 : c * im);
+        }
+        __syncthreads();
+    }
+}
+
 // ---------------------------------------------------------------- batched form (many plans)
 //
 // One persistent launch runs the Legendre tiles of many transforms (uneven lmax, any number of
@@ -689,6 +751,56 @@ cudaError_t launch_legendre_anal(const Plan &p, const double2 *delta, double2 *p
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
+}
+
+cudaError_t launch_legendre_synth_fix(const Plan &p, const double2 *alm, double2 *delta, const int *fix, int nmaps,
+                                      cudaStream_t st)
+{
+    SynArgs A{};
+    A.alm = alm;
+    A.delta = delta;
+    A.slotN = p.d_slotN;
+    A.slotS = p.d_slotS;
+    A.u = p.d_u;
+    A.s = p.d_s;
+    A.alpha = p.d_alpha;
+    A.cfac = p.d_cfac;
+    A.rein = p.d_rein;
+    A.mR = p.mR;
+    A.nslots = p.nslots;
+    A.nblk = (p.nslots + SYN_T - 1) / SYN_T;
+    A.lmax = p.lmax;
+    A.mmax = p.mmax;
+    A.nrings = p.nrings;
+    A.nalm = p.nalm;
+    legendre_synth_fix_kernel<<<(unsigned)(p.mmax + 1), SYN_T, 0, st>>>(A, fix, nmaps);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_legendre_anal_fix(const Plan &p, const double2 *delta, double2 *alm, double2 *partial, const int *fix,
+                                     int nmaps, int m0, int m1, int64_t idx0, int64_t nalm_part, cudaStream_t st)
+{
+    AnaArgs A{};
+    A.delta = delta;
+    A.partial = partial - idx0;
+    A.slotN = p.d_slotN;
+    A.slotS = p.d_slotS;
+    A.u = p.d_u;
+    A.s = p.d_s;
+    A.alpha = p.d_alpha;
+    A.cfac = p.d_cfac;
+    A.rein = p.d_rein;
+    A.mR = p.mR;
+    A.nslots = p.nslots;
+    A.nblk = (p.nslots + ANA_T - 1) / ANA_T;
+    A.lmax = p.lmax;
+    A.mmax = p.mmax;
+    A.nrings = p.nrings;
+    A.nalm = p.nalm;
+    A.part_map_stride = 0;
+    A.part_blk_stride = nalm_part;
+    legendre_anal_fix_kernel<<<(unsigned)(m1 - m0), ANA_T, 0, st>>>(A, fix, nmaps, m0, alm);
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- batched form: host side

@@ -298,160 +298,34 @@ __global__ void __launch_bounds__(DF_T) legendre_anal_df_kernel(DfArgs A)
 // a_lm = c_lm * sum over blocks of (hi + lo).  The blocks are added in order as double-float
 // pairs on the FP32 pipe (widening each partial to FP64 and adding there made this kernel
 // FP64-bound: four conversions and four adds per complex value and block) and the sum is widened
-// once.  Partial (block, map g, index i) sits at bk * blk_stride + g * map_stride + i * idx_stride:
-// [block][map][index] from the double-float kernel, [block][index][map] from the tensor-core one;
-// threads walk the innermost of the two.  For i < fp64_lim (m <= mR of a polar plan) the Reinsch
-// kernel's FP64 partial polar[g * polar_stride + i], split into hi + lo, stands for blocks
-// 0 .. polar_blocks - 1.
-__global__ void reduce_blocks_df_kernel(const float4 *__restrict__ partial, const double2 *__restrict__ polar,
-                                        int64_t polar_stride, int polar_blocks, const double *__restrict__ cfac,
+// once.  Partial (block, map g, index i) sits at bk * blk_stride + g * nalm + i.  For i < fp64_lim
+// (m <= mR of a polar plan) block 0 holds the Reinsch kernel's FP64 partial instead.
+__global__ void reduce_blocks_df_kernel(const float4 *__restrict__ partial, const double *__restrict__ cfac,
                                         double2 *__restrict__ alm, int nblk, int64_t nalm, int nmaps, int lmax,
-                                        int64_t blk_stride, int64_t map_stride, int64_t idx_stride, int64_t fp64_lim,
-                                        int64_t i0, int64_t nidx)
+                                        int64_t blk_stride, int64_t fp64_lim)
 {
-    // coefficient indices i0 .. i0 + nidx - 1; the partial sums are indexed from i0
-    const int64_t total = nidx * nmaps;
-    const bool maps_inner = map_stride < idx_stride;
+    const int64_t total = nalm * nmaps;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        int64_t g, il;
-        if (maps_inner) {
-            il = t / nmaps;
-            g = t - il * nmaps;
-        } else {
-            g = t / nidx;
-            il = t - g * nidx;
-        }
-        const int64_t i = i0 + il;
-        const float4 *src = partial + g * map_stride + il * idx_stride;
+        const int64_t g = t / nalm, i = t - g * nalm;
+        const float4 *src = partial + t;
         float2 re, im;
-        int bk0 = 1;
         if (i < fp64_lim) {
-            const double2 d = polar[g * polar_stride + i];
+            const double2 d = *reinterpret_cast<const double2 *>(src);
             re = d2df(d.x);
             im = d2df(d.y);
-            bk0 = polar_blocks;
         } else {
             const float4 v = src[0];
             re = make_float2(v.x, v.y);
             im = make_float2(v.z, v.w);
         }
 #pragma unroll 4
-        for (int bk = bk0; bk < nblk; ++bk) {
+        for (int bk = 1; bk < nblk; ++bk) {
             const float4 v = src[(int64_t)bk * blk_stride];
             re = df_add(re, make_float2(v.x, v.y));
             im = df_add(im, make_float2(v.z, v.w));
         }
         const double c = cfac[i];
-        alm[g * nalm + i] = make_double2(c * widen_df(re), i <= lmax ? 0.0 : c * widen_df(im));
-    }
-}
-
-// Polar slots of the precision-form synthesis (eq. DeltaDef): for m <= mR, slots 0 .. 127 (the
-// first block of the tensor-core synthesis), Reinsch's form of the recurrence in FP64 and the
-// sums E, O = sum over l of a_lm lambda_lm (l - m even, odd) in double-float on the FP32 pipe,
-// for up to NM maps per launch; Delta_N = E + O, Delta_S = E - O.  One CTA per m.
-constexpr int DFS_T = 128;  // threads = slots per CTA
-
-struct DfSynArgs {
-    const double2 *alm;    // [nmaps][nalm], first map of this launch
-    double2 *delta;        // [nmaps][nrings][mmax+1]
-    const int *slotN, *slotS;
-    const double *u, *s, *alpha;
-    const double3 *rein;   // Reinsch coefficients (beta_l, rho_l, b0_l) for m <= mR
-    int nslots, lmax, mmax, nrings, nmaps;
-    int64_t nalm;
-};
-
-template <int NM>
-__global__ void __launch_bounds__(DFS_T) synth_df_polar_kernel(DfSynArgs A)
-{
-    __shared__ double co[3][DF_CHL];     // beta_l, rho_l, b0_l of the chunk
-    __shared__ float4 sa[NM][DF_CHL];    // a_lm of the chunk as (re_hi, re_lo, im_hi, im_lo)
-    const int m = blockIdx.x;
-    const int tid = threadIdx.x;
-    const int slot = (int)blockIdx.y * DFS_T + tid;  // block y of the polar slot blocks
-    const bool active = slot < A.nslots;
-    const int L = A.lmax;
-    const int64_t base = (int64_t)m * (2 * L + 3 - m) / 2;
-
-    double u = 0.0, y1 = 0.0, y2 = 0.0;  // y1: lambda_(l-1), y2: D_(l-1)
-    int k = 0;
-    if (active) {
-        u = A.u[slot];
-        double y0;
-        sectoral_start(A.s[slot], A.alpha[base], m, y0, k);
-        y2 = y0;  // D_(m-1) = lambda_m with lambda_(m-1) = 0
-    }
-    float2 acc[2][NM][2];  // [E, O][map][re, im]
-#pragma unroll
-    for (int p = 0; p < 2; ++p)
-#pragma unroll
-        for (int g = 0; g < NM; ++g) acc[p][g][0] = acc[p][g][1] = make_float2(0.f, 0.f);
-
-    for (int l0 = m; l0 <= L; l0 += DF_CHL) {
-        const int nl = min(DF_CHL, L - l0 + 1);
-        __syncthreads();
-        for (int i = tid; i < DF_CHL * (NM + 1); i += DFS_T) {
-            const int row = i / DF_CHL, j = i - row * DF_CHL;
-            const int64_t ix = base + (l0 - m) + j;
-            if (row == 0) {
-                const double3 c = (j < nl) ? A.rein[ix] : make_double3(0.0, 0.0, 0.0);
-                co[0][j] = c.x;
-                co[1][j] = c.y;
-                co[2][j] = c.z;
-            } else {
-                const int g = row - 1;
-                double2 a = make_double2(0.0, 0.0);
-                if (j < nl && g < A.nmaps) a = A.alm[(int64_t)g * A.nalm + ix];
-                const float2 re = d2df(a.x), im = d2df(m == 0 ? 0.0 : a.y);
-                sa[g][j] = make_float4(re.x, re.y, im.x, im.y);
-            }
-        }
-        __syncthreads();
-        for (int j0 = 0; j0 < nl; j0 += 16) {
-            const bool scaled = __any_sync(0xffffffffu, k < 0);
-            const int jn = min(j0 + 16, nl);
-            // steps in pairs: j even is l - m even (l0 - m is a multiple of 32), j + 1 odd
-            for (int j = j0; j < jn; j += 2) {
-#pragma unroll
-                for (int p = 0; p < 2; ++p) {
-                    if (j + p < jn) {
-                        // D_l = (1 + rho_l) D_(l-1) + g_l lambda_(l-1), lambda_l = lambda_(l-1) + D_l
-                        const double gl = fma(-co[0][j + p], u, co[2][j + p]);
-                        const double t = fma(gl, y1, y2);
-                        y2 = fma(co[1][j + p], y2, t);
-                        y1 = y1 + y2;
-                        const float2 yd = (active && !(scaled && k < 0)) ? d2df(y1) : make_float2(0.f, 0.f);
-#pragma unroll
-                        for (int g = 0; g < NM; ++g) {
-                            const float4 a = sa[g][j + p];
-                            acc[p][g][0] = df_add(acc[p][g][0], df_mul(yd, make_float2(a.x, a.y)));
-                            acc[p][g][1] = df_add(acc[p][g][1], df_mul(yd, make_float2(a.z, a.w)));
-                        }
-                    }
-                }
-            }
-            if (scaled && k < 0 && max(dexp(y1), dexp(y2)) > RESCALE_THR) {
-                y1 *= 0x1p-512;
-                y2 *= 0x1p-512;
-                k += 1;
-            }
-        }
-    }
-    if (active) {
-        const int rn = A.slotN[slot], rs = A.slotS[slot];
-        const int64_t mstride = A.mmax + 1;
-#pragma unroll
-        for (int g = 0; g < NM; ++g) {
-            if (g >= A.nmaps) continue;
-            const double er = widen_df(acc[0][g][0]), ei = widen_df(acc[0][g][1]);
-            const double orr = widen_df(acc[1][g][0]), oi = widen_df(acc[1][g][1]);
-            double2 *d = A.delta + (int64_t)g * A.nrings * mstride;
-            if (rn >= 0 && SHT_CHK(rn < A.nrings && m <= A.mmax))
-                d[(int64_t)rn * mstride + m] = make_double2(er + orr, ei + oi);
-            if (rs >= 0 && SHT_CHK(rs < A.nrings && m <= A.mmax))
-                d[(int64_t)rs * mstride + m] = make_double2(er - orr, ei - oi);
-        }
+        alm[t] = make_double2(c * widen_df(re), i <= lmax ? 0.0 : c * widen_df(im));
     }
 }
 
@@ -497,56 +371,6 @@ DfArgs df_args(const Plan &p)
 
 }  // namespace
 
-cudaError_t launch_reduce_blocks_df(const float4 *partial, const double2 *polar, int64_t polar_stride,
-                                    int polar_blocks, const double *cfac, double2 *alm, int nblk, int64_t nalm,
-                                    int nmaps, int lmax, int64_t blk_stride, int64_t map_stride, int64_t idx_stride,
-                                    int64_t fp64_lim, cudaStream_t st, int64_t i0, int64_t nidx)
-{
-    if (nidx < 0) nidx = nalm - i0;
-    const int64_t total = nidx * nmaps;
-    const int rgrid = (int)std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, 152 * 16));
-    reduce_blocks_df_kernel<<<rgrid, 256, 0, st>>>(partial, polar, polar_stride, polar_blocks, cfac, alm, nblk, nalm,
-                                                   nmaps, lmax, blk_stride, map_stride, idx_stride, fp64_lim, i0, nidx);
-    return cudaGetLastError();
-}
-
-// The precision-form synthesis of the polar slots 0 .. 127 for m <= mR (nothing when the plan's
-// first ring is not polar), up to 8 maps per launch.
-cudaError_t launch_legendre_synth_df_polar(const Plan &p, const double2 *alm, double2 *delta, int nmaps,
-                                           cudaStream_t st, int *nlaunch)
-{
-    *nlaunch = 0;
-    if (p.mR < 0 || !p.polar_first_slot) return cudaSuccess;
-    DfSynArgs A{};
-    A.slotN = p.d_slotN;
-    A.slotS = p.d_slotS;
-    A.u = p.d_u;
-    A.s = p.d_s;
-    A.alpha = p.d_alpha;
-    A.rein = p.d_rein;
-    A.nslots = p.nslots;
-    A.lmax = p.lmax;
-    A.mmax = p.mmax;
-    A.nrings = p.nrings;
-    A.nalm = p.nalm;
-    const int64_t dstride = (int64_t)p.nrings * (p.mmax + 1);
-    for (int g0 = 0; g0 < nmaps;) {
-        const int nm = std::min(8, nmaps - g0);
-        A.nmaps = nm;
-        A.alm = alm + (int64_t)g0 * p.nalm;
-        A.delta = delta + (int64_t)g0 * dstride;
-        if (nm > 4)
-            synth_df_polar_kernel<8><<<dim3((unsigned)(p.mR + 1), (unsigned)p.polar_syn_blocks), DFS_T, 0, st>>>(A);
-        else
-            synth_df_polar_kernel<4><<<dim3((unsigned)(p.mR + 1), (unsigned)p.polar_syn_blocks), DFS_T, 0, st>>>(A);
-        ++*nlaunch;
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        g0 += nm;
-    }
-    return cudaSuccess;
-}
-
 cudaError_t configure_df_kernels()
 {
     cudaError_t e = configure_df<32, false>();
@@ -556,35 +380,6 @@ cudaError_t configure_df_kernels()
     if (e == cudaSuccess) e = configure_df<16, true>();
     if (e == cudaSuccess) e = configure_df<8, true>();
     return e;
-}
-
-int legendre_anal_df_polar_slots() { return DF_T; }
-
-// The Reinsch-form analysis of slots 0 .. 255 for m <= mR of a polar plan, in double-float:
-// a_lm / c_lm of map g at polar[g * polar_stride + index], index < index(mR + 1, mR + 1),
-// for groups of SHT_TUNE_DF_MAPS maps.
-cudaError_t launch_legendre_anal_df_polar(const Plan &p, const double2 *delta, double2 *polar, int64_t polar_stride,
-                                          int nmaps, cudaStream_t st, int *nlaunch)
-{
-    *nlaunch = 0;
-    DfArgs A = df_args(p);
-    if (A.mR < 0) return cudaSuccess;
-    A.nblk = 1;
-    A.polar_stride = polar_stride;
-    const int64_t dstride = (int64_t)p.nrings * (p.mmax + 1);
-    for (int g0 = 0; g0 < nmaps;) {
-        const int nm = std::min(p.tune[SHT_TUNE_DF_MAPS], nmaps - g0);
-        A.nmaps = nm;
-        A.delta = delta + (int64_t)g0 * dstride;
-        A.polar = polar + (int64_t)g0 * polar_stride;
-        cudaError_t e = nm > 8 ? launch_df_group<32, true>(p, A, st)
-                        : nm > 4 ? launch_df_group<16, true>(p, A, st)
-                                 : launch_df_group<8, true>(p, A, st);
-        ++*nlaunch;
-        if (e != cudaSuccess) return e;
-        g0 += nm;
-    }
-    return cudaSuccess;
 }
 
 int legendre_anal_df_nblk(const Plan &p) { return (p.nslots + DF_T - 1) / DF_T; }
@@ -617,18 +412,29 @@ cudaError_t launch_legendre_anal_df(const Plan &p, const double2 *delta, double2
         g0 += nm;
     }
     int64_t fp64_lim = 0;
-    if (A.mR >= 0) {  // FP64 partials in place of block 0 for m <= mR (16 bytes, as a float4)
-        int n = 0;
-        cudaError_t e = launch_legendre_anal_df_polar(p, delta, (double2 *)partial, p.nalm, nmaps, st, &n);
-        *nlaunch += n;
-        if (e != cudaSuccess) return e;
+    if (A.mR >= 0) {  // Reinsch form of slots 0 .. 255: FP64 partials in place of block 0 for m <= mR (16 bytes too)
+        A.nblk = 1;
+        A.polar_stride = p.nalm;
+        for (g0 = 0; g0 < nmaps;) {
+            const int nm = std::min(p.tune[SHT_TUNE_DF_MAPS], nmaps - g0);
+            A.nmaps = nm;
+            A.delta = delta + (int64_t)g0 * dstride;
+            A.polar = (double2 *)partial + (int64_t)g0 * p.nalm;
+            cudaError_t e = nm > 8 ? launch_df_group<32, true>(p, A, st)
+                            : nm > 4 ? launch_df_group<16, true>(p, A, st)
+                                     : launch_df_group<8, true>(p, A, st);
+            ++*nlaunch;
+            if (e != cudaSuccess) return e;
+            g0 += nm;
+        }
         fp64_lim = (int64_t)(A.mR + 1) * (2 * (int64_t)p.lmax + 3 - (A.mR + 1)) / 2;  // index(mR+1, mR+1)
     }
-    cudaError_t e = launch_reduce_blocks_df((const float4 *)partial, (const double2 *)partial, p.nalm, 1, p.d_cfac,
-                                            alm, A.nblk, p.nalm, nmaps, p.lmax, A.part_blk_stride, p.nalm, 1,
-                                            fp64_lim, st);
+    const int64_t total = p.nalm * nmaps;
+    const int rgrid = (int)std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, 152 * 16));
+    reduce_blocks_df_kernel<<<rgrid, 256, 0, st>>>((const float4 *)partial, p.d_cfac, alm, legendre_anal_df_nblk(p), p.nalm,
+                                                   nmaps, p.lmax, (int64_t)nmaps * p.nalm, fp64_lim);
     ++*nlaunch;
-    return e;
+    return cudaGetLastError();
 }
 
 namespace {

@@ -90,12 +90,8 @@ extern "C" sht_status sht_alm2map_noalloc(sht_plan_t plan, const void *alm, doub
     cudaStream_t s = (cudaStream_t)stream;
     int n = 0;
     if (prec) {  // the plan's precision form, as sht_alm2map runs it
-        e = sht::launch_legendre_synth_df_polar(p, (const double2 *)alm, d, nmaps, s, &n);
+        e = sht::launch_legendre_synth_tc(p, (const double2 *)alm, d, scratch, NOALLOC_SCRATCH_BYTES - delta, nmaps, s, &n);
         p.launches[SHT_STAGE_LEGENDRE_SYNTH] += n;
-        if (e == cudaSuccess) {
-            e = sht::launch_legendre_synth_tc(p, (const double2 *)alm, d, scratch, nmaps, s, &n);
-            p.launches[SHT_STAGE_LEGENDRE_SYNTH] += n;
-        }
     } else {
         e = sht::launch_legendre_synth(p, (const double2 *)alm, d, nmaps, s, &n);
         p.launches[SHT_STAGE_LEGENDRE_SYNTH] += n;

@@ -103,7 +103,7 @@ struct Plan {
     int64_t *d_tc_chunk_base = nullptr; // [mmax + 1]
     int *d_tc_chunk_m = nullptr;        // [tc_total_chunks]
     int *d_tc_Ey = nullptr;             // [2][mmax + 1][slot blocks]: scale exponent of y = lambda / c, first live chunk
-    double2 *d_tc_ck_y = nullptr;       // [mmax + 1][slot blocks][128] recurrence state at the first live chunk & ~1
+    double2 *d_tc_ck_y = nullptr;       // [mmax + 1][slot blocks][128] recurrence state at the first live chunk
     int *d_tc_ck_k = nullptr;           // its rescaling exponents
     int *d_status = nullptr;            // device status word (bounded waits that gave up)
     int *d_mflag = nullptr;             // [mmax + 1] m computed by the FP64 Legendre steps (null: all)
@@ -111,8 +111,6 @@ struct Plan {
     double4 *d_spin_tab = nullptr;      // spin 2: [nalm] (alpha, alpha (1 + g), alpha (1 - g), c), built on first use
     double *d_spin_start = nullptr;     // spin 2: [mmax + 1] start coefficients S_m
     bool polar_first_slot = false;      // slot 0 runs the Reinsch form (sin(theta) < 0.03)
-    int polar_syn_blocks = 0;     // leading 128-slot blocks whose first slot is polar (sin < 0.03): the
-                                  // precision-form synthesis runs them in the Reinsch form for m <= mR
 
     // launch tuning (sht_tune): maps or slots per thread per launch
     int tune[SHT_TUNE_COUNT] = {4, 2, 4, 8, 16, 1, 1, 2};
@@ -176,29 +174,22 @@ int legendre_anal_df_nblk(const Plan &p);
 size_t legendre_anal_df_partial_bytes(const Plan &p, int nmaps);
 cudaError_t launch_legendre_anal_df(const Plan &p, const double2 *delta, double2 *alm, void *partial, int nmaps,
                                     cudaStream_t st, int *nlaunch);
+// Legendre steps on the tensor cores (legendre_tc.cu, legendre_tc_anal.cu) in caller scratch; the
+// columns that their digits cannot carry are redone by the *_fix launches (legendre.cu)
+cudaError_t build_tc_tables(Plan &p);
+int64_t tc_chunks_below(const Plan &p, int m);   // 32-l chunks of all m' < m
 size_t tc_workspace_bytes(const Plan &p, int nmaps);
-// precision-form analysis on the tensor cores (groups of up to 16 maps, reduced per group)
+size_t tc_workspace_least(const Plan &p, int nmaps);
+cudaError_t launch_legendre_synth_tc(const Plan &p, const double2 *alm, double2 *delta, void *scratch,
+                                     size_t scratch_bytes, int nmaps, cudaStream_t st, int *nlaunch);
 cudaError_t launch_legendre_anal_tc(const Plan &p, const double2 *delta, double2 *alm, void *partial, int nmaps,
                                     cudaStream_t st, int *nlaunch);
 size_t tc_anal_partial_bytes(const Plan &p, int nmaps);
-// a_lm = c_lm * sum over blocks of double-float partials for the coefficient indices
-// i0 .. i0 + nidx - 1 (nidx < 0: to nalm); partial (block, map, index i) at
-// block * blk_stride + map * map_stride + (i - i0) * idx_stride; for i < fp64_lim blocks
-// 0 .. polar_blocks - 1 are replaced by the FP64 partial polar[map * polar_stride + i]
-cudaError_t launch_reduce_blocks_df(const float4 *partial, const double2 *polar, int64_t polar_stride,
-                                    int polar_blocks, const double *cfac, double2 *alm, int nblk, int64_t nalm,
-                                    int nmaps, int lmax, int64_t blk_stride, int64_t map_stride, int64_t idx_stride,
-                                    int64_t fp64_lim, cudaStream_t st, int64_t i0 = 0, int64_t nidx = -1);
-// precision-form Reinsch analysis of the first legendre_anal_df_polar_slots() slots for m <= mR
-int legendre_anal_df_polar_slots();
-cudaError_t launch_legendre_anal_df_polar(const Plan &p, const double2 *delta, double2 *polar, int64_t polar_stride,
-                                          int nmaps, cudaStream_t st, int *nlaunch);
-cudaError_t build_tc_scales(Plan &p);
-cudaError_t launch_legendre_synth_tc(const Plan &p, const double2 *alm, double2 *delta, void *scratch, int nmaps,
-                                     cudaStream_t st, int *nlaunch);
-// precision-form synthesis of the polar slots 0 .. 127 for m <= mR (Reinsch form, double-float sums)
-cudaError_t launch_legendre_synth_df_polar(const Plan &p, const double2 *alm, double2 *delta, int nmaps,
-                                           cudaStream_t st, int *nlaunch);
+cudaError_t configure_tc_anal_kernel();
+cudaError_t launch_legendre_synth_fix(const Plan &p, const double2 *alm, double2 *delta, const int *fix, int nmaps,
+                                      cudaStream_t st);
+cudaError_t launch_legendre_anal_fix(const Plan &p, const double2 *delta, double2 *alm, double2 *partial, const int *fix,
+                                     int nmaps, int m0, int m1, int64_t idx0, int64_t nalm_part, cudaStream_t st);
 
 // spin-2 transforms (spin.cu): Legendre steps on [nmaps][2] coefficient / Delta pairs
 cudaError_t build_spin_tables(Plan &p);
@@ -248,6 +239,7 @@ cudaError_t batch_ring_launch(const BatchLaunch &L, bool synth, double2 *scratch
 cudaError_t take_check_word_legendre(int *w);
 cudaError_t take_check_word_df(int *w);
 cudaError_t take_check_word_tc(int *w);
+cudaError_t take_check_word_tc_anal(int *w);
 cudaError_t take_check_word_spin(int *w);
 cudaError_t take_check_word_ring(int *w);
 

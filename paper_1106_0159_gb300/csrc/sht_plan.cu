@@ -312,12 +312,8 @@ sht_status run_legendre_synth(Plan &p, const double2 *alm, double2 *delta, void 
     int n = 0;
     cudaError_t e;
     if (p.mode == SHT_MODE_SPLIT_BF16) {
-        e = sht::launch_legendre_synth_df_polar(p, alm, delta, nmaps, s, &n);
+        e = sht::launch_legendre_synth_tc(p, alm, delta, tc_scratch, sht::tc_workspace_bytes(p, nmaps), nmaps, s, &n);
         p.launches[0] += n;
-        if (e == cudaSuccess) {
-            e = sht::launch_legendre_synth_tc(p, alm, delta, tc_scratch, nmaps, s, &n);
-            p.launches[0] += n;
-        }
     } else {
         e = sht::launch_legendre_synth(p, alm, delta, nmaps, s, &n);
         p.launches[0] += n;
@@ -477,7 +473,7 @@ sht_status sht_plan_set_mode(sht_plan_t plan, int mode)
         // the Reinsch-form kernels of the precision form cover the first 256 slots (the analysis: one
         // CTA over slots 0 .. 255 per m; the synthesis: the leading polar 128-slot blocks)
         if (p.nslots > 256 && p.slotTheta[256] > 0.0 && std::sin(p.slotTheta[256]) < 0.03) return SHT_EUNSUPPORTED;
-        cudaError_t e = sht::build_tc_scales(p);  // one FP64 pass of the recurrence, synchronous
+        cudaError_t e = sht::build_tc_tables(p);  // one FP64 pass of the recurrence, synchronous
         if (e == cudaSuccess) e = sht::build_df_ring_tables(p);
         if (e != cudaSuccess) return cuda_fail(p, e, "precision-form tables");
     }
@@ -500,6 +496,7 @@ sht_status sht_plan_device_status(sht_plan_t plan, int *status, int clear)
     if (e == cudaSuccess) e = sht::take_check_word_legendre(&w);
     if (e == cudaSuccess) e = sht::take_check_word_df(&w);
     if (e == cudaSuccess) e = sht::take_check_word_tc(&w);
+    if (e == cudaSuccess) e = sht::take_check_word_tc_anal(&w);
     if (e == cudaSuccess) e = sht::take_check_word_spin(&w);
     if (e == cudaSuccess) e = sht::take_check_word_ring(&w);
     if (e == cudaSuccess) *status |= w;
@@ -614,9 +611,6 @@ sht_status sht_plan_create(sht_plan_t *out, sht_grid grid, int nrings, const int
     std::vector<double3> rein;
     reinsch_tables(lmax, p.mR, rein);
     p.polar_first_slot = p.mR >= 0 && s[0] < 0.03;
-    p.polar_syn_blocks = 0;
-    if (p.mR >= 0)
-        while (p.polar_syn_blocks * 128 < p.nslots && s[p.polar_syn_blocks * 128] < 0.03) ++p.polar_syn_blocks;
     p.tune[SHT_TUNE_ANAL_SLOTS] = sht::legendre_anal_default_slots(p);
     // precision form: 32-l chunks per m
     std::vector<int64_t> chunk_base(mmax + 1);
