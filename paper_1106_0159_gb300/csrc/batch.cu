@@ -4,6 +4,8 @@
 //
 // alm2map:  Legendre synthesis tiles of every job -> ring synthesis units of every job;
 // map2alm:  ring analysis units -> Legendre analysis tiles -> block reduction of every job.
+// Plans whose FP64 Legendre steps run on the tensor cores (Plan::tc64) keep those one-plan launches,
+// whose tiles hold a whole SM each, so their results are the one-plan calls' too.
 // The batch owns its Delta slabs, partial sums, scratch and queue counters; sht_batch_run only
 // enqueues stream work (three memsets and the launches), so it can be captured in a CUDA graph and
 // replayed with new inputs written in place.
@@ -25,6 +27,12 @@ struct sht_batch_s {
     size_t ws_bytes = 0;
     int *d_counters = nullptr;               // one queue counter per launch
     sht::BatchLaunch leg, red, ring;
+    // jobs whose plans run on the tensor cores: their Legendre steps are the one-plan launches, one
+    // after another in one scratch, after the queue of the others
+    std::vector<size_t> queued, tc;
+    std::vector<double2 *> delta;
+    void *tc_scratch = nullptr;
+    size_t tc_bytes = 0;
     int maxlen = 1;
     double2 *ring_scratch = nullptr;
     bool ready = false;
@@ -69,11 +77,21 @@ sht_status prepare(sht_batch_s &b)
         doff[j] = off;
         off += al256((size_t)b.nmaps[j] * b.plans[j]->nrings * (b.plans[j]->mmax + 1) * sizeof(double2));
     }
+    b.queued.clear();
+    b.tc.clear();
+    b.tc_bytes = 0;
+    for (size_t j = 0; j < nj; ++j) {
+        const sht::Plan &p = *b.plans[j];
+        (p.tc64 ? b.tc : b.queued).push_back(j);
+        if (p.tc64)
+            b.tc_bytes = std::max(b.tc_bytes, al256(b.direction == 0 ? sht::tc_workspace_bytes(p, b.nmaps[j])
+                                                                     : sht::tc_anal_partial_bytes(p, b.nmaps[j])));
+    }
     const int k = b.tune[SHT_BATCH_ANAL_SLOTS];
     std::vector<size_t> poff(nj);
-    size_t pend = off;
+    size_t pend = off + b.tc_bytes;
     if (b.direction == 1)
-        for (size_t j = 0; j < nj; ++j) {
+        for (size_t j : b.queued) {
             poff[j] = pend;
             pend += al256(sht::batch_anal_partial_bytes(*b.plans[j], b.nmaps[j], k));
         }
@@ -93,36 +111,41 @@ sht_status prepare(sht_batch_s &b)
     b.ws_bytes = need;
     b.maxlen = maxlen;
     b.ring_scratch = (double2 *)((char *)b.d_ws + scratch_off);
-    std::vector<double2 *> delta(nj), partial(nj);
-    std::vector<const double2 *> cdelta(nj);
-    for (size_t j = 0; j < nj; ++j) {
-        delta[j] = (double2 *)((char *)b.d_ws + doff[j]);
-        cdelta[j] = delta[j];
-        partial[j] = (double2 *)((char *)b.d_ws + poff[j]);
+    b.tc_scratch = (char *)b.d_ws + off;
+    b.delta.resize(nj);
+    for (size_t j = 0; j < nj; ++j) b.delta[j] = (double2 *)((char *)b.d_ws + doff[j]);
+    std::vector<double2 *> qdelta, partial;  // of the queued jobs
+    std::vector<const double2 *> cdelta;
+    std::vector<const sht::Plan *> qplans;
+    std::vector<int> qmaps;
+    for (size_t j : b.queued) {
+        qdelta.push_back(b.delta[j]);
+        cdelta.push_back(b.delta[j]);
+        partial.push_back((double2 *)((char *)b.d_ws + poff[j]));
+        qplans.push_back(b.plans[j]);
+        qmaps.push_back(b.nmaps[j]);
     }
     int ml = 0;
     if (b.direction == 0) {
-        std::vector<const double2 *> alm(nj);
+        std::vector<const double2 *> alm;
         std::vector<const void *> rin(nj);
         std::vector<void *> rout(nj);
         for (size_t j = 0; j < nj; ++j) {
-            alm[j] = (const double2 *)b.in[j];
-            rin[j] = delta[j];
+            rin[j] = b.delta[j];
             rout[j] = b.out[j];
         }
-        e = sht::batch_legendre_synth_setup(b.plans, alm, delta, b.nmaps, b.tune[SHT_BATCH_SYNTH_MAPS], b.leg);
+        for (size_t j : b.queued) alm.push_back((const double2 *)b.in[j]);
+        e = sht::batch_legendre_synth_setup(qplans, alm, qdelta, qmaps, b.tune[SHT_BATCH_SYNTH_MAPS], b.leg);
         if (e == cudaSuccess) e = sht::batch_ring_setup(b.plans, rin, rout, b.nmaps, true, b.ring, ml);
     } else {
-        std::vector<double2 *> alm(nj);
+        std::vector<double2 *> alm;
         std::vector<void *> rout(nj);
-        for (size_t j = 0; j < nj; ++j) {
-            alm[j] = (double2 *)b.out[j];
-            rout[j] = delta[j];
-        }
+        for (size_t j = 0; j < nj; ++j) rout[j] = b.delta[j];
+        for (size_t j : b.queued) alm.push_back((double2 *)b.out[j]);
         e = sht::batch_ring_setup(b.plans, b.in, rout, b.nmaps, false, b.ring, ml);
         if (e == cudaSuccess)
-            e = sht::batch_legendre_anal_setup(b.plans, cdelta, partial, alm, b.nmaps, b.tune[SHT_BATCH_ANAL_MAPS], k,
-                                               b.leg, b.red);
+            e = sht::batch_legendre_anal_setup(qplans, cdelta, partial, alm, qmaps, b.tune[SHT_BATCH_ANAL_MAPS], k, b.leg,
+                                               b.red);
     }
     if (e != cudaSuccess) {
         b.last_error = std::string("batch set-up: ") + cudaGetErrorString(e);
@@ -203,14 +226,28 @@ sht_status sht_batch_run(sht_batch_t b, void *stream)
     cudaError_t e = cudaMemsetAsync(b->d_counters, 0, 4 * sizeof(int), s);
     const int lgrid = 152 * b->tune[SHT_BATCH_LEG_CTAS];
     if (b->direction == 0) {
-        if (e == cudaSuccess) e = sht::batch_legendre_synth_launch(b->leg, b->d_counters, lgrid, s);
+        if (e == cudaSuccess && !b->queued.empty())
+            e = sht::batch_legendre_synth_launch(b->leg, b->d_counters, lgrid, s);
+        for (size_t j : b->tc) {
+            int n = 0;
+            if (e == cudaSuccess)
+                e = sht::launch_legendre_synth_tc(*b->plans[j], (const double2 *)b->in[j], b->delta[j], b->tc_scratch,
+                                                  b->tc_bytes, b->nmaps[j], s, &n);
+        }
         if (e == cudaSuccess)
             e = sht::batch_ring_launch(b->ring, true, b->ring_scratch, b->maxlen, b->d_counters + 1, ring_ctas(*b), s);
     } else {
         if (e == cudaSuccess)
             e = sht::batch_ring_launch(b->ring, false, b->ring_scratch, b->maxlen, b->d_counters + 1, ring_ctas(*b),
                                        s);
-        if (e == cudaSuccess) e = sht::batch_legendre_anal_launch(b->leg, b->red, b->d_counters, lgrid, s);
+        if (e == cudaSuccess && !b->queued.empty())
+            e = sht::batch_legendre_anal_launch(b->leg, b->red, b->d_counters, lgrid, s);
+        for (size_t j : b->tc) {
+            int n = 0;
+            if (e == cudaSuccess)
+                e = sht::launch_legendre_anal_tc(*b->plans[j], b->delta[j], (double2 *)b->out[j], b->tc_scratch,
+                                                 b->nmaps[j], s, &n);
+        }
     }
     if (e != cudaSuccess) {
         b->last_error = std::string("batch run: ") + cudaGetErrorString(e);

@@ -496,6 +496,7 @@ __global__ void __launch_bounds__(SYN_T) legendre_synth_fix_kernel(SynArgs A, co
     __shared__ Coef C;
     __shared__ double2 s_a[1][CHL];
     const int m = blockIdx.x;
+    if (A.mflag && !A.mflag[m]) return;
     const int64_t dstride = (int64_t)A.nrings * (A.mmax + 1);
     for (int g = 0; g < nmaps; ++g) {
         if (!fix[m * 16 + g]) continue;
@@ -519,6 +520,7 @@ __global__ void __launch_bounds__(ANA_T) legendre_anal_fix_kernel(AnaArgs A, con
     __shared__ Coef C;
     __shared__ double s_red[NW][CHL][2];
     const int m = m0 + blockIdx.x;
+    if (A.mflag && !A.mflag[m]) return;
     const int64_t dstride = (int64_t)A.nrings * (A.mmax + 1);
     const int64_t base = (int64_t)m * (2 * A.lmax + 3 - m) / 2;
     for (int g = 0; g < nmaps; ++g) {
@@ -766,6 +768,7 @@ cudaError_t launch_legendre_synth_fix(const Plan &p, const double2 *alm, double2
     A.alpha = p.d_alpha;
     A.cfac = p.d_cfac;
     A.rein = p.d_rein;
+    A.mflag = p.d_mflag;
     A.mR = p.mR;
     A.nslots = p.nslots;
     A.nblk = (p.nslots + SYN_T - 1) / SYN_T;
@@ -790,6 +793,7 @@ cudaError_t launch_legendre_anal_fix(const Plan &p, const double2 *delta, double
     A.alpha = p.d_alpha;
     A.cfac = p.d_cfac;
     A.rein = p.d_rein;
+    A.mflag = p.d_mflag;
     A.mR = p.mR;
     A.nslots = p.nslots;
     A.nblk = (p.nslots + ANA_T - 1) / ANA_T;

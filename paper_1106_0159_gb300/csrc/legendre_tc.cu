@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(TC_NT + 32, 1) tc_synth_kernel(TcArgs A)
     const int cfirst = A.first[m * A.nblk + blk];           // chunks before it hold only dropped values
     const int nlive = nch - cfirst;
 
-    if (nlive <= 0) {  // every value dropped: Delta_m is zero on these rings
+    if (nlive <= 0 || (A.mflag && !A.mflag[m])) {  // every value dropped, or an m this plan does not compute: zeros
         if (!rec && !issuer && par == 0 && active) {
             const int rn = A.slotN[slot], rs = A.slotS[slot];
             const int64_t mstride = A.mmax + 1;
@@ -586,6 +586,15 @@ cudaError_t build_tc_tables(Plan &p)
     return cudaSuccess;
 }
 
+// FP64-mode plans whose Legendre steps run here instead of in the plain FP64 kernels of legendre.cu.
+// The results do not depend on how maps are grouped into calls, so the rule looks at the plan only.
+// Legendre synthesis / analysis of HEALPix plans (lmax = 2 Nside), plain kernels against these, us:
+//     lmax 128: 1 map 35 / 61, 58 / 61    4 maps 62 / 173, 62 / 64      16 maps 247 / 677, 71 / 67
+//     lmax 192: 1 map 78 / 132, 74 / 92   4 maps 151 / 404, 77 / 94     16 maps 603 / 1598, 95 / 106
+//     lmax 1024: 1 map 3435 / 4598, 2623 / 3456                         16 maps 31679 / 55869, 3039 / 4165
+// so that from lmax 192 on no number of maps loses.
+bool tc_fp64_plan(const Plan &p) { return p.lmax >= 192; }
+
 // scratch of the synthesis: the a_lm digits of one m-slab, then the scale exponents and marks
 size_t tc_workspace_bytes(const Plan &p, int nmaps)
 {
@@ -633,11 +642,13 @@ cudaError_t launch_legendre_synth_tc(const Plan &p, const double2 *alm, double2 
     A.nrings = p.nrings;
     A.mR = p.mR;
     A.nalm = p.nalm;
+    A.mflag = p.d_mflag;
     A.fix = (int *)scratch;  // [mmax + 1][16], then Ea [mmax + 1][N], then the digits
     A.Ea = A.fix + (size_t)(p.mmax + 1) * 16;
     const size_t head = (exponent_bytes(p) + 255) & ~(size_t)255;
     A.bdig = (uint4 *)((char *)scratch + head);
     const size_t cap = scratch_bytes - head;
+    if (scratch_bytes < tc_workspace_least(p, nmaps)) return cudaErrorInvalidValue;
     const int64_t dstride = (int64_t)p.nrings * (p.mmax + 1);
     for (int g0 = 0; g0 < nmaps;) {
         const int nm = std::min(p.tune[SHT_TUNE_TC_MAPS], nmaps - g0);

@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(TA_NT, 1) tc_anal_kernel(TcArgs A)
     const int cfirst = A.first[m * A.nblk + blk];           // chunks before it hold only dropped values:
     const int nlive = nch - cfirst;                         // the reduction leaves them out
     const int nm = A.nmaps;
-    if (nlive <= 0) return;
+    if (nlive <= 0 || (A.mflag && !A.mflag[m])) return;
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)), "r"(512));
@@ -425,7 +425,8 @@ __global__ void __launch_bounds__(TR_T) tc_reduce_kernel(TcArgs A, double2 *__re
     const int64_t bstride = A.nalm_part * nm;
     const double2 *src = A.partial + (ix0 - A.idx0) * nm;
     double2 v[2] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
-    for (int b0 = 0; b0 < A.nblk; b0 += TR_T) {
+    const int nblk = (A.mflag && !A.mflag[m]) ? 0 : A.nblk;  // an m this plan does not compute: zeros
+    for (int b0 = 0; b0 < nblk; b0 += TR_T) {
         __syncthreads();
         if (threadIdx.x < 32) {  // the live blocks of this batch, in order
             int n = 0;
@@ -549,6 +550,7 @@ cudaError_t launch_legendre_anal_tc(const Plan &p, const double2 *delta, double2
     A.nrings = p.nrings;
     A.mR = p.mR;
     A.nalm = p.nalm;
+    A.mflag = p.d_mflag;
     A.fix = (int *)partial;
     A.partial = (double2 *)((char *)partial + fix_bytes(p));
     const int64_t dstride = (int64_t)p.nrings * (p.mmax + 1);

@@ -64,9 +64,13 @@ extern "C" sht_status sht_alm2map_noalloc(sht_plan_t plan, const void *alm, doub
     }
     const size_t delta = ((size_t)nmaps * p.nrings * (p.mmax + 1) * sizeof(double2) + 255) & ~(size_t)255;
     const size_t per_cta = (size_t)3 * p.fft_maxlen * sizeof(double2);
-    // the precision form's digit tiles of c_lm a_lm share the region after Delta with the ring
-    // buffers (the Legendre step is done with them before the ring step starts)
-    const size_t tc = prec ? sht::tc_workspace_bytes(p, nmaps) : 0;
+    // the digit tiles of c_lm a_lm share the region after Delta with the ring buffers (the Legendre
+    // step is done with them before the ring step starts).  They come in slabs of whole m, so that one
+    // m is enough; the precision form asks for room for all of them, an FP64 plan that runs on the
+    // tensor cores takes the plain FP64 kernels when not even one m fits.
+    const size_t tc = prec ? (size_t)p.tc_total_chunks * (std::min(nmaps, p.tune[SHT_TUNE_TC_MAPS]) > 8 ? 16384 : 8192) +
+                                 (size_t)(p.mmax + 1) * 32 * sizeof(int) + 256
+                           : 0;
     const size_t need = delta + std::max(per_cta, tc);
     if (need > NOALLOC_SCRATCH_BYTES) {
         p.last_error = "sht_alm2map_noalloc: " + std::to_string(nmaps) + " map(s) need " + std::to_string(need) +
@@ -89,8 +93,9 @@ extern "C" sht_status sht_alm2map_noalloc(sht_plan_t plan, const void *alm, doub
     double2 *scratch = (double2 *)((char *)base + delta);
     cudaStream_t s = (cudaStream_t)stream;
     int n = 0;
-    if (prec) {  // the plan's precision form, as sht_alm2map runs it
-        e = sht::launch_legendre_synth_tc(p, (const double2 *)alm, d, scratch, NOALLOC_SCRATCH_BYTES - delta, nmaps, s, &n);
+    const size_t left = NOALLOC_SCRATCH_BYTES - delta;
+    if ((prec || p.tc64) && left >= sht::tc_workspace_least(p, nmaps)) {  // as sht_alm2map runs it
+        e = sht::launch_legendre_synth_tc(p, (const double2 *)alm, d, scratch, left, nmaps, s, &n);
         p.launches[SHT_STAGE_LEGENDRE_SYNTH] += n;
     } else {
         e = sht::launch_legendre_synth(p, (const double2 *)alm, d, nmaps, s, &n);

@@ -110,6 +110,8 @@ struct Plan {
     int n_mlist = 0;                    // number of listed m (0: all)
     double4 *d_spin_tab = nullptr;      // spin 2: [nalm] (alpha, alpha (1 + g), alpha (1 - g), c), built on first use
     double *d_spin_start = nullptr;     // spin 2: [mmax + 1] start coefficients S_m
+    bool tc64 = false;                  // the FP64 mode's Legendre steps take the tensor-core kernels (tc_fp64_plan)
+    bool split_ready = false;           // the plan has been switched to the precision form once
     bool polar_first_slot = false;      // slot 0 runs the Reinsch form (sin(theta) < 0.03)
 
     // launch tuning (sht_tune): maps or slots per thread per launch
@@ -177,6 +179,7 @@ cudaError_t launch_legendre_anal_df(const Plan &p, const double2 *delta, double2
 // Legendre steps on the tensor cores (legendre_tc.cu, legendre_tc_anal.cu) in caller scratch; the
 // columns that their digits cannot carry are redone by the *_fix launches (legendre.cu)
 cudaError_t build_tc_tables(Plan &p);
+bool tc_fp64_plan(const Plan &p);                // the rule for Plan::tc64
 int64_t tc_chunks_below(const Plan &p, int m);   // 32-l chunks of all m' < m
 size_t tc_workspace_bytes(const Plan &p, int nmaps);
 size_t tc_workspace_least(const Plan &p, int nmaps);

@@ -294,7 +294,12 @@ sht_status check_call(sht_plan_t plan, const void *in, const void *out, int nmap
 using sht::StageEvents;
 using StageScope = StageEvents;
 
-// tc_scratch: tc_workspace_bytes(p, min(nmaps, 16)) bytes, used in the precision form only
+// the Legendre steps run on the tensor cores: always in the precision form, in the FP64 mode for the
+// plans of tc_fp64_plan
+bool uses_tc(const Plan &p) { return p.mode == SHT_MODE_SPLIT_BF16 || p.tc64; }
+bool anal_df(const Plan &p) { return p.mode == SHT_MODE_SPLIT_BF16 && !p.tune[SHT_TUNE_PREC_ANAL]; }
+
+// tc_scratch: synth_scratch_bytes(p, nmaps) bytes
 sht_status mlist_guard(Plan &p)
 {
     if (p.n_mlist > 0 && p.mode != SHT_MODE_FP64) {
@@ -311,7 +316,7 @@ sht_status run_legendre_synth(Plan &p, const double2 *alm, double2 *delta, void 
     StageScope sc(p, 0, s);
     int n = 0;
     cudaError_t e;
-    if (p.mode == SHT_MODE_SPLIT_BF16) {
+    if (uses_tc(p)) {
         e = sht::launch_legendre_synth_tc(p, alm, delta, tc_scratch, sht::tc_workspace_bytes(p, nmaps), nmaps, s, &n);
         p.launches[0] += n;
     } else {
@@ -323,16 +328,12 @@ sht_status run_legendre_synth(Plan &p, const double2 *alm, double2 *delta, void 
     return SHT_OK;
 }
 
-size_t synth_scratch_bytes(const Plan &p, int nmaps)
-{
-    return p.mode == SHT_MODE_SPLIT_BF16 ? sht::tc_workspace_bytes(p, nmaps) : 0;
-}
+size_t synth_scratch_bytes(const Plan &p, int nmaps) { return uses_tc(p) ? sht::tc_workspace_bytes(p, nmaps) : 0; }
 
 size_t anal_partial_bytes(const Plan &p, int nmaps)
 {
-    if (p.mode != SHT_MODE_SPLIT_BF16) return sht::legendre_anal_partial_bytes(p, nmaps);
-    return p.tune[SHT_TUNE_PREC_ANAL] ? sht::tc_anal_partial_bytes(p, nmaps)
-                                      : sht::legendre_anal_df_partial_bytes(p, nmaps);
+    if (!uses_tc(p)) return sht::legendre_anal_partial_bytes(p, nmaps);
+    return anal_df(p) ? sht::legendre_anal_df_partial_bytes(p, nmaps) : sht::tc_anal_partial_bytes(p, nmaps);
 }
 
 sht_status run_ring_synth(Plan &p, const double2 *delta, double *map, double2 *scratch, int nmaps, cudaStream_t s)
@@ -359,13 +360,13 @@ sht_status run_legendre_anal(Plan &p, const double2 *delta, double2 *alm, double
                              cudaStream_t s)
 {
     if (sht_status g = mlist_guard(p)) return g;
-    if (p.mode == SHT_MODE_SPLIT_BF16) {
-        // precision form (reduction included): the l-sum contraction on the tensor cores, or
+    if (uses_tc(p)) {
+        // reduction included: the ring sums on the tensor cores, or (a precision-form option)
         // double-float products and slot sums on the FP32 pipe
         StageScope sc(p, 3, s);
         int n = 0;
-        cudaError_t e = p.tune[SHT_TUNE_PREC_ANAL] ? sht::launch_legendre_anal_tc(p, delta, alm, partial, nmaps, s, &n)
-                                                   : sht::launch_legendre_anal_df(p, delta, alm, partial, nmaps, s, &n);
+        cudaError_t e = anal_df(p) ? sht::launch_legendre_anal_df(p, delta, alm, partial, nmaps, s, &n)
+                                   : sht::launch_legendre_anal_tc(p, delta, alm, partial, nmaps, s, &n);
         p.launches[3] += n;
         if (e != cudaSuccess) return cuda_fail(p, e, "legendre_anal");
         sc.done();
@@ -476,6 +477,7 @@ sht_status sht_plan_set_mode(sht_plan_t plan, int mode)
         cudaError_t e = sht::build_tc_tables(p);  // one FP64 pass of the recurrence, synchronous
         if (e == cudaSuccess) e = sht::build_df_ring_tables(p);
         if (e != cudaSuccess) return cuda_fail(p, e, "precision-form tables");
+        p.split_ready = true;
     }
     p.mode = mode;
     return SHT_OK;
@@ -546,7 +548,7 @@ sht_status sht_plan_live_steps(sht_plan_t plan, int64_t *live, int64_t *total)
 {
     if (!plan || !live || !total) return SHT_EINVAL;
     Plan &p = plan->p;
-    if (!p.d_tc_Ey) return SHT_EINVAL;  // the tables come with the first switch to the precision form
+    if (!p.split_ready) return SHT_EINVAL;  // only after the first switch to the precision form
     const int nblk = (p.nslots + 127) / 128;
     std::vector<int> first((size_t)(p.mmax + 1) * nblk);
     cudaError_t e = cudaMemcpy(first.data(), p.d_tc_Ey + first.size(), sizeof(int) * first.size(),
@@ -656,6 +658,11 @@ sht_status sht_plan_create(sht_plan_t *out, sht_grid grid, int nrings, const int
     if (e == cudaSuccess) {
         where = "ring tables";
         e = sht::build_fft_tables(p);
+    }
+    if (e == cudaSuccess && sht::tc_fp64_plan(p)) {
+        where = "tensor-core tables";
+        e = sht::build_tc_tables(p);
+        p.tc64 = e == cudaSuccess;
     }
     if (e != cudaSuccess) {
         cudaGetLastError();

@@ -202,6 +202,7 @@ struct TcArgs {
     const double *u, *s;
     const double *alpha, *cfac;
     const double3 *rein;     // Reinsch coefficients for m <= mR (polar blocks)
+    const int *mflag;        // [mmax+1] 1 for the m this plan computes (null: all)
     const int *Ey;           // [mmax+1][nblk] scale exponent of y per slot block
     const int *first;        // [mmax+1][nblk] first chunk with a kept y value (nch: none)
     const double2 *ck_y;     // [mmax+1][nblk][128] recurrence state at chunk first
