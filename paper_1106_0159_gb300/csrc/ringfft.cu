@@ -12,8 +12,8 @@
 //             Delta^S_m = w exp(-i m phi0) S_(m mod nphi).
 //
 // Each complex DFT is run by one CTA of a persistent grid in three
-// CTA-private scratch buffers: Stockham passes of radix 4, 2, 3, 5, 7, 11 or
-// 13 when nphi factors into those, otherwise Bluestein's chirp-z form with a
+// CTA-private scratch buffers: Stockham passes of radix 4, 2 and the odd primes
+// for which a direct sum is the cheaper form, otherwise Bluestein's chirp-z form with a
 // power-of-two convolution.  The minus-sign DFT is taken as
 // conj(DFT+(conj(x))).  Twiddles, chirps and Bluestein filters are plan
 // tables built on the device at plan creation.
@@ -40,9 +40,10 @@ constexpr int FFT_T = RING_T;
 // for two): 1024 at 64 registers each (lmax 4096, HEALPix 2048, 16 maps: synthesis / analysis
 // 42.4 / 38.0 ms, against 46.4 / 38.8 with 512 threads at 128 registers); the FP64 ones keep 512.
 constexpr int RING_DF_WIDE_T = 1024;
+constexpr int FOLD_T = 512;  // threads (and scratch entries) that share the folding of a short ring
+static_assert(FOLD_T <= FFT_T && FOLD_T <= RING_DF_WIDE_T, "every ring kernel has FOLD_T threads");
 
 #include "check.cuh"
-constexpr int MAXR = 13;
 
 // Division by a divisor d fixed for a loop, without the integer divide: q = umulhi(b, M) with
 // M = floor((2^32 - 1) / d) + 1 is floor(b / d) whenever b d < 2^32 (here b, d < 2^16).
@@ -97,6 +98,10 @@ struct F64 {
     }
     static __device__ __forceinline__ C half(C a) { return make_double2(0.5 * a.x, 0.5 * a.y); }
     using S = double;  // a real scalar
+    static __device__ __forceinline__ S tre(T t) { return t.x; }
+    static __device__ __forceinline__ S tim(T t) { return t.y; }
+    // acc + a w, a complex and w real
+    static __device__ __forceinline__ C sfma(C acc, C a, S w) { return make_double2(fma(a.x, w, acc.x), fma(a.y, w, acc.y)); }
     static __device__ __forceinline__ S sfrom(double w) { return w; }
     static __device__ __forceinline__ C smul(C a, S w) { return make_double2(a.x * w, a.y * w); }
     static __device__ __forceinline__ C from(double2 v) { return v; }
@@ -210,6 +215,12 @@ struct DF {
     }
     static __device__ __forceinline__ C half(C a) { return make_float4(0.5f * a.x, 0.5f * a.y, 0.5f * a.z, 0.5f * a.w); }
     using S = float2;  // a real scalar, double-float
+    static __device__ __forceinline__ S tre(T t) { return make_float2(t.x, t.y); }
+    static __device__ __forceinline__ S tim(T t) { return make_float2(t.z, t.w); }
+    static __device__ __forceinline__ C sfma(C acc, C a, S w)
+    {
+        return mk(dfn_add(R(acc), dfn_mul(R(a), w)), dfn_add(I(acc), dfn_mul(I(a), w)));
+    }
     static __device__ __forceinline__ S sfrom(double w) { return dfn_from(w); }
     static __device__ __forceinline__ C smul(C a, S w) { return mk(dfn_mul(R(a), w), dfn_mul(I(a), w)); }
     static __device__ __forceinline__ C from(double2 v) { return mk(dfn_from(v.x), dfn_from(v.y)); }
@@ -219,18 +230,119 @@ struct DF {
     static __device__ __forceinline__ double im(C v) { return dfn_to(I(v)); }
 };
 
-// One Stockham pass: sub-transforms of length Lsub become length Lsub * p.
-// Input  X[j * (n / Lsub) + q],  j < Lsub, q < n / Lsub
-// Output Y[k * (n / (Lsub p)) + q'], k < Lsub p
+// Radix-p butterflies.  Radices 2 and 4 are written out; 3 and 5 use the symmetry below in registers;
+// prime radices of 7 and more are direct sums over that symmetry, shared out over the threads by
+// output: with a_r = x_r + x_(p-r), b_r = x_r - x_(p-r), r = 1 .. h = (p - 1) / 2,
+//     X_k, X_(p-k) = C +- i S,  C = x_0 + sum_r a_r cos(2 pi r k / p),  S = sum_r b_r sin(2 pi r k / p),
+// about p real operations on each of the two parts per point.  Against the plain p^2 complex products
+// of one thread that this replaced (radix 13: 676 dependent FP64 instructions) it takes a quarter of the
+// operations and gives every output a thread, which is what a short ring is short of (HEALPix 32,
+// one map: 57 us of ring synthesis, most of it in the slowest ring's butterflies); and it is cheaper
+// than Bluestein's form for primes up to a few hundred (direct_radix), which took every prime from 17.
+
+// X_0 .. X_(p-1) of x (p = 3 or 5, the + sign), w1, w2 = exp(2 pi i / p), exp(4 pi i / p)
+template <class P, int p>
+__device__ __forceinline__ void odd_dft(typename P::C *x, typename P::T w1, typename P::T w2)
+{
+    using C = typename P::C;
+    const C a1 = P::add(x[1], x[p - 1]), b1 = P::sub(x[1], x[p - 1]);
+    if (p == 3) {
+        const C c = P::sfma(x[0], a1, P::tre(w1)), s = P::itimes(P::smul(b1, P::tim(w1)));
+        x[0] = P::add(x[0], a1);
+        x[1] = P::add(c, s);
+        x[2] = P::sub(c, s);
+    } else {
+        const C a2 = P::add(x[2], x[3]), b2 = P::sub(x[2], x[3]);
+        const C c1 = P::sfma(P::sfma(x[0], a1, P::tre(w1)), a2, P::tre(w2));
+        const C c2 = P::sfma(P::sfma(x[0], a1, P::tre(w2)), a2, P::tre(w1));
+        const C s1 = P::itimes(P::sfma(P::smul(b1, P::tim(w1)), b2, P::tim(w2)));
+        const C s2 = P::itimes(P::sub(P::smul(b1, P::tim(w2)), P::smul(b2, P::tim(w1))));
+        x[0] = P::add(x[0], P::add(a1, a2));
+        x[1] = P::add(c1, s1);
+        x[p - 1] = P::sub(c1, s1);
+        x[2] = P::add(c2, s2);
+        x[3] = P::sub(c2, s2);
+    }
+}
+
+// C and S of output k from the folded inputs at base + r m (a_r at r, b_r at p - r); wp = exp(2 pi i e / p)
 template <class P>
-__device__ void stockham_pass(const typename P::C *__restrict__ X, typename P::C *__restrict__ Y, int n, int Lsub,
-                              int p, const typename P::T *__restrict__ tw)
+__device__ __forceinline__ void direct_sums(const typename P::C *base, int m, int p, int k,
+                                            const typename P::T *__restrict__ wp, typename P::C &c, typename P::C &s)
+{
+    using C = typename P::C;
+    const int h = (p - 1) >> 1;
+    c = base[0];
+    s = P::zero();
+    int e = 0;
+#pragma unroll 2
+    for (int r = 1; r <= h; ++r) {
+        e += k;
+        if (e >= p) e -= p;
+        const typename P::T w = wp[e];
+        const C a = base[r * m], b = base[(p - r) * m];
+        c = P::sfma(c, a, P::tre(w));
+        s = P::sfma(s, b, P::tim(w));
+    }
+    s = P::itimes(s);
+}
+
+// a Stockham pass of a direct radix (kept out of line: its registers are not the other radices'):
+// twiddle and fold the inputs in place, then one thread per output pair
+template <class P>
+__device__ __noinline__ void stockham_direct_pass(typename P::C *__restrict__ X, typename P::C *__restrict__ Y, int n,
+                                                  int Lsub, int p, const typename P::T *__restrict__ tw,
+                                                  const typename P::T *__restrict__ wp)
 {
     using C = typename P::C;
     const int nq = n / (Lsub * p);
     const int nbf = Lsub * nq;
     const int inStride = n / Lsub;
     const Div by_nq(nq, nbf);
+    const int h = (p - 1) >> 1;
+    const Div by_h(h, (int64_t)nbf * h);
+    for (int i = threadIdx.x; i < nbf * h; i += blockDim.x) {
+        const int b = by_h.q(i), r = 1 + i - b * h;
+        const int k1 = by_nq.q(b);
+        C *src = X + (int64_t)k1 * inStride + (b - k1 * nq);
+        C u = src[(int64_t)r * nq], v = src[(int64_t)(p - r) * nq];
+        if (k1) {
+            u = P::mul(u, tw[(int64_t)r * k1 * nq]);
+            v = P::mul(v, tw[(int64_t)(p - r) * k1 * nq]);
+        }
+        src[(int64_t)r * nq] = P::add(u, v);
+        src[(int64_t)(p - r) * nq] = P::sub(u, v);
+    }
+    __syncthreads();
+    const Div by_h1(h + 1, (int64_t)nbf * (h + 1));
+    const int64_t ostride = (int64_t)Lsub * nq;
+    for (int i = threadIdx.x; i < nbf * (h + 1); i += blockDim.x) {
+        const int b = by_h1.q(i), k = i - b * (h + 1);
+        const int k1 = by_nq.q(b), q = b - k1 * nq;
+        C c, s;
+        direct_sums<P>(X + (int64_t)k1 * inStride + q, nq, p, k, wp, c, s);
+        C *dst = Y + (int64_t)k1 * nq + q;
+        dst[(int64_t)k * ostride] = P::add(c, s);
+        if (k) dst[(int64_t)(p - k) * ostride] = P::sub(c, s);
+    }
+}
+
+// One Stockham pass: sub-transforms of length Lsub become length Lsub * p.
+// Input  X[j * (n / Lsub) + q],  j < Lsub, q < n / Lsub
+// Output Y[k * (n / (Lsub p)) + q'], k < Lsub p
+template <class P>
+__device__ void stockham_pass(typename P::C *__restrict__ X, typename P::C *__restrict__ Y, int n, int Lsub,
+                              int p, const typename P::T *__restrict__ tw, const typename P::T *__restrict__ wp)
+{
+    using C = typename P::C;
+    const int nq = n / (Lsub * p);
+    const int nbf = Lsub * nq;
+    const int inStride = n / Lsub;
+    const Div by_nq(nq, nbf);
+    if (p >= 7) {
+        stockham_direct_pass<P>(X, Y, n, Lsub, p, tw, wp);
+        return;
+    }
     for (int b = threadIdx.x; b < nbf; b += blockDim.x) {
         const int k1 = by_nq.q(b);
         const int q = b - k1 * nq;
@@ -257,24 +369,25 @@ __device__ void stockham_pass(const typename P::C *__restrict__ X, typename P::C
             if (k1) a1 = P::mul(a1, tw[k1 * nq]);
             dst[0] = P::add(a0, a1);
             dst[ostride] = P::sub(a0, a1);
+        } else if (p == 3) {
+            C a[3] = {src[0], src[nq], src[2 * nq]};
+            if (k1) {
+                a[1] = P::mul(a[1], tw[k1 * nq]);
+                a[2] = P::mul(a[2], tw[2 * k1 * nq]);
+            }
+            odd_dft<P, 3>(a, tw[n / 3], tw[n / 3]);
+            dst[0] = a[0];
+            dst[ostride] = a[1];
+            dst[2 * ostride] = a[2];
         } else {
-            C a[MAXR];
-            a[0] = src[0];
-            for (int r = 1; r < p; ++r) {
-                a[r] = src[(int64_t)r * nq];
-                if (k1) a[r] = P::mul(a[r], tw[(int64_t)r * k1 * nq]);
+            C a[5] = {src[0], src[nq], src[2 * nq], src[3 * nq], src[4 * nq]};
+            if (k1) {
+#pragma unroll
+                for (int r = 1; r < 5; ++r) a[r] = P::mul(a[r], tw[(int64_t)r * k1 * nq]);
             }
-            const int wstep = n / p;  // exp(2 pi i / p) = tw[n / p]
-            for (int k2 = 0; k2 < p; ++k2) {
-                C acc = a[0];
-                int e = 0;
-                for (int r = 1; r < p; ++r) {
-                    e += k2;
-                    if (e >= p) e -= p;
-                    acc = P::add(acc, P::mul(a[r], tw[(int64_t)e * wstep]));
-                }
-                dst[(int64_t)k2 * ostride] = acc;
-            }
+            odd_dft<P, 5>(a, tw[n / 5], tw[2 * (n / 5)]);
+#pragma unroll
+            for (int r = 0; r < 5; ++r) dst[(int64_t)r * ostride] = a[r];
         }
     }
 }
@@ -291,7 +404,7 @@ __device__ typename P::C *cta_dft(const FftLen &F, const typename P::T *__restri
         int Lsub = 1;
         for (int f = 0; f < F.nfac; ++f) {
             __syncthreads();
-            stockham_pass<P>(X, Y, F.n, Lsub, F.fac[f], tab + F.tw);
+            stockham_pass<P>(X, Y, F.n, Lsub, F.fac[f], tab + F.tw, tab + F.fac_tw[f]);
             C *t = X;
             X = Y;
             Y = t;
@@ -308,7 +421,7 @@ __device__ typename P::C *cta_dft(const FftLen &F, const typename P::T *__restri
     int Lsub = 1;
     for (int f = 0; f < F.nfac; ++f) {
         __syncthreads();
-        stockham_pass<P>(X, Y, M, Lsub, F.fac[f], tab + F.tw);
+        stockham_pass<P>(X, Y, M, Lsub, F.fac[f], tab + F.tw, tab);
         C *t = X;
         X = Y;
         Y = t;
@@ -319,7 +432,7 @@ __device__ typename P::C *cta_dft(const FftLen &F, const typename P::T *__restri
     Lsub = 1;
     for (int f = 0; f < F.nfac; ++f) {
         __syncthreads();
-        stockham_pass<P>(X, Y, M, Lsub, F.fac[f], tab + F.tw);
+        stockham_pass<P>(X, Y, M, Lsub, F.fac[f], tab + F.tw, tab);
         C *t = X;
         X = Y;
         Y = t;
@@ -341,8 +454,6 @@ __device__ typename P::C *cta_dft(const FftLen &F, const typename P::T *__restri
 // t_0 m_0 + t_1 m_1 + ...), read back through a position table.  The transpose (decimation in
 // time: the twiddles before the butterflies, stages in reverse order) takes digit-reversed input
 // to natural order; Bluestein's convolution uses the pair, so it needs no reordering at all.
-constexpr int DIF_MAXR = 13;
-
 // exp(2 pi i e / n), e < n, from the plan's table in global memory
 template <class P>
 struct GlobalTw {
@@ -394,19 +505,71 @@ __device__ void dif_stage(typename P::C *x, int nt, int n, int N, int p, const T
             if (j) y1 = P::mul(y1, tw((int64_t)j * tstep));
             base[0] = P::add(a0, a1);
             base[m] = y1;
+        } else if (p == 3) {
+            C a[3] = {base[0], base[m], base[2 * m]};
+            odd_dft<P, 3>(a, tw(n / 3), tw(n / 3));
+            base[0] = a[0];
+            base[m] = j ? P::mul(a[1], tw((int64_t)j * tstep)) : a[1];
+            base[2 * m] = j ? P::mul(a[2], tw((int64_t)2 * j * tstep)) : a[2];
         } else {
-            C a[DIF_MAXR];
-            for (int r = 0; r < p; ++r) a[r] = base[r * m];  // all p inputs held before any output
-            const int wstep = n / p;  // exp(2 pi i / p) = tw(n / p)
-            for (int t = 0; t < p; ++t) {
-                C acc = a[0];
-                int e = 0;
-                for (int r = 1; r < p; ++r) {
-                    e += t;
-                    if (e >= p) e -= p;
-                    acc = P::add(acc, P::mul(a[r], tw((int64_t)e * wstep)));
+            C a[5] = {base[0], base[m], base[2 * m], base[3 * m], base[4 * m]};
+            odd_dft<P, 5>(a, tw(n / 5), tw(2 * (n / 5)));
+            base[0] = a[0];
+#pragma unroll
+            for (int t = 1; t < 5; ++t) base[t * m] = j ? P::mul(a[t], tw((int64_t)j * t * tstep)) : a[t];
+        }
+    }
+}
+
+// dif_stage for a direct radix p >= 7 (one DFT of length n): batches of butterflies whose output pairs
+// are at most DIRECT_K per thread: fold the inputs in place, form the pairs in registers, write them
+// back over the inputs.  Ends after a barrier of the last batch's reads; the writes need one more.
+constexpr int DIRECT_K = 2;
+template <class P, class TW>
+__device__ __noinline__ void dif_direct_stage(typename P::C *x, int n, int N, int p, const TW &tw, const typename P::T *__restrict__ wp)
+{
+    using C = typename P::C;
+    const int m = N / p, tstep = n / N, nbf = n / p, h = (p - 1) >> 1;
+    const int most = max(1, (DIRECT_K * (int)blockDim.x) / (h + 1));  // butterflies per batch
+    const int nb0 = min(most, nbf);
+    const Div by_m(m, nbf), by_h(h, (int64_t)nb0 * h), by_h1(h + 1, (int64_t)nb0 * (h + 1));
+    for (int b0 = 0; b0 < nbf; b0 += most) {
+        const int nb = min(most, nbf - b0);
+        for (int i = threadIdx.x; i < nb * h; i += blockDim.x) {
+            const int bb = by_h.q(i), r = 1 + i - bb * h, b = b0 + bb;
+            const int blk = by_m.q(b), j = b - blk * m;
+            C *base = x + blk * N + j;
+            const C u = base[r * m], v = base[(p - r) * m];
+            base[r * m] = P::add(u, v);
+            base[(p - r) * m] = P::sub(u, v);
+        }
+        __syncthreads();
+        C c[DIRECT_K], s[DIRECT_K];
+#pragma unroll
+        for (int q = 0; q < DIRECT_K; ++q) {
+            const int i = threadIdx.x + q * blockDim.x;
+            if (i < nb * (h + 1)) {
+                const int bb = by_h1.q(i), k = i - bb * (h + 1), b = b0 + bb;
+                const int blk = by_m.q(b), j = b - blk * m;
+                direct_sums<P>(x + blk * N + j, m, p, k, wp, c[q], s[q]);
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < DIRECT_K; ++q) {
+            const int i = threadIdx.x + q * blockDim.x;
+            if (i < nb * (h + 1)) {
+                const int bb = by_h1.q(i), k = i - bb * (h + 1), b = b0 + bb;
+                const int blk = by_m.q(b), j = b - blk * m;
+                C *base = x + blk * N + j;
+                const C u = P::add(c[q], s[q]);
+                if (k == 0) {
+                    base[0] = u;
+                } else {
+                    const C v = P::sub(c[q], s[q]);
+                    base[k * m] = j ? P::mul(u, tw((int64_t)j * k * tstep)) : u;
+                    base[(p - k) * m] = j ? P::mul(v, tw((int64_t)j * (p - k) * tstep)) : v;
                 }
-                base[t * m] = (j && t) ? P::mul(acc, tw((int64_t)j * t * tstep)) : acc;
             }
         }
     }
@@ -495,7 +658,10 @@ __device__ void smem_stages(const FftLen &F, const typename P::T *__restrict__ t
     }
     for (int k = k0; k < F.nst; ++k) {
         __syncthreads();
-        dif_stage<P>(D, 1, n, N, F.rad[k], twn);
+        if (F.rad[k] >= 7)
+            dif_direct_stage<P>(D, n, N, F.rad[k], twn, tab + F.rad_tw[k]);
+        else
+            dif_stage<P>(D, 1, n, N, F.rad[k], twn);
         N /= F.rad[k];
     }
     __syncthreads();
@@ -553,15 +719,17 @@ struct RingArgs {
     double2 *delta_out;           // analysis output
 };
 
-// folded, phased spectrum bin k of one ring
+// terms of spectrum bin k of one ring, folded and phased: m = k + n (i0 + i di) and, conjugated,
+// m = n - k + n (i0 + i di) up to mmax (k < n; -m = k mod n with m >= 1)
 template <class P>
 __device__ __forceinline__ typename P::C fold_bin(const double2 *__restrict__ d, const typename P::T *__restrict__ ph,
-                                                  int k, int n, int mmax)
+                                                  int k, int n, int mmax, int i0, int di)
 {
     typename P::C c = P::zero();
-    for (int m = k; m <= mmax; m += n) c = P::add(c, P::mul(P::from(d[m]), ph[m]));
-    // the conjugate terms: -m = k mod n with m >= 1 (k < n)
-    for (int m = n - k; m <= mmax; m += n) c = P::add(c, P::conj(P::mul(P::from(d[m]), ph[m])));
+    const int64_t step = (int64_t)n * di;
+    for (int64_t m = k + (int64_t)n * i0; m <= mmax; m += step) c = P::add(c, P::mul(P::from(d[m]), ph[m]));
+    for (int64_t m = n - k + (int64_t)n * i0; m <= mmax; m += step)
+        c = P::add(c, P::conj(P::mul(P::from(d[m]), ph[m])));
     return c;
 }
 
@@ -585,14 +753,30 @@ __device__ void ring_synth_unit(const RingArgs<P> &A, int item, int g, typename 
     extern __shared__ __align__(16) unsigned char ring_smem[];
     const bool sm = smem_path(F, A.use_sm);
     C *D = sm ? (C *)ring_smem : B0;
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        const C ca = fold_bin<P>(dA, pA, k, n, A.mmax);
-        C z = ca;
-        if (dB) {
-            const C cb = fold_bin<P>(dB, pB, k, n, A.mmax);
-            z = P::add(ca, P::itimes(cb));  // C_A + i C_B
+    // A bin of a ring of n pixels folds about 2 mmax / n terms of each ring, one after another: on the
+    // shortest rings (4 pixels: 1024 terms at mmax 2048) that chain was the longest of the whole stage.
+    // So up to FOLD_T threads share the bins of a short ring, and the parts of a bin are added in order
+    // (the same number whatever the launch: the plan's scratch and shared memory hold FOLD_T entries).
+    const int parts = max(1, min(FOLD_T / n, 2 * A.mmax / n + 1));
+    if (parts > 1) {
+        const int part = threadIdx.x / n, k = threadIdx.x - part * n;
+        if (part < parts) {
+            C z = fold_bin<P>(dA, pA, k, n, A.mmax, part, parts);
+            if (dB) z = P::add(z, P::itimes(fold_bin<P>(dB, pB, k, n, A.mmax, part, parts)));
+            D[threadIdx.x] = z;
         }
-        D[k] = z;
+        __syncthreads();
+        C z = P::zero();
+        if (threadIdx.x < n)
+            for (int q = 0; q < parts; ++q) z = P::add(z, D[q * n + threadIdx.x]);
+        __syncthreads();
+        if (threadIdx.x < n) D[threadIdx.x] = z;
+    } else {
+        for (int k = threadIdx.x; k < n; k += blockDim.x) {
+            C z = fold_bin<P>(dA, pA, k, n, A.mmax, 0, 1);
+            if (dB) z = P::add(z, P::itimes(fold_bin<P>(dB, pB, k, n, A.mmax, 0, 1)));  // C_A + i C_B
+            D[k] = z;
+        }
     }
     double *outA = A.map_out + (int64_t)g * A.npix + A.ofs[it.ringA];
     double *outB = it.ringB >= 0 ? A.map_out + (int64_t)g * A.npix + A.ofs[it.ringB] : nullptr;
@@ -788,7 +972,7 @@ __global__ void __launch_bounds__(FFT_T) bluestein_filter_kernel(const FftLen *l
         int Lsub = 1;
         for (int f = 0; f < F.nfac; ++f) {
             __syncthreads();
-            stockham_pass<F64>(X, Y, M, Lsub, F.fac[f], tab + F.tw);
+            stockham_pass<F64>(X, Y, M, Lsub, F.fac[f], tab + F.tw, tab);
             double2 *tmp = X;
             X = Y;
             Y = tmp;
@@ -838,10 +1022,27 @@ __global__ void phase_table_kernel(const double *phi0, int nrings, int mmax, dou
     }
 }
 
-bool factor_smooth(int n, std::vector<int> &fac)
+// Whether a prime p runs as a direct radix: about p + 7 real operations per point and part against
+// Bluestein's two power-of-two transforms of length M >= 2 p - 1 (3.5 per point and factor of two) with
+// its chirps and filter.  Holds for every p <= 127 and, where 2 p - 1 lies just above a power of two
+// (so that M is nearly 4 p), up to about 280.
+bool direct_radix(int p)
+{
+    if (p > 1021) return false;
+    int M = 1, lg = 0;
+    while (M < 2 * p - 1) {
+        M <<= 1;
+        ++lg;
+    }
+    return p + 7.0 <= (2.0 * 3.5 * lg * M + 4.0 * M) / p + 8.0;
+}
+
+// n as radices 4, 2 and primes (ascending); true when every prime runs as a radix, otherwise the
+// remaining factor is left in *rest
+bool factor_smooth(int n, std::vector<int> &fac, int *rest = nullptr)
 {
     fac.clear();
-    int r = n;
+    int r = n, left = 1;
     while (r % 4 == 0) {
         fac.push_back(4);
         r /= 4;
@@ -850,13 +1051,18 @@ bool factor_smooth(int n, std::vector<int> &fac)
         fac.push_back(2);
         r /= 2;
     }
-    for (int p : {3, 5, 7, 11, 13}) {
+    for (int p = 3; r > 1; p += 2) {
+        if ((int64_t)p * p > r) p = r;  // r is prime
         while (r % p == 0) {
-            fac.push_back(p);
+            if (direct_radix(p))
+                fac.push_back(p);
+            else
+                left *= p;
             r /= p;
         }
     }
-    return r == 1;
+    if (rest) *rest = left;
+    return left == 1;
 }
 
 // opt-in dynamic shared memory of one CTA on this part, less room for the kernels' static words
@@ -899,23 +1105,16 @@ int ring_occupancy(int smem)
 
 constexpr int RING_SMEM_HALF = 112 * 1024;  // two CTAs per SM, with room for static words
 
-// Shared-memory form of a length-n DFT within `cap` complex entries: n = sm_part pb, sm_part smooth
-// (its radices in sfac) and pb the product of the prime factors above 13; pb > 1 takes Bluestein
+// Shared-memory form of a length-n DFT within `cap` complex entries: n = sm_part pb, sm_part the
+// product of the radices in sfac and pb that of the other prime factors; pb > 1 takes Bluestein
 // DFTs of length pb on power-of-two buffers of Mb >= 2 pb - 1 entries, bat >= 1 at a time.  When
 // 4 | n and room is left, the twq = n / 4 twiddles of the first quarter wave follow.  Returns
 // whether it fits (entries = n + bat Mb + twq <= cap, at most 16 stages).
 bool ring_sm_shape(int n, int64_t cap, int &pb, int &sm_part, int &Mb, int &bat, int &twq, int64_t &entries,
                    std::vector<int> &sfac)
 {
-    sm_part = 1;
-    int r = n;
-    for (int q : {2, 3, 5, 7, 11, 13})
-        while (r % q == 0) {
-            r /= q;
-            sm_part *= q;
-        }
-    pb = r;
-    factor_smooth(sm_part, sfac);
+    factor_smooth(n, sfac, &pb);
+    sm_part = n / pb;
     Mb = 1;
     bat = 0;
     twq = 0;
@@ -1140,9 +1339,19 @@ cudaError_t build_fft_tables(Plan &p)
         int Mb, nbr, brad[16];
     };
     std::map<int, Aux> aux_of;       // Bluestein tables of the split stage, by its length
+    std::map<int, int64_t> prime_tw;  // exp(2 pi i k / p) of the direct radices
     std::vector<FftLen> pending_aux;  // their extra length entries, stored after the length in hand
     int64_t off = 0;
     int maxlen = 1, filt_maxlen = 1, smem_bytes = 0;
+    auto direct_tw = [&](int q) {
+        if (q < 7) return (int64_t)0;
+        auto f = prime_tw.find(q);
+        if (f != prime_tw.end()) return f->second;
+        prime_tw[q] = off;
+        jobs.push_back({off, q, 0});
+        off += q;
+        return off - q;
+    };
     p.lens.clear();
     // Shared memory of one launch: every CTA gets the largest need of the plan's lengths (one
     // Bluestein buffer per split length); the split lengths batch more Bluestein DFTs only within
@@ -1188,7 +1397,10 @@ cudaError_t build_fft_tables(Plan &p)
         }
         if ((int)fac.size() > 24) return cudaErrorInvalidValue;
         L.nfac = (int)fac.size();
-        for (size_t i = 0; i < fac.size(); ++i) L.fac[i] = fac[i];
+        for (size_t i = 0; i < fac.size(); ++i) {
+            L.fac[i] = fac[i];
+            L.fac_tw[i] = L.M ? 0 : direct_tw(fac[i]);
+        }
 
         // shared-memory path (ring_sm_shape), Bluestein DFTs of the split stage up to the budget
         int pb = 1, Mb = 1, bat = 0, sm_part = 1, twq = 0;
@@ -1243,7 +1455,10 @@ cudaError_t build_fft_tables(Plan &p)
                 L.bat = bat;
                 L.rad[L.nst++] = pb;
             }
-            for (int q : sfac) L.rad[L.nst++] = q;
+            for (int q : sfac) {
+                L.rad_tw[L.nst] = direct_tw(q);
+                L.rad[L.nst++] = q;
+            }
             L.sm = 1;
             L.twq = twq;
             L.smem_entries = (int)entries;
@@ -1267,9 +1482,10 @@ cudaError_t build_fft_tables(Plan &p)
     }
     p.nitems = (int)items.size();
     p.nlens = (int)p.lens.size();
+    maxlen = std::max(maxlen, (FOLD_T + 2) / 3);  // three buffers hold FOLD_T entries
     p.fft_maxlen = maxlen;
     p.fft_tab_len = off;
-    p.ring_smem = smem_bytes;
+    p.ring_smem = smem_bytes ? std::max(smem_bytes, FOLD_T * 16) : 0;
     maxlen = std::max(maxlen, filt_maxlen);  // scratch of the filter kernel
 
     cudaError_t e;

@@ -32,22 +32,25 @@ struct FftItem {
 };
 
 // Everything a CTA needs to run a length-n DFT with the + sign,
-// y_k = sum_j x_j exp(+2 pi i j k / n).  Smooth n runs as Stockham passes
-// with the radices fac[]; otherwise Bluestein with a power-of-two M.
+// y_k = sum_j x_j exp(+2 pi i j k / n).  An n without prime factors that Bluestein's form is
+// cheaper for runs as Stockham passes with the radices fac[] (prime radices of 7 and more: direct
+// sums); otherwise Bluestein with a power-of-two M.
 struct FftLen {
     int n;
     int M;            // Bluestein convolution length, 0 when n is smooth
     int nfac;         // radices of n (smooth) or of M (Bluestein)
     int fac[24];
+    int64_t fac_tw[24];  // offset of exp(2 pi i k / p), k < p, of each radix p >= 7
     int64_t tw;       // offset of exp(2 pi i k / n), k < n   (smooth) or of exp(2 pi i k / M), k < M (Bluestein)
     int64_t chirp;    // offset of exp(i pi j^2 / n), j < n   (Bluestein)
     int64_t filt;     // offset of FFT_M(h) / M, M entries      (Bluestein)
     // Shared-memory path (sm != 0; ringfft.cu): in-place DIF stages with radices rad[0 .. nst-1] over
     // the data in shared memory leave the spectrum in digit-reversed order, bin k at position
-    // perm[k].  split != 0: stage 0 (radix p = rad[0], not smooth) runs as Bluestein DFTs of length p
+    // perm[k].  split != 0: stage 0 (radix p = rad[0]) runs as Bluestein DFTs of length p
     // in a second shared buffer, bat at a time: forward DIF of length Mb (radices brad), the filter
     // multiplied in the DIF output order, DIT back to natural order.
     int sm, nst, rad[16];
+    int64_t rad_tw[16];  // offset of exp(2 pi i k / p), k < p, of each direct radix p >= 7
     int split, Mb, nbr, brad[16], bat;
     int64_t tw_n;     // exp(2 pi i k / n), k < n
     int64_t perm;     // offset into the int table: perm[k], k < n
