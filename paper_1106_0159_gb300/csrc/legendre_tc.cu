@@ -33,6 +33,13 @@
 // so one MMA A_a x stack adds class a + b to accumulator block a + b and class a + b + 1 to block
 // a + b + 1 (20 MMAs per parity and chunk instead of 36).
 //
+// Spin 2 (polarisation).  With P+- = sum (E +- iB) lambda+- (spin.cu), Delta^Q = -(P+ + P-) / 2 and
+// Delta^U = i (P+ - P-) / 2, and a mirror ring swaps lambda+ and lambda- up to (-1)^(l+m).  So a map's
+// pair is two complex columns E + iB, E - iB, and two passes, one per sign of the recurrence, give
+// P+- everywhere: the column of the pass's own sign on the northern rings (E + O), the other on the
+// southern ones (E - O).  spin_combine_kernel then forms Q and U.  4 FP64 instructions per step and
+// ring pair for up to 8 maps, where the FP64 kernels take 6 + 8 per map.
+//
 // What bounds it: the FP64 recurrence, 64 FP64 instructions per warp and chunk = 4096 SM cycles.
 #include "sht_internal.h"
 
@@ -72,10 +79,29 @@ static_assert(TcTile<8>::B_CHUNK == 8 * 512 && TcTile<32>::B_CHUNK == 32 * 512, 
 
 // ---------------------------------------------------------------- a_lm side
 
+// coefficient (l, m) at index ix of column pair g: a_lm of map g, or (spin) E + iB (g even) / E - iB (g
+// odd) of polarised map g / 2; imaginary parts at m = 0 are ignored
+template <bool SPIN>
+__device__ __forceinline__ double2 column_value(const TcArgs &A, int g, int m, int64_t ix)
+{
+    if (!SPIN) {
+        const double2 a = A.alm[(int64_t)g * A.nalm + ix];
+        return make_double2(a.x, m == 0 ? 0.0 : a.y);
+    }
+    double2 e = A.alm[(int64_t)(g & ~1) * A.nalm + ix], b = A.alm[(int64_t)(g | 1) * A.nalm + ix];
+    if (m == 0) e.y = b.y = 0.0;
+    return (g & 1) ? make_double2(e.x + b.y, e.y - b.x) : make_double2(e.x - b.y, e.y + b.x);
+}
+template <bool SPIN>
+__device__ __forceinline__ double c_factor(const TcArgs &A, int64_t ix)
+{
+    return SPIN ? A.tab[ix].w : A.cfac[ix];
+}
+
 // E_a[m][n] with |c_lm a_lm| < 2^E_a for all l (from exponent fields, no FP64 work), and the columns
 // the digits cannot carry: a value that is not finite or subnormal, or a maximum near the ends of the
 // FP64 range.
-template <int N>
+template <int N, bool SPIN>
 __global__ void tc_scale_kernel(TcArgs A)
 {
     __shared__ int s_max[N];
@@ -90,14 +116,13 @@ __global__ void tc_scale_kernel(TcArgs A)
     unsigned odd = 0;  // maps with a non-finite value or a nonzero subnormal
 #pragma unroll
     for (int n = 0; n < N; ++n) mx[n] = 0;
-    for (int l = m + threadIdx.x; l <= L; l += blockDim.x) {
+    for (int l = first_l<SPIN ? REC_SPIN : REC_Y>(m) + threadIdx.x; l <= L; l += blockDim.x) {
         const int64_t ix = base + (l - m);
-        const int ec = dexp(A.cfac[ix]);
+        const int ec = dexp(c_factor<SPIN>(A, ix));
 #pragma unroll
         for (int g = 0; g < N / 2; ++g) {
             if (g < A.nmaps) {
-                double2 a = A.alm[(int64_t)g * A.nalm + ix];
-                if (m == 0) a.y = 0.0;  // Im a_l0 is ignored
+                const double2 a = column_value<SPIN>(A, g, m, ix);
                 const int er = dexp(a.x), ei = dexp(a.y);
                 if (er == 0x7ff || ei == 0x7ff || (!er && a.x != 0.0) || (!ei && a.y != 0.0)) odd |= 1u << g;
                 if (er) mx[2 * g] = max(mx[2 * g], er + ec);
@@ -129,7 +154,7 @@ __global__ void tc_scale_kernel(TcArgs A)
 // (n2/8, k/8) at ((k/8) (N2/8) + n2/8) * 64 elements.  Thread (parity, k/8, n)
 // cuts the 8 values k/8 .. k/8 + 7 of its column: each digit's 8 values are one core-matrix row,
 // 16 contiguous bytes, stored as one vector.
-template <int N>
+template <int N, bool SPIN>
 __global__ void tc_split_b_kernel(TcArgs A)
 {
     const int64_t chunk = A.chunk0 + blockIdx.x;
@@ -149,12 +174,12 @@ __global__ void tc_split_b_kernel(TcArgs A)
         uint2 f[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const int l = m + TC_CH * c + 2 * (8 * kh + kk + h) + eo;
+            const int l = first_l<SPIN ? REC_SPIN : REC_Y>(m) + TC_CH * c + 2 * (8 * kh + kk + h) + eo;
             double v = 0.0;
             if (l <= L && g < A.nmaps) {
                 const int64_t ix = base + (l - m);
-                const double2 a = A.alm[(int64_t)g * A.nalm + ix];
-                v = A.cfac[ix] * ((n & 1) ? (m == 0 ? 0.0 : a.y) : a.x);
+                const double2 a = column_value<SPIN>(A, g, m, ix);
+                v = c_factor<SPIN>(A, ix) * ((n & 1) ? a.y : a.x);
             }
             f[h] = digit_fields(v, E);
         }
@@ -176,7 +201,7 @@ __global__ void tc_split_b_kernel(TcArgs A)
 // start of that chunk, where the tensor-core kernels begin (at lmax 4096 on HEALPix about a quarter
 // of the steps lie before it).  Same recurrence, operation for operation, as recurrence_warps, so
 // that both see the same rescaling steps and the same values.
-template <bool REIN>
+template <int KIND>
 __device__ __forceinline__ void tables_body(const TcArgs &A, int m, int blk, int *s_max, int *s_first, RecCoef *s_c,
                                             double2 *ck_y, int *ck_k)
 {
@@ -185,22 +210,29 @@ __device__ __forceinline__ void tables_body(const TcArgs &A, int m, int blk, int
     const bool active = slot < A.nslots;
     const int L = A.lmax;
     const int64_t base = (int64_t)m * (2 * L + 3 - m) / 2;
-    const int nch = (L - m + TC_CH) / TC_CH;
+    const int lb = first_l<KIND>(m);
+    const int nch = (L - lb + TC_CH) / TC_CH;
     const int64_t ci = (int64_t)(m * A.nblk + blk) * TC_T + tid;
     double u = 0.0, y1 = 0.0, y2 = 0.0;
     int k = 0;
     if (active) {
         u = A.u[slot];
         double y0;
-        sectoral_start(A.s[slot], A.alpha[base], m, y0, k);
-        y2 = REIN ? y0 : -y0;
+        if (KIND == REC_SPIN) {  // S_m sin^|m-2| times sin^p(theta/2) (+) or sigma cos^p(theta/2) (-): spin.cu
+            sectoral_start(A.s[slot], A.start[m], m >= 2 ? m - 2 : 2 - m, y0, k);
+            const double f = A.sig > 0 ? 0.5 * u : 1.0 - 0.5 * u;
+            y0 *= m >= 2 ? f * f : m == 1 ? (A.sig > 0 ? f : -f) : 1.0;
+        } else {
+            sectoral_start(A.s[slot], A.alpha[base], m, y0, k);
+        }
+        y2 = KIND == REC_REIN ? y0 : -y0;
     }
     double c1 = y1, c2 = y2;  // state at the start of the first live chunk
     int ckk = k, mx = 0;
     for (int c = 0; c < nch; ++c) {
-        const int l0 = m + TC_CH * c;
+        const int l0 = lb + TC_CH * c;
         __syncthreads();
-        if (tid < TC_CH) s_c[tid] = load_coef<REIN>(A, base, m, l0 + tid);
+        if (tid < TC_CH) s_c[tid] = load_coef<KIND>(A, base, m, l0 + tid);
         const bool dead = *s_first >= c;  // no value kept in the chunks before c
         __syncthreads();
         if (dead) {
@@ -216,10 +248,10 @@ __device__ __forceinline__ void tables_body(const TcArgs &A, int m, int blk, int
             for (int j = 16 * h; j < 16 * h + 16; ++j) {
                 const RecCoef C = s_c[j];
                 double y;
-                if (REIN) {
+                if (KIND == REC_REIN) {
                     y = rein_step(C.a, C.rh, C.b0, C.ci, u, y1, y2);
                 } else {
-                    y = fma(fma(-C.a, u, C.a), y1, -y2);
+                    y = fma(fma(-C.a, u, KIND == REC_SPIN ? C.rh : C.a), y1, -y2);
                     y2 = y1;
                     y1 = y;
                 }
@@ -241,6 +273,7 @@ __device__ __forceinline__ void tables_body(const TcArgs &A, int m, int blk, int
     ck_k[ci] = ckk;
 }
 
+template <bool SPIN>
 __global__ void __launch_bounds__(TC_T) tc_tables_kernel(TcArgs A, int *Ey_out, int *first_out, double2 *ck_y, int *ck_k)
 {
     __shared__ RecCoef s_c[TC_CH];
@@ -249,13 +282,15 @@ __global__ void __launch_bounds__(TC_T) tc_tables_kernel(TcArgs A, int *Ey_out, 
     const int blk = blockIdx.x - m * A.nblk;
     if (threadIdx.x == 0) {
         s_max = 0;
-        s_first = (A.lmax - m + TC_CH) / TC_CH;
+        s_first = (A.lmax - first_l<SPIN ? REC_SPIN : REC_Y>(m) + TC_CH) / TC_CH;
     }
     __syncthreads();
-    if (polar_block(A, m, blk))
-        tables_body<true>(A, m, blk, &s_max, &s_first, s_c, ck_y, ck_k);
+    if (SPIN)
+        tables_body<REC_SPIN>(A, m, blk, &s_max, &s_first, s_c, ck_y, ck_k);
+    else if (polar_block(A, m, blk))
+        tables_body<REC_REIN>(A, m, blk, &s_max, &s_first, s_c, ck_y, ck_k);
     else
-        tables_body<false>(A, m, blk, &s_max, &s_first, s_c, ck_y, ck_k);
+        tables_body<REC_Y>(A, m, blk, &s_max, &s_first, s_c, ck_y, ck_k);
     __syncthreads();
     if (threadIdx.x == 0) {
         Ey_out[m * A.nblk + blk] = s_max ? s_max - 1022 : -1000;
@@ -277,7 +312,7 @@ __global__ void __launch_bounds__(TC_T) tc_tables_kernel(TcArgs A, int *Ey_out, 
 // Stages: the y buffer is handed over with named barriers (FULL: recurrence arrives, split
 // waits; EMPTY: split arrives, recurrence waits, only where a later chunk reuses the stage);
 // the A/B tiles of a stage are rewritten after the done mbarrier of the MMAs that read them.
-template <int N>
+template <int N, bool SPIN>
 __global__ void __launch_bounds__(TC_NT + 32, 1) tc_synth_kernel(TcArgs A)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -302,7 +337,7 @@ __global__ void __launch_bounds__(TC_NT + 32, 1) tc_synth_kernel(TcArgs A)
     const bool active = slot < A.nslots;
     const int L = A.lmax;
     const int64_t base = (int64_t)m * (2 * L + 3 - m) / 2;
-    const int nch = (L - m + TC_CH) / TC_CH;
+    const int nch = (L - first_l<SPIN ? REC_SPIN : REC_Y>(m) + TC_CH) / TC_CH;
     const int cfirst = A.first[m * A.nblk + blk];           // chunks before it hold only dropped values
     const int nlive = nch - cfirst;
 
@@ -312,8 +347,10 @@ __global__ void __launch_bounds__(TC_NT + 32, 1) tc_synth_kernel(TcArgs A)
             const int64_t mstride = A.mmax + 1;
             for (int g = 0; g < A.nmaps; ++g) {
                 double2 *d = A.delta + (int64_t)g * A.nrings * mstride;
-                if (rn >= 0 && SHT_CHK(rn < A.nrings)) d[(int64_t)rn * mstride + m] = make_double2(0.0, 0.0);
-                if (rs >= 0 && SHT_CHK(rs < A.nrings)) d[(int64_t)rs * mstride + m] = make_double2(0.0, 0.0);
+                const bool own = !SPIN || ((g & 1) == 0) == (A.sig > 0);  // spin: see the epilogue
+                if (own && rn >= 0 && SHT_CHK(rn < A.nrings)) d[(int64_t)rn * mstride + m] = make_double2(0.0, 0.0);
+                if ((!SPIN || !own) && rs >= 0 && SHT_CHK(rs < A.nrings))
+                    d[(int64_t)rs * mstride + m] = make_double2(0.0, 0.0);
             }
         }
         return;
@@ -338,10 +375,12 @@ __global__ void __launch_bounds__(TC_NT + 32, 1) tc_synth_kernel(TcArgs A)
 
     bool ok = true;
     if (rec) {
-        if (polar_block(A, m, blk))
-            recurrence_warps<true, false, TC_T, 8>(A, m, blk, r, active, base, nch, cfirst, ybuf, abuf);
+        if (SPIN)
+            recurrence_warps<REC_SPIN, false, TC_T, 8>(A, m, blk, r, active, base, nch, cfirst, ybuf, abuf);
+        else if (polar_block(A, m, blk))
+            recurrence_warps<REC_REIN, false, TC_T, 8>(A, m, blk, r, active, base, nch, cfirst, ybuf, abuf);
         else
-            recurrence_warps<false, false, TC_T, 8>(A, m, blk, r, active, base, nch, cfirst, ybuf, abuf);
+            recurrence_warps<REC_Y, false, TC_T, 8>(A, m, blk, r, active, base, nch, cfirst, ybuf, abuf);
     } else if (issuer) {
         // ------------------------------------------------ MMA issue (one lane of the last warp)
         // per chunk: wait until the stage's tiles are written, issue its 2 x 20 MMAs (per parity eo,
@@ -465,18 +504,24 @@ __global__ void __launch_bounds__(TC_NT + 32, 1) tc_synth_kernel(TcArgs A)
                 for (int gg = 0; gg < 4; ++gg) {
                     const int g = 4 * cg + gg;  // map
                     if (g >= A.nmaps) break;
+                    const bool own = !SPIN || ((g & 1) == 0) == (A.sig > 0);
                     double vn[2], vs[2];
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
                         const int t = 2 * gg + c;
                         const int e = Ey + A.Ea[m * N + 8 * cg + t] - 36;  // class 3: 2^(-6 - 6 - 24)
-                        vn[c] = pair_to_double(hi[0][t] + hi[1][t], lo[0][t] + lo[1][t], e);
-                        vs[c] = pair_to_double(hi[0][t] - hi[1][t], lo[0][t] - lo[1][t], e);
+                        if (own) vn[c] = pair_to_double(hi[0][t] + hi[1][t], lo[0][t] + lo[1][t], e);
+                        if (!SPIN || !own) vs[c] = pair_to_double(hi[0][t] - hi[1][t], lo[0][t] - lo[1][t], e);
+                    }
+                    // spin: l - m starts odd at m = 1, where (-1)^(l+m) and with it E - O change sign
+                    if (SPIN && m == 1 && !own) {
+                        vs[0] = -vs[0];
+                        vs[1] = -vs[1];
                     }
                     double2 *d = A.delta + (int64_t)g * A.nrings * mstride;
-                    if (rn >= 0 && SHT_CHK(rn < A.nrings && m <= A.mmax))
+                    if (own && rn >= 0 && SHT_CHK(rn < A.nrings && m <= A.mmax))
                         d[(int64_t)rn * mstride + m] = make_double2(vn[0], vn[1]);
-                    if (rs >= 0 && SHT_CHK(rs < A.nrings && m <= A.mmax))
+                    if ((!SPIN || !own) && rs >= 0 && SHT_CHK(rs < A.nrings && m <= A.mmax))
                         d[(int64_t)rs * mstride + m] = make_double2(vs[0], vs[1]);
                 }
             }
@@ -489,15 +534,40 @@ __global__ void __launch_bounds__(TC_NT + 32, 1) tc_synth_kernel(TcArgs A)
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(W::TMEM_COLS));
 }
 
-template <int N>
+// Q and U from P+ and P- (see above), in place: [nmaps][2] planes of n values
+__global__ void spin_combine_kernel(double2 *__restrict__ delta, int64_t n, int nmaps)
+{
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n * nmaps; t += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t g = t / n, i = t - g * n;
+        double2 *q = delta + 2 * g * n + i, *u = q + n;
+        const double2 p = *q, w = *u;
+        *q = make_double2(-0.5 * (p.x + w.x), -0.5 * (p.y + w.y));
+        *u = make_double2(-0.5 * (p.y - w.y), 0.5 * (p.x - w.x));
+    }
+}
+
+template <int N, bool SPIN>
 cudaError_t launch_slab(const Plan &p, const TcArgs &A, int count_m, int64_t nchunks, cudaStream_t st)
 {
-    tc_scale_kernel<N><<<count_m, 256, 0, st>>>(A);
-    tc_split_b_kernel<N><<<(unsigned)nchunks, 4 * N, 0, st>>>(A);  // one thread per (parity, k half, column)
-    StageEvents ev(p, SHT_STAGE_TC_SYNTH_KERNEL, st);
-    tc_synth_kernel<N><<<(unsigned)(count_m * A.nblk), TC_NT + 32, TcTile<N>::SMEM, st>>>(A);
-    p.launches[SHT_STAGE_TC_SYNTH_KERNEL] += 1;
-    ev.done();
+    tc_scale_kernel<N, SPIN><<<count_m, 256, 0, st>>>(A);
+    tc_split_b_kernel<N, SPIN><<<(unsigned)nchunks, 4 * N, 0, st>>>(A);  // one thread per (parity, k half, column)
+    if (!SPIN) {
+        StageEvents ev(p, SHT_STAGE_TC_SYNTH_KERNEL, st);
+        tc_synth_kernel<N, false><<<(unsigned)(count_m * A.nblk), TC_NT + 32, TcTile<N>::SMEM, st>>>(A);
+        p.launches[SHT_STAGE_TC_SYNTH_KERNEL] += 1;
+        ev.done();
+    } else {  // both signs of the recurrence on the same columns
+        const size_t tables = (size_t)(p.mmax + 1) * A.nblk;
+        TcArgs B = A;
+        for (int sig = 1; sig >= -1; sig -= 2) {
+            B.sig = sig;
+            tc_synth_kernel<N, true><<<(unsigned)(count_m * A.nblk), TC_NT + 32, TcTile<N>::SMEM, st>>>(B);
+            B.Ey += 2 * tables;
+            B.first += 2 * tables;
+            B.ck_y += tables * TC_T;
+            B.ck_k += tables * TC_T;
+        }
+    }
     return cudaGetLastError();
 }
 
@@ -540,37 +610,46 @@ size_t exponent_bytes(const Plan &p) { return (size_t)(p.mmax + 1) * (32 + 16) *
 cudaError_t configure_tc_kernels()
 {
     const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaError_t e = cudaFuncSetAttribute(tc_synth_kernel<32>, a, TcTile<32>::SMEM);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_synth_kernel<16>, a, TcTile<16>::SMEM);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_synth_kernel<8>, a, TcTile<8>::SMEM);
+    cudaError_t e = cudaFuncSetAttribute(tc_synth_kernel<32, false>, a, TcTile<32>::SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_synth_kernel<16, false>, a, TcTile<16>::SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_synth_kernel<8, false>, a, TcTile<8>::SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_synth_kernel<32, true>, a, TcTile<32>::SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_synth_kernel<16, true>, a, TcTile<16>::SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_synth_kernel<8, true>, a, TcTile<8>::SMEM);
     if (e == cudaSuccess) e = configure_tc_anal_kernel();
     return e;
 }
 
-// Plan tables of the tensor-core kernels (synchronous, once per plan).
-cudaError_t build_tc_tables(Plan &p)
+// Plan tables of the tensor-core kernels (synchronous, once per plan); spin: for both signs, + first.
+static cudaError_t build_tables(const Plan &p, bool spin, int **ey_out, double2 **cky_out, int **ckk_out)
 {
-    if (p.d_tc_Ey) return cudaSuccess;
     TcArgs A{};
     A.u = p.d_u;
     A.s = p.d_s;
     A.alpha = p.d_alpha;
     A.cfac = p.d_cfac;
     A.rein = p.d_rein;
+    A.tab = p.d_spin_tab;
+    A.start = p.d_spin_start;
     A.mR = p.mR;
     A.nslots = p.nslots;
     A.nblk = (p.nslots + TC_T - 1) / TC_T;
     A.lmax = p.lmax;
     A.mmax = p.mmax;
-    int *ey = nullptr;  // [2][mmax + 1][nblk]: y exponents, then first live chunks
-    const size_t n = (size_t)(p.mmax + 1) * A.nblk;
+    int *ey = nullptr;  // per sign [2][mmax + 1][nblk]: y exponents, then first live chunks
+    const size_t n = (size_t)(p.mmax + 1) * A.nblk, ns = spin ? 2 : 1;
     double2 *cky = nullptr;
     int *ckk = nullptr;
-    cudaError_t e = sht::dev_malloc(&ey, sizeof(int) * 2 * n);
-    if (e == cudaSuccess) e = sht::dev_malloc(&cky, sizeof(double2) * n * TC_T);
-    if (e == cudaSuccess) e = sht::dev_malloc(&ckk, sizeof(int) * n * TC_T);
-    if (e == cudaSuccess) {
-        tc_tables_kernel<<<(unsigned)n, TC_T>>>(A, ey, ey + n, cky, ckk);
+    cudaError_t e = sht::dev_malloc(&ey, sizeof(int) * 2 * n * ns);
+    if (e == cudaSuccess) e = sht::dev_malloc(&cky, sizeof(double2) * n * TC_T * ns);
+    if (e == cudaSuccess) e = sht::dev_malloc(&ckk, sizeof(int) * n * TC_T * ns);
+    for (size_t k = 0; k < ns && e == cudaSuccess; ++k) {
+        A.sig = k == 0 ? 1 : -1;
+        int *ek = ey + 2 * n * k;
+        if (spin)
+            tc_tables_kernel<true><<<(unsigned)n, TC_T>>>(A, ek, ek + n, cky + n * TC_T * k, ckk + n * TC_T * k);
+        else
+            tc_tables_kernel<false><<<(unsigned)n, TC_T>>>(A, ek, ek + n, cky, ckk);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -580,10 +659,20 @@ cudaError_t build_tc_tables(Plan &p)
         cudaFree(ckk);
         return e;
     }
-    p.d_tc_Ey = ey;
-    p.d_tc_ck_y = cky;
-    p.d_tc_ck_k = ckk;
+    *ey_out = ey;
+    *cky_out = cky;
+    *ckk_out = ckk;
     return cudaSuccess;
+}
+
+cudaError_t build_tc_tables(Plan &p)
+{
+    return p.d_tc_Ey ? cudaSuccess : build_tables(p, false, &p.d_tc_Ey, &p.d_tc_ck_y, &p.d_tc_ck_k);
+}
+
+cudaError_t build_tc_spin_tables(Plan &p)
+{
+    return p.d_sp_Ey ? cudaSuccess : build_tables(p, true, &p.d_sp_Ey, &p.d_sp_ck_y, &p.d_sp_ck_k);
 }
 
 // FP64-mode plans whose Legendre steps run here instead of in the plain FP64 kernels of legendre.cu.
@@ -615,9 +704,9 @@ size_t tc_workspace_least(const Plan &p, int nmaps)
 // Legendre synthesis on the tensor cores in `scratch_bytes` of scratch (tc_workspace_least or more):
 // per group of up to 16 maps and per slab of whole m whose digits fit, the scale, split and synthesis
 // kernels, and last the plain FP64 sums of the columns that were marked.  The slabs do not change
-// the results.
-cudaError_t launch_legendre_synth_tc(const Plan &p, const double2 *alm, double2 *delta, void *scratch,
-                                     size_t scratch_bytes, int nmaps, cudaStream_t st, int *nlaunch)
+// the results.  spin: nmaps counts the column pairs (two per polarised map), delta ends as Q and U.
+static cudaError_t synth_tc(const Plan &p, bool spin, const double2 *alm, double2 *delta, void *scratch,
+                            size_t scratch_bytes, int nmaps, cudaStream_t st, int *nlaunch)
 {
     *nlaunch = 0;
     TcArgs A{};
@@ -628,21 +717,22 @@ cudaError_t launch_legendre_synth_tc(const Plan &p, const double2 *alm, double2 
     A.alpha = p.d_alpha;
     A.cfac = p.d_cfac;
     A.rein = p.d_rein;
-    A.Ey = p.d_tc_Ey;
-    A.first = p.d_tc_Ey + (size_t)(p.mmax + 1) * ((p.nslots + TC_T - 1) / TC_T);
-    A.ck_y = p.d_tc_ck_y;
-    A.ck_k = p.d_tc_ck_k;
+    A.tab = p.d_spin_tab;
+    A.nblk = (p.nslots + TC_T - 1) / TC_T;
+    A.Ey = spin ? p.d_sp_Ey : p.d_tc_Ey;
+    A.first = A.Ey + (size_t)(p.mmax + 1) * A.nblk;
+    A.ck_y = spin ? p.d_sp_ck_y : p.d_tc_ck_y;
+    A.ck_k = spin ? p.d_sp_ck_k : p.d_tc_ck_k;
     A.chunk_base = p.d_tc_chunk_base;
     A.chunk_m = p.d_tc_chunk_m;
     A.status = p.d_status;
     A.nslots = p.nslots;
-    A.nblk = (p.nslots + TC_T - 1) / TC_T;
     A.lmax = p.lmax;
     A.mmax = p.mmax;
     A.nrings = p.nrings;
     A.mR = p.mR;
     A.nalm = p.nalm;
-    A.mflag = p.d_mflag;
+    A.mflag = spin ? nullptr : p.d_mflag;
     A.fix = (int *)scratch;  // [mmax + 1][16], then Ea [mmax + 1][N], then the digits
     A.Ea = A.fix + (size_t)(p.mmax + 1) * 16;
     const size_t head = (exponent_bytes(p) + 255) & ~(size_t)255;
@@ -661,19 +751,47 @@ cudaError_t launch_legendre_synth_tc(const Plan &p, const double2 *alm, double2 
             A.m0 = m0;
             A.chunk0 = tc_chunks_below(p, m0);
             const int64_t nch = tc_chunks_below(p, m1) - A.chunk0;
-            cudaError_t e = N == 32   ? launch_slab<32>(p, A, m1 - m0, nch, st)
-                            : N == 16 ? launch_slab<16>(p, A, m1 - m0, nch, st)
-                                      : launch_slab<8>(p, A, m1 - m0, nch, st);
-            *nlaunch += 3;
+            cudaError_t e;
+            if (spin)
+                e = N == 32   ? launch_slab<32, true>(p, A, m1 - m0, nch, st)
+                    : N == 16 ? launch_slab<16, true>(p, A, m1 - m0, nch, st)
+                              : launch_slab<8, true>(p, A, m1 - m0, nch, st);
+            else
+                e = N == 32   ? launch_slab<32, false>(p, A, m1 - m0, nch, st)
+                    : N == 16 ? launch_slab<16, false>(p, A, m1 - m0, nch, st)
+                              : launch_slab<8, false>(p, A, m1 - m0, nch, st);
+            *nlaunch += spin ? 4 : 3;
             if (e != cudaSuccess) return e;
             m0 = m1;
         }
-        cudaError_t e = launch_legendre_synth_fix(p, A.alm, A.delta, A.fix, nm, st);
+        cudaError_t e;
+        if (spin) {
+            spin_combine_kernel<<<152 * 16, 256, 0, st>>>(A.delta, dstride, nm / 2);
+            ++*nlaunch;
+            e = cudaGetLastError();
+            if (e == cudaSuccess) e = launch_spin_synth_fix(p, A.alm, A.delta, A.fix, nm / 2, st);
+        } else {
+            e = launch_legendre_synth_fix(p, A.alm, A.delta, A.fix, nm, st);
+        }
         *nlaunch += 1;
         if (e != cudaSuccess) return e;
         g0 += nm;
     }
     return cudaSuccess;
+}
+
+cudaError_t launch_legendre_synth_tc(const Plan &p, const double2 *alm, double2 *delta, void *scratch,
+                                     size_t scratch_bytes, int nmaps, cudaStream_t st, int *nlaunch)
+{
+    return synth_tc(p, false, alm, delta, scratch, scratch_bytes, nmaps, st, nlaunch);
+}
+
+// spin 2: alm [nmaps][2][nalm] (E, B) to delta [nmaps][2][nrings][mmax + 1] (Q, U), in
+// tc_workspace_bytes(p, 2 nmaps) of scratch
+cudaError_t launch_spin_synth_tc(const Plan &p, const double2 *alm, double2 *delta, void *scratch, size_t scratch_bytes,
+                                 int nmaps, cudaStream_t st, int *nlaunch)
+{
+    return synth_tc(p, true, alm, delta, scratch, scratch_bytes, 2 * nmaps, st, nlaunch);
 }
 
 namespace {

@@ -27,6 +27,12 @@
 // so the MMAs run region by region (t = 0, 2, 4, 6) over the chunk's 8 K-steps, and the epilogue
 // reads one region while the next is computed: each region has its own full and free barrier.
 //
+// Spin 2 (polarisation).  With a+- = sum over rings of lambda+- (Dq +- i Du) (spin.cu), E = -(a+ + a-) / 2
+// and B = i (a+ - a-) / 2.  A map's pair is two complex columns, and two passes, one per sign of the
+// recurrence, each add to both: the northern ring of the pass's own sign, the same for every l, and
+// the southern ring of the other sign times (-1)^(l+m).  The reduction of the second pass adds the
+// first's result and forms E and B.
+//
 // What bounds it: the FP64 recurrence, 64 FP64 instructions per warp and chunk = 4096 SM cycles.
 #include "sht_internal.h"
 
@@ -103,6 +109,7 @@ __device__ __forceinline__ void tmem_st4(uint32_t addr, uint32_t a, uint32_t b, 
 // their outcome (bar.red) so that their named barriers stay balanced.
 // The code of the roles competes for the instruction caches, and each warp runs in order: with four
 // epilogue warps of twice the code (everything unrolled) a chunk took them 9.7K cycles.
+template <bool SPIN>
 __global__ void __launch_bounds__(TA_NT, 1) tc_anal_kernel(TcArgs A)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -130,7 +137,8 @@ __global__ void __launch_bounds__(TA_NT, 1) tc_anal_kernel(TcArgs A)
     const bool active = slot < A.nslots;
     const int L = A.lmax;
     const int64_t base = (int64_t)m * (2 * L + 3 - m) / 2;
-    const int nch = (L - m + TC_CH) / TC_CH;
+    const int lb = first_l<SPIN ? REC_SPIN : REC_Y>(m);
+    const int nch = (L - lb + TC_CH) / TC_CH;
     const int cfirst = A.first[m * A.nblk + blk];           // chunks before it hold only dropped values:
     const int nlive = nch - cfirst;                         // the reduction leaves them out
     const int nm = A.nmaps;
@@ -160,10 +168,12 @@ __global__ void __launch_bounds__(TA_NT, 1) tc_anal_kernel(TcArgs A)
     bool ok = true;
     if (rec) {
         bar_sync(BAR_STAGED, TC_NT);  // X staged: its additions need the FP64 pipe first
-        if (polar_block(A, m, blk))
-            recurrence_warps<true, true, TA_YS, 4>(A, m, blk, r, active, base, nch, cfirst, ybuf, abuf);
+        if (SPIN)
+            recurrence_warps<REC_SPIN, true, TA_YS, 4>(A, m, blk, r, active, base, nch, cfirst, ybuf, abuf);
+        else if (polar_block(A, m, blk))
+            recurrence_warps<REC_REIN, true, TA_YS, 4>(A, m, blk, r, active, base, nch, cfirst, ybuf, abuf);
         else
-            recurrence_warps<false, true, TA_YS, 4>(A, m, blk, r, active, base, nch, cfirst, ybuf, abuf);
+            recurrence_warps<REC_Y, true, TA_YS, 4>(A, m, blk, r, active, base, nch, cfirst, ybuf, abuf);
     } else if (issuer) {
         // ------------------------------------------------ MMA issue (one lane of the last warp)
         const uint32_t idesc = umma_idesc<TA_N>();  // M = 128, N = 64
@@ -212,22 +222,49 @@ __global__ void __launch_bounds__(TA_NT, 1) tc_anal_kernel(TcArgs A)
             const double2 *dN = A.delta + (int64_t)(bn ? rn : 0) * mstride + m;
             const double2 *dS = A.delta + (int64_t)(bs ? rs : 0) * mstride + m;
             double2 n8[8], s8[8];
+            if (SPIN) {
+                // column pair 2 h + c of polarised map h (this thread: h = hh, hh + 2, ...): Q and U of the
+                // northern ring for the pass's own sign c, of the southern ring for the other
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int g = hh + 2 * i;
-                n8[i] = (bn && g < nm) ? dN[g * dstride] : make_double2(0.0, 0.0);
-                s8[i] = (bs && g < nm) ? dS[g * dstride] : make_double2(0.0, 0.0);
-            }
+                for (int i = 0; i < 8; ++i) {
+                    const int g = 2 * (hh + 2 * (i >> 1)), c = i & 1;  // Q plane of the map, sign (0: +)
+                    const bool own = (c == 0) == (A.sig > 0);
+                    const bool have = (own ? bn : bs) && g < nm;
+                    const double2 *d = own ? dN : dS;
+                    n8[i] = have ? d[g * dstride] : make_double2(0.0, 0.0);
+                    s8[i] = have ? d[(g + 1) * dstride] : make_double2(0.0, 0.0);
+                }
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int row = 2 * (hh + 2 * i);
-                if (hh + 2 * i < nm) {
-                    xr[row] = n8[i].x + s8[i].x;
-                    xr[row + 1] = n8[i].y + s8[i].y;
-                    xr[32 + row] = n8[i].x - s8[i].x;
-                    xr[33 + row] = n8[i].y - s8[i].y;
-                } else {
-                    xr[row] = xr[row + 1] = xr[32 + row] = xr[33 + row] = 0.0;
+                for (int i = 0; i < 8; ++i) {
+                    const int c = i & 1, row = 2 * (2 * (hh + 2 * (i >> 1)) + c);
+                    const bool own = (c == 0) == (A.sig > 0);
+                    // Dq +- i Du; even and odd l - max(m, 2) rows
+                    const double re = c == 0 ? n8[i].x - s8[i].y : n8[i].x + s8[i].y;
+                    const double im = c == 0 ? n8[i].y + s8[i].x : n8[i].y - s8[i].x;
+                    const bool neg = !own && m == 1;  // (-1)^(l+m) of the even rows
+                    xr[row] = neg ? -re : re;
+                    xr[row + 1] = neg ? -im : im;
+                    xr[32 + row] = own || neg ? re : -re;
+                    xr[33 + row] = own || neg ? im : -im;
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int g = hh + 2 * i;
+                    n8[i] = (bn && g < nm) ? dN[g * dstride] : make_double2(0.0, 0.0);
+                    s8[i] = (bs && g < nm) ? dS[g * dstride] : make_double2(0.0, 0.0);
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int row = 2 * (hh + 2 * i);
+                    if (hh + 2 * i < nm) {
+                        xr[row] = n8[i].x + s8[i].x;
+                        xr[row + 1] = n8[i].y + s8[i].y;
+                        xr[32 + row] = n8[i].x - s8[i].x;
+                        xr[33 + row] = n8[i].y - s8[i].y;
+                    } else {
+                        xr[row] = xr[row + 1] = xr[32 + row] = xr[33 + row] = 0.0;
+                    }
                 }
             }
         }
@@ -327,7 +364,7 @@ __global__ void __launch_bounds__(TA_NT, 1) tc_anal_kernel(TcArgs A)
         float4 *mine = xch + (tid - TC_NT), *other = xch + ((tid - TC_NT) ^ 64);
         const uint32_t row0 = tmem + ((uint32_t)(32 * qd) << 16) + (uint32_t)(16 * es);
         // partial sum of column t0 + j: l = l1 + 2 j of the chunk
-        const int l1 = m + TC_CH * cfirst + es + 2 * t0;
+        const int l1 = lb + TC_CH * cfirst + es + 2 * t0;
         double *dst = (double *)(A.partial + (int64_t)blk * A.nalm_part * nm + (base - A.idx0 + (l1 - m)) * nm + eg) + ec;
         for (int q = 0; q < nlive; ++q) {
             float v[TA_REG][2][4];
@@ -411,7 +448,9 @@ __global__ void __launch_bounds__(TA_NT, 1) tc_anal_kernel(TcArgs A)
 // 32-l chunk of one m: it reads the [32 l][nmaps] partial sums of each block as one contiguous
 // piece and turns them through shared memory into the coefficient rows of each map.  Bound by
 // DRAM: live blocks x 16 B read per coefficient and map, 16 B written.
+// Spin: the first pass writes c_lm a+-, the second adds its own and turns the pair into E and B.
 constexpr int TR_T = 256;
+template <bool SPIN>
 __global__ void __launch_bounds__(TR_T) tc_reduce_kernel(TcArgs A, double2 *__restrict__ alm)
 {
     __shared__ double2 s_v[TC_CH * (TA_MAPS + 1)];
@@ -419,8 +458,12 @@ __global__ void __launch_bounds__(TR_T) tc_reduce_kernel(TcArgs A, double2 *__re
     const int64_t chunk = A.chunk0 + blockIdx.x;
     const int m = A.chunk_m[chunk];
     const int c = (int)(chunk - A.chunk_base[m]);
-    const int l0 = m + TC_CH * c, nl = min(TC_CH, A.lmax - l0 + 1), nm = A.nmaps;
+    const int lb = first_l<SPIN ? REC_SPIN : REC_Y>(m);
+    const int l0 = lb + TC_CH * c, nl = max(0, min(TC_CH, A.lmax - l0 + 1)), nm = A.nmaps;
     const int64_t ix0 = (int64_t)m * (2 * A.lmax + 3 - m) / 2 + (l0 - m);
+    if (SPIN && c == 0)  // no spin-2 function below l = 2
+        for (int t = threadIdx.x; t < (min(lb, A.lmax + 1) - m) * nm; t += TR_T)
+            alm[(int64_t)(t % nm) * A.nalm + ix0 - (lb - m) + t / nm] = make_double2(0.0, 0.0);
     const int tot = nl * nm;
     const int64_t bstride = A.nalm_part * nm;
     const double2 *src = A.partial + (ix0 - A.idx0) * nm;
@@ -463,9 +506,26 @@ __global__ void __launch_bounds__(TR_T) tc_reduce_kernel(TcArgs A, double2 *__re
     __syncthreads();
     for (int t = threadIdx.x; t < tot; t += TR_T) {
         const int g = t / nl, l = t - g * nl;
-        const double cf = A.cfac[ix0 + l];
-        const double2 s = s_v[l * (TA_MAPS + 1) + g];
-        alm[(int64_t)g * A.nalm + ix0 + l] = make_double2(cf * s.x, m == 0 ? 0.0 : cf * s.y);
+        double2 *out = alm + (int64_t)g * A.nalm + ix0 + l;
+        if (!SPIN) {
+            const double cf = A.cfac[ix0 + l];
+            const double2 s = s_v[l * (TA_MAPS + 1) + g];
+            *out = make_double2(cf * s.x, m == 0 ? 0.0 : cf * s.y);
+        } else if ((g & 1) == 0) {
+            const double cf = A.tab[ix0 + l].w;
+            const double2 s = s_v[l * (TA_MAPS + 1) + g], r = s_v[l * (TA_MAPS + 1) + g + 1];
+            double2 p = make_double2(cf * s.x, cf * s.y), q = make_double2(cf * r.x, cf * r.y);
+            if (A.sig < 0) {
+                const double2 p0 = out[0], q0 = out[A.nalm];
+                p = make_double2(p.x + p0.x, p.y + p0.y);
+                q = make_double2(q.x + q0.x, q.y + q0.y);
+                out[0] = make_double2(-0.5 * (p.x + q.x), m == 0 ? 0.0 : -0.5 * (p.y + q.y));
+                out[A.nalm] = make_double2(-0.5 * (p.y - q.y), m == 0 ? 0.0 : 0.5 * (p.x - q.x));
+            } else {
+                out[0] = p;
+                out[A.nalm] = q;
+            }
+        }
     }
 }
 static_assert(2 * TR_T >= TC_CH * TA_MAPS, "two values a thread");
@@ -507,7 +567,9 @@ size_t fix_bytes(const Plan &p) { return ((size_t)(p.mmax + 1) * 16 * sizeof(int
 
 cudaError_t configure_tc_anal_kernel()
 {
-    return cudaFuncSetAttribute(tc_anal_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TA_SMEM);
+    const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    const cudaError_t e = cudaFuncSetAttribute(tc_anal_kernel<false>, a, TA_SMEM);
+    return e == cudaSuccess ? cudaFuncSetAttribute(tc_anal_kernel<true>, a, TA_SMEM) : e;
 }
 
 // marks of the columns left to the plain FP64 sums, then the partial a_lm / c_lm per 128-slot block
@@ -523,9 +585,9 @@ size_t tc_anal_partial_bytes(const Plan &p, int nmaps)
 
 // Legendre analysis on the tensor cores: per group of up to 16 maps and per m-slab the tensor-core
 // kernel, the fixed-order block reduction of that slab into a_lm and the plain FP64 sums of the
-// columns that were marked.
-cudaError_t launch_legendre_anal_tc(const Plan &p, const double2 *delta, double2 *alm, void *partial, int nmaps,
-                                    cudaStream_t st, int *nlaunch)
+// columns that were marked.  spin: nmaps counts the column pairs (two per polarised map).
+static cudaError_t anal_tc(const Plan &p, bool spin, const double2 *delta, double2 *alm, void *partial, int nmaps,
+                           cudaStream_t st, int *nlaunch)
 {
     *nlaunch = 0;
     TcArgs A{};
@@ -536,21 +598,19 @@ cudaError_t launch_legendre_anal_tc(const Plan &p, const double2 *delta, double2
     A.alpha = p.d_alpha;
     A.cfac = p.d_cfac;
     A.rein = p.d_rein;
-    A.Ey = p.d_tc_Ey;
-    A.first = p.d_tc_Ey + (size_t)(p.mmax + 1) * ((p.nslots + TC_T - 1) / TC_T);
-    A.ck_y = p.d_tc_ck_y;
-    A.ck_k = p.d_tc_ck_k;
+    A.tab = p.d_spin_tab;
+    A.nblk = (p.nslots + TC_T - 1) / TC_T;
+    const size_t tables = (size_t)(p.mmax + 1) * A.nblk;
     A.chunk_base = p.d_tc_chunk_base;
     A.chunk_m = p.d_tc_chunk_m;
     A.status = p.d_status;
     A.nslots = p.nslots;
-    A.nblk = (p.nslots + TC_T - 1) / TC_T;
     A.lmax = p.lmax;
     A.mmax = p.mmax;
     A.nrings = p.nrings;
     A.mR = p.mR;
     A.nalm = p.nalm;
-    A.mflag = p.d_mflag;
+    A.mflag = spin ? nullptr : p.d_mflag;
     A.fix = (int *)partial;
     A.partial = (double2 *)((char *)partial + fix_bytes(p));
     const int64_t dstride = (int64_t)p.nrings * (p.mmax + 1);
@@ -570,22 +630,49 @@ cudaError_t launch_legendre_anal_tc(const Plan &p, const double2 *delta, double2
             A.idx0 = idx(mlo);
             A.nalm_part = (mhi > p.mmax ? p.nalm : idx(mhi)) - A.idx0;
             A.chunk0 = tc_chunks_below(p, mlo);
-            {
-                StageEvents ev(p, SHT_STAGE_TC_ANAL_KERNEL, st);
-                tc_anal_kernel<<<(unsigned)((mhi - mlo) * A.nblk), TA_NT, TA_SMEM, st>>>(A);
-                p.launches[SHT_STAGE_TC_ANAL_KERNEL] += 1;
-                ev.done();
+            const unsigned grid = (unsigned)((mhi - mlo) * A.nblk);
+            const unsigned rgrid = (unsigned)(tc_chunks_below(p, mhi) - A.chunk0);
+            for (int pass = 0; pass < (spin ? 2 : 1); ++pass) {
+                A.sig = pass == 0 ? 1 : -1;
+                A.Ey = (spin ? p.d_sp_Ey : p.d_tc_Ey) + 2 * tables * pass;
+                A.first = A.Ey + tables;
+                A.ck_y = (spin ? p.d_sp_ck_y : p.d_tc_ck_y) + tables * TC_T * pass;
+                A.ck_k = (spin ? p.d_sp_ck_k : p.d_tc_ck_k) + tables * TC_T * pass;
+                if (spin) {
+                    tc_anal_kernel<true><<<grid, TA_NT, TA_SMEM, st>>>(A);
+                    tc_reduce_kernel<true><<<rgrid, TR_T, 0, st>>>(A, out);
+                } else {
+                    StageEvents ev(p, SHT_STAGE_TC_ANAL_KERNEL, st);
+                    tc_anal_kernel<false><<<grid, TA_NT, TA_SMEM, st>>>(A);
+                    p.launches[SHT_STAGE_TC_ANAL_KERNEL] += 1;
+                    ev.done();
+                    tc_reduce_kernel<false><<<rgrid, TR_T, 0, st>>>(A, out);
+                }
+                *nlaunch += 2;
+                e = cudaGetLastError();
+                if (e != cudaSuccess) return e;
             }
-            tc_reduce_kernel<<<(unsigned)(tc_chunks_below(p, mhi) - A.chunk0), TR_T, 0, st>>>(A, out);
-            *nlaunch += 2;
-            e = cudaGetLastError();
-            if (e != cudaSuccess) return e;
-            e = launch_legendre_anal_fix(p, A.delta, out, A.partial, A.fix, nm, mlo, mhi, A.idx0, A.nalm_part, st);
+            e = spin ? launch_spin_anal_fix(p, A.delta, out, A.partial, A.fix, nm / 2, mlo, mhi, A.idx0, A.nalm_part, st)
+                     : launch_legendre_anal_fix(p, A.delta, out, A.partial, A.fix, nm, mlo, mhi, A.idx0, A.nalm_part, st);
             *nlaunch += 1;
             if (e != cudaSuccess) return e;
         }
     }
     return cudaSuccess;
+}
+
+cudaError_t launch_legendre_anal_tc(const Plan &p, const double2 *delta, double2 *alm, void *partial, int nmaps,
+                                    cudaStream_t st, int *nlaunch)
+{
+    return anal_tc(p, false, delta, alm, partial, nmaps, st, nlaunch);
+}
+
+// spin 2: delta [nmaps][2][nrings][mmax + 1] (Q, U) to alm [nmaps][2][nalm] (E, B), in
+// tc_anal_partial_bytes(p, 2 nmaps) of scratch
+cudaError_t launch_spin_anal_tc(const Plan &p, const double2 *delta, double2 *alm, void *partial, int nmaps,
+                                cudaStream_t st, int *nlaunch)
+{
+    return anal_tc(p, true, delta, alm, partial, 2 * nmaps, st, nlaunch);
 }
 
 namespace {

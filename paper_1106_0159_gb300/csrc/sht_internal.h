@@ -113,6 +113,9 @@ struct Plan {
     int n_mlist = 0;                    // number of listed m (0: all)
     double4 *d_spin_tab = nullptr;      // spin 2: [nalm] (alpha, alpha (1 + g), alpha (1 - g), c), built on first use
     double *d_spin_start = nullptr;     // spin 2: [mmax + 1] start coefficients S_m
+    int *d_sp_Ey = nullptr;             // spin 2 on the tensor cores: as d_tc_Ey, d_tc_ck_*, for the signs + and -
+    double2 *d_sp_ck_y = nullptr;
+    int *d_sp_ck_k = nullptr;
     bool tc64 = false;                  // the FP64 mode's Legendre steps take the tensor-core kernels (tc_fp64_plan)
     bool split_ready = false;           // the plan has been switched to the precision form once
     bool polar_first_slot = false;      // slot 0 runs the Reinsch form (sin(theta) < 0.03)
@@ -196,6 +199,16 @@ cudaError_t launch_legendre_synth_fix(const Plan &p, const double2 *alm, double2
                                       cudaStream_t st);
 cudaError_t launch_legendre_anal_fix(const Plan &p, const double2 *delta, double2 *alm, double2 *partial, const int *fix,
                                      int nmaps, int m0, int m1, int64_t idx0, int64_t nalm_part, cudaStream_t st);
+
+cudaError_t build_tc_spin_tables(Plan &p);
+cudaError_t launch_spin_synth_tc(const Plan &p, const double2 *alm, double2 *delta, void *scratch, size_t scratch_bytes,
+                                 int nmaps, cudaStream_t st, int *nlaunch);
+cudaError_t launch_spin_anal_tc(const Plan &p, const double2 *delta, double2 *alm, void *partial, int nmaps,
+                                cudaStream_t st, int *nlaunch);
+cudaError_t launch_spin_synth_fix(const Plan &p, const double2 *alm, double2 *delta, const int *fix, int nmaps,
+                                  cudaStream_t st);
+cudaError_t launch_spin_anal_fix(const Plan &p, const double2 *delta, double2 *alm, double2 *partial, const int *fix,
+                                 int nmaps, int m0, int m1, int64_t idx0, int64_t nalm_part, cudaStream_t st);
 
 // spin-2 transforms (spin.cu): Legendre steps on [nmaps][2] coefficient / Delta pairs
 cudaError_t build_spin_tables(Plan &p);

@@ -98,7 +98,8 @@ void free_plan_device(Plan &p)
     void *ptrs[] = {p.d_slotN, p.d_slotS, p.d_u,     p.d_s,     p.d_alpha,   p.d_cfac,    p.d_ofs, p.d_nphi,
                     p.d_w,     p.d_phase, p.d_items, p.d_lens,  p.d_fft_tab, p.d_rein, p.d_ws,
                     p.d_tc_chunk_base, p.d_tc_chunk_m, p.d_tc_Ey, p.d_status, p.d_fft_tab_df, p.d_phase_df,
-                    p.d_tc_ck_y, p.d_tc_ck_k, p.d_spin_tab, p.d_spin_start, p.d_mflag, p.d_fft_perm};
+                    p.d_tc_ck_y, p.d_tc_ck_k, p.d_spin_tab, p.d_spin_start, p.d_mflag, p.d_fft_perm,
+                    p.d_sp_Ey, p.d_sp_ck_y, p.d_sp_ck_k};
     for (void *q : ptrs)
         if (q) cudaFree(q);
     p.d_slotN = p.d_slotS = nullptr;
@@ -121,6 +122,9 @@ void free_plan_device(Plan &p)
     p.d_tc_ck_k = nullptr;
     p.d_spin_tab = nullptr;
     p.d_spin_start = nullptr;
+    p.d_sp_Ey = nullptr;
+    p.d_sp_ck_y = nullptr;
+    p.d_sp_ck_k = nullptr;
     p.d_mflag = nullptr;
     p.n_mlist = 0;
     p.d_fft_perm = nullptr;
@@ -777,6 +781,7 @@ static sht_status spin_prepare(Plan &p, int spin)
         return SHT_EUNSUPPORTED;
     }
     cudaError_t e = sht::build_spin_tables(p);
+    if (e == cudaSuccess && sht::tc_fp64_plan(p)) e = sht::build_tc_spin_tables(p);
     if (e != cudaSuccess) return cuda_fail(p, e, "spin tables");
     return SHT_OK;
 }
@@ -786,7 +791,10 @@ size_t sht_spin_workspace_bytes(sht_plan_t plan, int nmaps)
     if (!plan || nmaps <= 0) return 0;
     const Plan &p = plan->p;
     return align256(delta_bytes(p, 2 * nmaps)) +
-           std::max(align256(sht::ring_scratch_bytes(p)), align256(sht::spin_partial_bytes(p, std::min(nmaps, 2))));
+           std::max(align256(sht::ring_scratch_bytes(p)),
+                    sht::tc_fp64_plan(p) ? std::max(align256(sht::tc_workspace_bytes(p, 2 * nmaps)),
+                                                    align256(sht::tc_anal_partial_bytes(p, 2 * nmaps)))
+                                         : align256(sht::spin_partial_bytes(p, std::min(nmaps, 2))));
 }
 
 sht_status sht_alm2map_spin(sht_plan_t plan, int spin, const void *alm, double *map, int nmaps, void *stream)
@@ -804,7 +812,10 @@ sht_status sht_alm2map_spin(sht_plan_t plan, int spin, const void *alm, double *
     {
         StageScope sc(p, SHT_STAGE_LEGENDRE_SYNTH, s);
         int n = 0;
-        cudaError_t e = sht::launch_spin_synth(p, (const double2 *)alm, delta, nmaps, s, &n);
+        cudaError_t e = sht::tc_fp64_plan(p)
+                            ? sht::launch_spin_synth_tc(p, (const double2 *)alm, delta, scratch,
+                                                        sht::tc_workspace_bytes(p, 2 * nmaps), nmaps, s, &n)
+                            : sht::launch_spin_synth(p, (const double2 *)alm, delta, nmaps, s, &n);
         p.launches[SHT_STAGE_LEGENDRE_SYNTH] += n;
         if (e != cudaSuccess) return cuda_fail(p, e, "spin legendre_synth");
         sc.done();
@@ -828,7 +839,8 @@ sht_status sht_map2alm_spin(sht_plan_t plan, int spin, const double *map, void *
     if (st != SHT_OK) return st;
     StageScope sc(p, SHT_STAGE_LEGENDRE_ANAL, s);
     int n = 0;
-    cudaError_t e = sht::launch_spin_anal(p, delta, (double2 *)alm, scratch, nmaps, s, &n);
+    cudaError_t e = sht::tc_fp64_plan(p) ? sht::launch_spin_anal_tc(p, delta, (double2 *)alm, scratch, nmaps, s, &n)
+                                         : sht::launch_spin_anal(p, delta, (double2 *)alm, scratch, nmaps, s, &n);
     p.launches[SHT_STAGE_LEGENDRE_ANAL] += n;
     if (e != cudaSuccess) return cuda_fail(p, e, "spin legendre_anal");
     sc.done();

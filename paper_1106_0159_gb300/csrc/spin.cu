@@ -109,12 +109,9 @@ __device__ __forceinline__ bool spin_rescale(double &p1, double &p2, double &m1,
 }
 
 template <int NM>
-__global__ void __launch_bounds__(SP_T) spin_synth_kernel(SpinArgs A)
+__device__ __forceinline__ void spin_synth_body(const SpinArgs &A, int m, int blk, double4 *s_t, double2 (*s_e)[SP_CH],
+                                                double2 (*s_b)[SP_CH])
 {
-    __shared__ double4 s_t[SP_CH];
-    __shared__ double2 s_e[NM][SP_CH], s_b[NM][SP_CH];
-    const int m = blockIdx.x / A.nblk;
-    const int blk = blockIdx.x - m * A.nblk;
     const int slot = blk * SP_T + threadIdx.x;
     const bool active = slot < A.nslots;
     const int L = A.lmax;
@@ -196,6 +193,29 @@ __global__ void __launch_bounds__(SP_T) spin_synth_kernel(SpinArgs A)
     }
 }
 
+template <int NM>
+__global__ void __launch_bounds__(SP_T) spin_synth_kernel(SpinArgs A)
+{
+    __shared__ double4 s_t[SP_CH];
+    __shared__ double2 s_e[NM][SP_CH], s_b[NM][SP_CH];
+    spin_synth_body<NM>(A, blockIdx.x / A.nblk, blockIdx.x % A.nblk, s_t, s_e, s_b);
+}
+
+// the maps whose columns the tensor-core kernels left (fix[m][2 g], fix[m][2 g + 1]; see legendre.cu)
+__global__ void __launch_bounds__(SP_T) spin_synth_fix_kernel(SpinArgs A, const int *__restrict__ fix, int nmaps)
+{
+    __shared__ double4 s_t[SP_CH];
+    __shared__ double2 s_e[1][SP_CH], s_b[1][SP_CH];
+    const int m = blockIdx.x;
+    for (int g = 0; g < nmaps; ++g) {
+        if (!fix[m * 16 + 2 * g] && !fix[m * 16 + 2 * g + 1]) continue;
+        SpinArgs B = A;
+        B.alm += (int64_t)g * 2 * A.nalm;
+        B.delta += (int64_t)g * 2 * A.nrings * (A.mmax + 1);
+        for (int blk = 0; blk < A.nblk; ++blk) spin_synth_body<1>(B, m, blk, s_t, s_e, s_b);
+    }
+}
+
 // afterwards every lane holds the warp total of value (lane & 7)
 __device__ __forceinline__ double reduce_scatter8(double v[SP_RED])
 {
@@ -218,15 +238,13 @@ __device__ __forceinline__ double reduce_scatter8(double v[SP_RED])
 
 // Analysis: one CTA per (m, 128 slots), NM maps.  Per l, every thread forms the four products of
 // its slot, the warps reduce-scatter them over their 32 slots, and the CTA adds its warps and
-// writes the block's partial E_lm, B_lm (coefficient -+c/2 applied), [blk][map][E|B][nalm].
+// writes the block's partial E_lm, B_lm (coefficient -+c/2 applied) to planes of `plane` values, E and B
+// of map g at 2 g and 2 g + 1.
 template <int NM>
-__global__ void __launch_bounds__(SP_T) spin_anal_kernel(SpinArgs A)
+__device__ __forceinline__ void spin_anal_body(const SpinArgs &A, int m, int blk, double2 *part, int64_t plane,
+                                               double4 *s_t, double (*s_red)[SP_CH][4 * NM])
 {
     constexpr int NW = SP_T / 32;
-    __shared__ double4 s_t[SP_CH];
-    __shared__ double s_red[NW][SP_CH][4 * NM];
-    const int m = blockIdx.x / A.nblk;
-    const int blk = blockIdx.x - m * A.nblk;
     const int slot = blk * SP_T + threadIdx.x;
     const bool active = slot < A.nslots;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -234,13 +252,12 @@ __global__ void __launch_bounds__(SP_T) spin_anal_kernel(SpinArgs A)
     const int l0 = max(m, 2);
     const int64_t base = (int64_t)m * (2 * L + 3 - m) / 2;
     const int64_t mstride = A.mmax + 1;
-    double2 *part = A.partial + (int64_t)blk * A.nmaps * 2 * A.nalm;
 
     // l < l0: no spin-2 function
     for (int l = m + threadIdx.x; l < min(l0, L + 1); l += SP_T)
         for (int g = 0; g < A.nmaps; ++g) {
-            part[(int64_t)(2 * g) * A.nalm + base + (l - m)] = make_double2(0.0, 0.0);
-            part[(int64_t)(2 * g + 1) * A.nalm + base + (l - m)] = make_double2(0.0, 0.0);
+            part[(2 * g) * plane + base + (l - m)] = make_double2(0.0, 0.0);
+            part[(2 * g + 1) * plane + base + (l - m)] = make_double2(0.0, 0.0);
         }
     if (l0 > L) return;
 
@@ -333,8 +350,46 @@ __global__ void __launch_bounds__(SP_T) spin_anal_kernel(SpinArgs A)
             const double hc = 0.5 * s_t[j].w;
             const int64_t ix = base + (c0 - m) + j;
             if (!SHT_CHK(ix < A.nalm)) continue;
-            part[(int64_t)(2 * g) * A.nalm + ix] = make_double2(-hc * t[0], -hc * t[1]);
-            part[(int64_t)(2 * g + 1) * A.nalm + ix] = make_double2(hc * t[2], hc * t[3]);
+            part[(2 * g) * plane + ix] = make_double2(-hc * t[0], -hc * t[1]);
+            part[(2 * g + 1) * plane + ix] = make_double2(hc * t[2], hc * t[3]);
+        }
+    }
+}
+
+template <int NM>
+__global__ void __launch_bounds__(SP_T) spin_anal_kernel(SpinArgs A)
+{
+    __shared__ double4 s_t[SP_CH];
+    __shared__ double s_red[SP_T / 32][SP_CH][4 * NM];
+    const int m = blockIdx.x / A.nblk, blk = blockIdx.x % A.nblk;
+    spin_anal_body<NM>(A, m, blk, A.partial + (int64_t)blk * A.nmaps * 2 * A.nalm, A.nalm, s_t, s_red);
+}
+
+// the maps whose columns the tensor-core kernels left: E and B of one map at a time, block after block
+// into one pair of planes of A.partial (indices from idx0 on), added up in `alm`
+__global__ void __launch_bounds__(SP_T) spin_anal_fix_kernel(SpinArgs A, const int *__restrict__ fix, int nmaps, int m0,
+                                                             int64_t idx0, int64_t nalm_part, double2 *__restrict__ alm)
+{
+    __shared__ double4 s_t[SP_CH];
+    __shared__ double s_red[SP_T / 32][SP_CH][4];
+    const int m = m0 + blockIdx.x;
+    const int64_t base = (int64_t)m * (2 * A.lmax + 3 - m) / 2;
+    for (int g = 0; g < nmaps; ++g) {
+        if (!fix[m * 16 + 2 * g] && !fix[m * 16 + 2 * g + 1]) continue;
+        SpinArgs B = A;
+        B.delta += (int64_t)g * 2 * A.nrings * (A.mmax + 1);
+        B.nmaps = 1;
+        double2 *part = A.partial - idx0, *out = alm + (int64_t)g * 2 * A.nalm;
+        for (int blk = 0; blk < A.nblk; ++blk) {
+            spin_anal_body<1>(B, m, blk, part, nalm_part, s_t, s_red);
+            __syncthreads();
+            for (int i = threadIdx.x; i <= A.lmax - m; i += SP_T)
+                for (int h = 0; h < 2; ++h) {
+                    const double2 v = part[h * nalm_part + base + i], o = out[h * A.nalm + base + i];
+                    const double2 s = blk ? make_double2(v.x + o.x, v.y + o.y) : v;
+                    out[h * A.nalm + base + i] = make_double2(s.x, m == 0 ? 0.0 : s.y);
+                }
+            __syncthreads();
         }
     }
 }
@@ -500,6 +555,27 @@ cudaError_t launch_spin_anal(const Plan &p, const double2 *delta, double2 *alm, 
         g0 += nm;
     }
     return cudaSuccess;
+}
+
+cudaError_t launch_spin_synth_fix(const Plan &p, const double2 *alm, double2 *delta, const int *fix, int nmaps,
+                                  cudaStream_t st)
+{
+    SpinArgs A = spin_args(p);
+    A.alm = alm;
+    A.delta = delta;
+    A.nmaps = 1;
+    spin_synth_fix_kernel<<<(unsigned)(p.mmax + 1), SP_T, 0, st>>>(A, fix, nmaps);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_spin_anal_fix(const Plan &p, const double2 *delta, double2 *alm, double2 *partial, const int *fix,
+                                 int nmaps, int m0, int m1, int64_t idx0, int64_t nalm_part, cudaStream_t st)
+{
+    SpinArgs A = spin_args(p);
+    A.delta = const_cast<double2 *>(delta);
+    A.partial = partial;
+    spin_anal_fix_kernel<<<(unsigned)(m1 - m0), SP_T, 0, st>>>(A, fix, nmaps, m0, idx0, nalm_part, alm);
+    return cudaGetLastError();
 }
 
 namespace {

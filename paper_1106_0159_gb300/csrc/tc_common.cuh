@@ -202,6 +202,9 @@ struct TcArgs {
     const double *u, *s;
     const double *alpha, *cfac;
     const double3 *rein;     // Reinsch coefficients for m <= mR (polar blocks)
+    const double4 *tab;      // spin: (alpha, alpha (1 + g), alpha (1 - g), c) per (l, m)
+    const double *start;     // spin: [mmax+1] start coefficients S_m
+    int sig;                 // spin: this pass's sign, +1 or -1
     const int *mflag;        // [mmax+1] 1 for the m this plan computes (null: all)
     const int *Ey;           // [mmax+1][nblk] scale exponent of y per slot block
     const int *first;        // [mmax+1][nblk] first chunk with a kept y value (nch: none)
@@ -227,18 +230,33 @@ __device__ __forceinline__ bool polar_block(const TcArgs &A, int m, int blk)
     return m <= A.mR && A.s[blk * TC_T] < POLAR_SIN;
 }
 
-// Recurrence coefficients of one l (the lane's own): (alpha, -, -, -) or Reinsch (beta, rho, b0, 1 / c);
-// all zero above lmax.
+// The recurrence of a block: the y form, Reinsch's form (polar blocks), or one sign of the spin-2 pair
+// (spin.cu: y_l = alpha_l (x + sig g) y_{l-1} - y_{l-2} from l = max(m, 2) on).
+enum : int { REC_Y = 0, REC_REIN = 1, REC_SPIN = 2 };
+
+// first l of the recurrence: its chunks of 32 start here
+template <int KIND>
+__device__ __forceinline__ int first_l(int m)
+{
+    return KIND == REC_SPIN ? max(m, 2) : m;
+}
+
+// Recurrence coefficients of one l (the lane's own): (alpha, -, -, -), Reinsch (beta, rho, b0, 1 / c) or
+// spin (alpha, alpha (1 + sig g), -, -); all zero above lmax.
 struct RecCoef {
     double a, rh, b0, ci;
 };
-template <bool REIN>
+template <int KIND>
 __device__ __forceinline__ RecCoef load_coef(const TcArgs &A, int64_t base, int m, int l)
 {
     RecCoef c{0.0, 0.0, 0.0, 0.0};
     if (l <= A.lmax) {
         const int64_t ix = base + (l - m);
-        if (REIN) {
+        if (KIND == REC_SPIN) {
+            const double4 t = A.tab[ix];
+            c.a = t.x;
+            c.rh = A.sig > 0 ? t.y : t.z;
+        } else if (KIND == REC_REIN) {
             const double3 t = A.rein[ix];
             c = RecCoef{t.x, t.y, t.z, 1.0 / A.cfac[ix]};
         } else {
@@ -281,11 +299,12 @@ __device__ __forceinline__ int y_row(int j)
     return PAR ? (j & 1) * (TC_CH / 2) + (j >> 1) : j;
 }
 
-template <bool REIN, bool PAR, int YS, int G>
+template <int KIND, bool PAR, int YS, int G>
 __device__ __forceinline__ void recurrence_warps(const TcArgs &A, int m, int blk, int r, bool active, int64_t base,
                                                  int nch, int cfirst, double *ybuf, double *abuf)
 {
-    const int lane = r & 31;
+    constexpr bool REIN = KIND == REC_REIN, SPIN = KIND == REC_SPIN;
+    const int lane = r & 31, lb = first_l<KIND>(m);
     double u = 0.0, y1 = 0.0, y2 = 0.0;
     int k = 0;
     if (active) {
@@ -297,10 +316,10 @@ __device__ __forceinline__ void recurrence_warps(const TcArgs &A, int m, int blk
         k = A.ck_k[ci];
     }
     abuf += (r >> 5) * TC_CH;
-    RecCoef cur = load_coef<REIN>(A, base, m, m + TC_CH * cfirst + lane);
+    RecCoef cur = load_coef<KIND>(A, base, m, lb + TC_CH * cfirst + lane);
     int c = cfirst;
     for (; c < nch && (REIN || __any_sync(0xffffffffu, k < 0)); ++c) {
-        const RecCoef nxt = load_coef<REIN>(A, base, m, m + TC_CH * (c + 1) + lane);
+        const RecCoef nxt = load_coef<KIND>(A, base, m, lb + TC_CH * (c + 1) + lane);
         const int q = c - cfirst;
         double *yb = ybuf + (size_t)(q & 1) * TC_CH * YS + r;
         if (q >= 2) bar_sync(BAR_EMPTY + (q & 1), TC_NT);  // the split warps read chunk q - 2
@@ -321,7 +340,7 @@ __device__ __forceinline__ void recurrence_warps(const TcArgs &A, int m, int blk
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const double a = __shfl_sync(0xffffffffu, cur.a, j0 + j);
-                    f[j] = fma(-a, u, a);
+                    f[j] = fma(-a, u, SPIN ? __shfl_sync(0xffffffffu, cur.rh, j0 + j) : a);
                 }
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -344,35 +363,63 @@ __device__ __forceinline__ void recurrence_warps(const TcArgs &A, int m, int blk
         cur = nxt;
     }
     if (REIN || c >= nch) return;
-    double ax[G], al[G], pv[G];  // factors of this group, coefficients of the next, values of the previous
-    abuf[lane] = cur.a;
+    // factors of this group, coefficients of the next (spin: a second one), values of the previous
+    double ax[G], al[G], al1[SPIN ? G : 1], pv[G];
+    double2 *abuf2 = reinterpret_cast<double2 *>(abuf);  // spin: 16 steps of coefficient pairs
+    if (SPIN) {
+        if (lane < 16) abuf2[lane] = make_double2(cur.a, cur.rh);
+    } else {
+        abuf[lane] = cur.a;
+    }
     __syncwarp();
 #pragma unroll
     for (int j = 0; j < G; ++j) {
-        const double a = abuf[j];
-        ax[j] = fma(-a, u, a);
-        al[j] = abuf[G + j];
+        if (SPIN) {
+            const double2 t = abuf2[j], w = abuf2[G + j];
+            ax[j] = fma(-t.x, u, t.y);
+            al[j] = w.x;
+            al1[SPIN ? j : 0] = w.y;
+        } else {
+            const double a = abuf[j];
+            ax[j] = fma(-a, u, a);
+            al[j] = abuf[G + j];
+        }
         pv[j] = 0.0;
     }
     double *pp = ybuf + r;  // where the previous group goes
     for (const int c0 = c; c < nch; ++c) {
-        const RecCoef nxt = load_coef<REIN>(A, base, m, m + TC_CH * (c + 1) + lane);
+        const RecCoef nxt = load_coef<KIND>(A, base, m, lb + TC_CH * (c + 1) + lane);
         const int q = c - cfirst;
         double *yb = ybuf + (size_t)(q & 1) * TC_CH * YS + r;
 #pragma unroll
         for (int j0 = 0; j0 < TC_CH; j0 += G) {
-            if (j0 == TC_CH - 2 * G) {  // the next chunk's coefficients replace this one's, which are all read
+            // coefficients that are all read make room for the next ones: a chunk's 32, or (spin) 16 pairs
+            if (SPIN && ((j0 + 2 * G) & 15) == 0) {
+                const bool up = j0 + 2 * G < TC_CH;  // steps 16-31 of this chunk, else 0-15 of the next
+                __syncwarp();
+                if ((lane >= 16) == up) abuf2[lane & 15] = up ? make_double2(cur.a, cur.rh) : make_double2(nxt.a, nxt.rh);
+                __syncwarp();
+            } else if (!SPIN && j0 == TC_CH - 2 * G) {
                 __syncwarp();
                 abuf[lane] = nxt.a;
                 __syncwarp();
             }
-            double yv[G], axn[G], aln[G];
-            const double2 *as = reinterpret_cast<const double2 *>(abuf + ((j0 + 2 * G) & 31));
+            double yv[G], axn[G], aln[G], al1n[SPIN ? G : 1];
+            if (SPIN) {
 #pragma unroll
-            for (int j = 0; j < G / 2; ++j) {
-                const double2 t = as[j];
-                aln[2 * j] = t.x;
-                aln[2 * j + 1] = t.y;
+                for (int j = 0; j < G; ++j) {
+                    const double2 t = abuf2[((j0 + 2 * G) & 15) + j];
+                    aln[j] = t.x;
+                    al1n[SPIN ? j : 0] = t.y;
+                }
+            } else {
+                const double2 *as = reinterpret_cast<const double2 *>(abuf + ((j0 + 2 * G) & 31));
+#pragma unroll
+                for (int j = 0; j < G / 2; ++j) {
+                    const double2 t = as[j];
+                    aln[2 * j] = t.x;
+                    aln[2 * j + 1] = t.y;
+                }
             }
             const bool store = j0 > 0 || c > c0;
 #pragma unroll
@@ -381,7 +428,7 @@ __device__ __forceinline__ void recurrence_warps(const TcArgs &A, int m, int blk
                 y2 = y1;
                 y1 = y;
                 yv[j] = y;
-                axn[j] = fma(-al[j], u, al[j]);
+                axn[j] = fma(-al[j], u, SPIN ? al1[SPIN ? j : 0] : al[j]);
                 if (store) pp[y_row<PAR>(((j0 - G) & 31) + j) * YS] = pv[j];  // steps j0 - G .. j0 - 1
             }
             if (j0 == 0) {
@@ -393,9 +440,11 @@ __device__ __forceinline__ void recurrence_warps(const TcArgs &A, int m, int blk
             for (int j = 0; j < G; ++j) {
                 ax[j] = axn[j];
                 al[j] = aln[j];
+                if (SPIN) al1[SPIN ? j : 0] = al1n[SPIN ? j : 0];
                 pv[j] = yv[j];
             }
         }
+        cur = nxt;
     }
 #pragma unroll
     for (int j = 0; j < G; ++j) pp[y_row<PAR>(TC_CH - G + j) * YS] = pv[j];
