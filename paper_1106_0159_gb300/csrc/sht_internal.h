@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <functional>
 #include <string>
 #include <vector>
 
@@ -20,6 +21,10 @@ cudaError_t dev_malloc(T **ptr, size_t bytes)
 {
     return dev_malloc((void **)ptr, bytes);
 }
+
+// Runs f(0) .. f(n - 1) on the host's cores (at most 16 threads, fewer when they cannot be had); the
+// plan tables of each m are independent.  f must not throw.
+void host_parallel(int n, const std::function<void(int)> &f);
 
 // One complex FFT of length n on the ring stage: ring ringA rides on the real
 // part and ringB (or -1) on the imaginary part (two real rings per complex

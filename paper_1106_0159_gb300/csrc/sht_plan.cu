@@ -11,6 +11,7 @@
 #include <cstring>
 #include <new>
 #include <numeric>
+#include <thread>
 
 namespace sht {
 
@@ -28,6 +29,22 @@ cudaError_t dev_malloc(void **ptr, size_t bytes)
         if (g_alloc_budget.compare_exchange_weak(b, b - 1)) break;
     }
     return cudaMalloc(ptr, bytes);
+}
+
+void host_parallel(int n, const std::function<void(int)> &f)
+{
+    std::atomic<int> next{0};
+    auto work = [&] {
+        for (int i = next++; i < n; i = next++) f(i);
+    };
+    std::vector<std::thread> pool;
+    const int want = std::min({16, n / 64, (int)std::thread::hardware_concurrency()}) - 1;
+    try {
+        for (int t = 0; t < want; ++t) pool.emplace_back(work);
+    } catch (...) {  // no more threads: those that run and this one do the rest
+    }
+    work();
+    for (auto &t : pool) t.join();
 }
 
 static cudaEvent_t pool_event(const Plan &p)
@@ -204,10 +221,12 @@ void recurrence_tables(int lmax, int mmax, std::vector<double> &alpha, std::vect
     long double mu2 = 1.0L / (4.0L * 3.14159265358979323846264338327950288L);  // mu_0^2
     for (int m = 0; m <= mmax; ++m) {
         if (m > 0) mu2 *= (long double)(2 * m + 1) / (long double)(2 * m);  // eq. (pmm)
+        alpha[sht_alm_index(lmax, m, m)] = (double)std::sqrt(mu2);
+    }
+    sht::host_parallel(mmax + 1, [&](int m) {
         const int64_t base = sht_alm_index(lmax, m, m);
-        alpha[base] = (double)std::sqrt(mu2);
         cfac[base] = 1.0;
-        if (m + 1 > lmax) continue;
+        if (m + 1 > lmax) return;
         alpha[base + 1] = std::sqrt(2.0 * m + 3.0);
         cfac[base + 1] = 1.0;
         double c2 = 1.0, c1 = 1.0;            // c_{l-2}, c_{l-1}
@@ -223,7 +242,7 @@ void recurrence_tables(int lmax, int mmax, std::vector<double> &alpha, std::vect
             c1 = c;
             bprev = b;
         }
-    }
+    });
 }
 
 // Reinsch-form tables for polar slots, m <= mR: (beta_l, rho_l, b0_l) with
@@ -239,10 +258,10 @@ void reinsch_tables(int lmax, int mR, std::vector<double3> &rein)
     }
     const int64_t n = sht_alm_index(lmax, lmax, mR) + 1;
     rein.assign(n, make_double3(0.0, 0.0, 0.0));
-    for (int m = 0; m <= mR; ++m) {
+    sht::host_parallel(mR + 1, [&](int m) {
         const int64_t base = sht_alm_index(lmax, m, m);
         rein[base] = make_double3(0.0, 0.0, 0.0);
-        if (m + 1 > lmax) continue;
+        if (m + 1 > lmax) return;
         const double b1 = std::sqrt(2.0 * m + 3.0);
         rein[base + 1] = make_double3(b1, -1.0, b1 - 1.0);
         const double m2 = (double)m * m, q = 4.0 * m2 - 1.0;
@@ -257,7 +276,7 @@ void reinsch_tables(int lmax, int mR, std::vector<double3> &rein)
             bprev = b;
             dprev = d;
         }
-    }
+    });
 }
 
 sht_status ensure_workspace(Plan &p, size_t need)

@@ -439,7 +439,7 @@ cudaError_t build_spin_tables(Plan &p)
     std::vector<double4> tab((size_t)p.nalm, make_double4(0.0, 0.0, 0.0, 0.0));
     std::vector<double> start((size_t)M + 1, 0.0);
     const long double PI_L = 3.14159265358979323846264338327950288L;
-    for (int m = 0; m <= M; ++m) {
+    host_parallel(M + 1, [&](int m) {
         const int l0 = std::max(m, 2);
         const int64_t base = (int64_t)m * (2 * L + 3 - m) / 2;
         // S_m: +2 lambda_{l0, m} = S_m sin(theta)^|m-2| sin(theta/2)^(2 min(m, 2))
@@ -454,7 +454,7 @@ cudaError_t build_spin_tables(Plan &p)
             start[m] = (double)(2.0L * sqrtl(30.0L / (96.0L * PI_L)));   // K_1 / 2, K_1 = 4 sqrt(30 / 96 pi)
         else
             start[m] = (double)(1.5L * sqrtl(20.0L / (96.0L * PI_L)));   // K_0 / 4, K_0 = 6 sqrt(20 / 96 pi)
-        if (l0 > L) continue;
+        if (l0 > L) return;
         const long double mm = (long double)m * m;
         long double c2 = 1.0L, c1 = 1.0L;  // c_{l-2}, c_{l-1}
         tab[base + (l0 - m)] = make_double4(0.0, 0.0, 0.0, 1.0);
@@ -477,7 +477,7 @@ cudaError_t build_spin_tables(Plan &p)
             c2 = c1;
             c1 = c;
         }
-    }
+    });
     double4 *dt = nullptr;
     double *ds = nullptr;
     cudaError_t e = sht::dev_malloc(&dt, sizeof(double4) * tab.size());
