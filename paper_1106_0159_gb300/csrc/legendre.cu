@@ -261,6 +261,7 @@ __global__ void __launch_bounds__(SYN_T) legendre_synth_kernel(SynArgs A)
 struct AnaArgs {
     const double2 *delta;  // [nmaps][nrings][mmax+1], first map of this launch
     double2 *partial;      // [nblk][nmaps_total][nalm]
+    double2 *alm;          // not null: the only block writes a_lm itself, [nmaps][nalm] (no reduction follows)
     const int *slotN, *slotS;
     const double *u, *s;
     const double *alpha, *cfac;
@@ -435,7 +436,11 @@ __device__ __forceinline__ void anal_body(const AnaArgs &A, int m, int blk, Coef
                 re /= c;
                 im /= c;
             }
-            if (SHT_CHK(ix >= 0 && ix < A.nalm && blk < A.nblk))
+            if (A.alm) {
+                const double c = A.cfac[ix];
+                if (SHT_CHK(ix >= 0 && ix < A.nalm))
+                    A.alm[(int64_t)g * A.nalm + ix] = make_double2(c * re, m == 0 ? 0.0 : c * im);
+            } else if (SHT_CHK(ix >= 0 && ix < A.nalm && blk < A.nblk))
                 A.partial[(int64_t)blk * A.part_blk_stride + (int64_t)g * A.part_map_stride + ix] = make_double2(re, im);
         }
     }
@@ -453,8 +458,11 @@ __global__ void __launch_bounds__(ANA_T) legendre_anal_kernel(AnaArgs A)
         const int64_t base = (int64_t)m * (2 * A.lmax + 3 - m) / 2;
         for (int i = threadIdx.x; i < (A.lmax - m + 1) * NM; i += ANA_T) {
             const int j = i % (A.lmax - m + 1), g = i / (A.lmax - m + 1);
-            A.partial[(int64_t)blk * A.part_blk_stride + (int64_t)g * A.part_map_stride + base + j] =
-                make_double2(0.0, 0.0);
+            if (A.alm)
+                A.alm[(int64_t)g * A.nalm + base + j] = make_double2(0.0, 0.0);
+            else
+                A.partial[(int64_t)blk * A.part_blk_stride + (int64_t)g * A.part_map_stride + base + j] =
+                    make_double2(0.0, 0.0);
         }
         return;
     }
@@ -705,12 +713,12 @@ int legendre_anal_nblk(const Plan &p)
     return (p.nslots + per - 1) / per;
 }
 
-cudaError_t launch_legendre_anal(const Plan &p, const double2 *delta, double2 *partial, int nmaps, cudaStream_t st,
-                                 int *nlaunch)
+cudaError_t launch_legendre_anal(const Plan &p, const double2 *delta, double2 *partial, double2 *alm, int nmaps,
+                                 cudaStream_t st, int *nlaunch)
 {
     *nlaunch = 0;
     const int per = anal_slots_per_cta(p);
-    AnaArgs A;
+    AnaArgs A{};
     A.slotN = p.d_slotN;
     A.slotS = p.d_slotS;
     A.u = p.d_u;
@@ -735,6 +743,9 @@ cudaError_t launch_legendre_anal(const Plan &p, const double2 *delta, double2 *p
         const int left = nmaps - g0;
         A.delta = delta + (int64_t)g0 * dstride;
         A.partial = partial + (int64_t)g0 * p.nalm;
+        // the reduction of one block is a launch of its own for nothing (HEALPix 32, lmax 64, one map:
+        // 6 of 51 us)
+        A.alm = A.nblk == 1 ? alm + (int64_t)g0 * p.nalm : nullptr;
         if (left >= 2 && p.tune[SHT_TUNE_ANAL_MAPS] >= 2) {
             if (per == 4 * ANA_T)
                 legendre_anal_kernel<2, 4><<<grid, ANA_T, 0, st>>>(A);

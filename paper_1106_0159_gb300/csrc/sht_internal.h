@@ -163,8 +163,8 @@ struct StageEvents {
 // launch helpers (legendre.cu, ringfft.cu); return cudaGetLastError(), count launches in *nlaunch
 cudaError_t launch_legendre_synth(const Plan &p, const double2 *alm, double2 *delta, int nmaps, cudaStream_t st,
                                   int *nlaunch);
-cudaError_t launch_legendre_anal(const Plan &p, const double2 *delta, double2 *partial, int nmaps, cudaStream_t st,
-                                 int *nlaunch);
+cudaError_t launch_legendre_anal(const Plan &p, const double2 *delta, double2 *partial, double2 *alm, int nmaps,
+                                 cudaStream_t st, int *nlaunch);  // alm: written when one block holds every slot
 cudaError_t launch_block_reduce(const Plan &p, const double2 *partial, double2 *alm, int nmaps, cudaStream_t st);
 int legendre_anal_nblk(const Plan &p);
 int legendre_anal_default_slots(const Plan &p);  // default SHT_TUNE_ANAL_SLOTS for the plan's slot count

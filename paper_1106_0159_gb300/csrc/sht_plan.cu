@@ -398,11 +398,12 @@ sht_status run_legendre_anal(Plan &p, const double2 *delta, double2 *alm, double
     {
         StageScope sc(p, 3, s);
         int n = 0;
-        cudaError_t e = sht::launch_legendre_anal(p, delta, partial, nmaps, s, &n);
+        cudaError_t e = sht::launch_legendre_anal(p, delta, partial, alm, nmaps, s, &n);
         p.launches[3] += n;
         if (e != cudaSuccess) return cuda_fail(p, e, "legendre_anal");
         sc.done();
     }
+    if (sht::legendre_anal_nblk(p) == 1) return SHT_OK;  // one block: the kernel wrote a_lm itself
     StageScope sc(p, 4, s);
     cudaError_t e = sht::launch_block_reduce(p, partial, alm, nmaps, s);
     p.launches[4] += 1;
