@@ -388,27 +388,9 @@ def ours_arm(a, rank, world, local_rank):
 
     S = sum(L - m + 1 for m in range(L + 1)) * plan.npairs  # (l, m, ring-pair) steps of one transform
 
-    def fp64_roofline(run, steps):
-        # dominant Legendre stage on the FP64 pipe: nominal 3 flops per step for each launch's
-        # recurrence plus 4 flops per step per map for the accumulation
-        legendre = {k: v for k, v in run["stages"].items() if k in ("legendre_synth", "legendre_anal")}
-        dom = max(legendre, key=lambda k: legendre[k][0])
-        dom_ms, dom_launches = legendre[dom]
-        flops = S * (3.0 * dom_launches + 4.0 * B * steps)
-        achieved = flops / (dom_ms * 1e-3) / 1e12
-        key = "legendre_anal_kernel" if dom == "legendre_anal" else "legendre_synth_kernel"
-        return {"bound": "alu", "pipe": "fp64", "kernel": key, "achieved": achieved, "peak": peak_tf,
-                "unit": "TFLOP/s", "frac": achieved / peak_tf, "traffic": traffic_from_profiles(key),
-                "peak_source": "derived: 2 FP64 FMA/clk/SM x %d SMs x %d MHz x 2 flop; in-run FMA probe %.3f "
-                               "TF/s" % (nsm, SM_MAX_MHZ, probe_tf),
-                "work": "7 flops per (l, m, ring-pair) step over the full triangle, per map (3 recurrence + 4 "
-                        "accumulate); steps whose lambda is below 2^-224 are skipped, so frac can exceed 1",
-                "time": "the Legendre stage (all its launches)",
-                "live_share": live_share, "frac_of_executed": achieved / peak_tf * live_share}
-
     # live share of the (l, m, ring-pair) steps: the precision-form tables mark the first 32-l chunk
-    # per (m, 128-slot block) above the dropping threshold; the plain kernels skip the same prefix
-    # per warp, so the nominal fractions below count about 1 / live more work than is executed
+    # per (m, 128-slot block) above the dropping threshold; the kernels start there, so the nominal
+    # fractions below count about 1 / live more work than is executed
     plan.set_mode(sht.MODE_SPLIT_BF16)
     live_steps, total_steps = plan.live_steps()
     live_share = live_steps / total_steps
@@ -427,43 +409,46 @@ def ours_arm(a, rank, world, local_rank):
                     "peak_source": "derived: 128 FP32 FMA/clk/SM x %d SMs x %d MHz x 2 flop" % (nsm, SM_MAX_MHZ),
                     "work": "30 FP32 flops per (l, m, ring-pair, map): two double-float real products and sums",
                     "time": "analysis stage (includes the polar kernel and the block reduction)"}
+        return tc_roofline(run, steps)
+
+    def tc_roofline(run, steps):
         # the tensor-core kernels, each timed alone by its own CUDA events on the call's stream
-        # (stage ids tc_synth_kernel / tc_anal_kernel: no polar kernel, no block reduction)
+        # (stage ids tc_synth_kernel / tc_anal_kernel: no digit split, no block reduction); both modes
+        # run them at this size
+        st = run["stages"]
         ka_ms, ka_n = st["tc_anal_kernel"]
         ks_ms, ks_n = st["tc_synth_kernel"]
         anal = ka_ms >= ks_ms
         ms, nl = (ka_ms, ka_n) if anal else (ks_ms, ks_n)
         key = "tc_anal_kernel" if anal else "tc_synth_kernel"
         groups = -(-B // 16) * steps            # passes of the recurrence: one per group of <= 16 maps
-        per_group_s = ms * 1e-3 / groups         # the analysis runs a group as about eight m-slab launches
+        per_group_s = ms * 1e-3 / groups         # a group is several m-slab launches
         maps_per_group = min(B, 16)
-        # binding pipe: the tensor cores.  Useful work = the 28 digit-pair slice-products, each the
-        # whole contraction of 4 flops per (l, m, ring-pair) step and map (complex x real), over the
-        # full triangle S
-        tflops = 28 * 4.0 * maps_per_group * S / per_group_s / 1e12
+        # binding pipe: the FP64 recurrence, two FMA-pipe instructions per (l, m, ring-pair) step, once
+        # per group
+        fflops = 4.0 * S / per_group_s / 1e12
+        # beside it the digit products: 36 of them, each the whole contraction of 4 flops per step and
+        # map (complex x real), over the full triangle S
+        tflops = 36 * 4.0 * maps_per_group * S / per_group_s / 1e12
         tpeak = MEASURED.get("bf16_tflops_sustained") or 1725.1
-        # the FP64 recurrence beside it: 3 flops per step, once per group
-        fflops = 3.0 * S / per_group_s / 1e12
         # algorithmic bytes per group: Delta read and a_lm written (analysis), a_lm read and
         # Delta written (synthesis)
         alg = maps_per_group * (plan.nrings * (L + 1) + nalm) * 16
         traffic = traffic_from_profiles(key)
-        return {"bound": "tensor", "kernel": key, "achieved": tflops, "peak": tpeak, "unit": "TFLOP/s",
-                "frac": tflops / tpeak, "traffic": traffic,
-                "peak_source": "measured bf16 GEMM, sustained (MEASURED_PEAKS.json bf16_tflops_sustained): the "
-                               "kernel is timed inside a long step",
-                "work": "28 bf16 digit-pair products x 4 flops per (l, m, ring-pair) step and map, nominal full "
-                        "triangle S = %d steps, %d maps per group: %.3e flops per group" %
-                        (S, maps_per_group, 28 * 4.0 * maps_per_group * S),
+        return {"bound": "alu", "pipe": "fp64", "kernel": key, "achieved": fflops, "peak": peak_tf, "unit": "TFLOP/s",
+                "frac": fflops / peak_tf, "traffic": traffic,
+                "peak_source": "derived: 2 FP64 FMA/clk/SM x %d SMs x %d MHz x 2 flop; in-run FMA probe %.3f "
+                               "TF/s" % (nsm, SM_MAX_MHZ, probe_tf),
+                "work": "2 FP64 FMA (4 flops) of the recurrence per (l, m, ring-pair) step, once per group of %d maps, "
+                        "nominal full triangle S = %d steps" % (maps_per_group, S),
                 "time": "the kernel's own launches (CUDA events around each launch on the call's stream): "
                         "%.2f ms per group of %d maps, %d launches in %d groups" %
                         (per_group_s * 1e3, maps_per_group, nl, groups),
                 "live_share": live_share,
-                "frac_of_executed": tflops / tpeak / live_share,
-                "fp64": {"achieved": fflops, "peak": peak_tf, "unit": "TFLOP/s", "frac": fflops / peak_tf,
-                         "work": "3 FP64 flops per (l, m, ring-pair) step of the recurrence, once per launch",
-                         "peak_source": "derived: 2 FP64 FMA/clk/SM x %d SMs x %d MHz x 2 flop; in-run FMA probe "
-                                        "%.3f TF/s" % (nsm, SM_MAX_MHZ, probe_tf)},
+                "frac_of_executed": fflops / peak_tf * live_share,
+                "tensor": {"achieved": tflops, "peak": tpeak, "unit": "TFLOP/s", "frac": tflops / tpeak,
+                           "work": "36 fp16 digit-pair products x 4 flops per step and map",
+                           "peak_source": "measured bf16 GEMM, sustained (MEASURED_PEAKS.json bf16_tflops_sustained)"},
                 "algorithmic_bytes": alg,
                 "traffic_over_algorithmic": (traffic / alg) if traffic else None}
 
@@ -476,7 +461,7 @@ def ours_arm(a, rank, world, local_rank):
     head = timed(a.mode, a.steps, a.warmup, True)
     total_ms, step_ms, stages, clk = head["total_ms"], head["step_ms"], head["stages"], head["clocks"]
     value = job_throughput(world, B * a.steps, total_ms)
-    roofline = split_roofline(head, a.steps) if a.mode == "split" else fp64_roofline(head, a.steps)
+    roofline = split_roofline(head, a.steps) if a.mode == "split" else tc_roofline(head, a.steps)
     launches = sum(v[1] for v in stages.values())
 
     plain = None
@@ -485,7 +470,7 @@ def ours_arm(a, rank, world, local_rank):
         plain = {"value": job_throughput(world, B * a.plain_steps, pr["total_ms"]), "unit": "maps/s",
                  "ms_per_step": pr["total_ms"] / a.plain_steps, "steps": a.plain_steps, "warmup": 1,
                  "stages_ms_per_step": {k: v[0] / a.plain_steps for k, v in pr["stages"].items()},
-                 "roofline": fp64_roofline(pr, a.plain_steps),
+                 "roofline": tc_roofline(pr, a.plain_steps),
                  "ring_stages": ring_stages(pr, a.plain_steps, False)}
         plan.set_mode(sht.MODE_SPLIT_BF16)
 
@@ -704,7 +689,7 @@ def c2_leg(a, rep, local_rank, nsm, peak_tf):
         n = reps + 1
 
         def roof(ms_total):
-            ach = 7.0 * S / (ms_total / n * 1e-3) / 1e12
+            ach = 4.0 * S / (ms_total / n * 1e-3) / 1e12
             return {"achieved": ach, "peak": peak_tf, "unit": "TFLOP/s", "frac": ach / peak_tf}
 
         r = {"npix": plan.npix, "nrings": plan.nrings, "alm2map_ms": t_syn, "map2alm_ms": t_ana,
@@ -713,7 +698,7 @@ def c2_leg(a, rep, local_rank, nsm, peak_tf):
                            "map2alm": {k: v[0] / n for k, v in st_ana.items() if v[1]}},
              "fp64_roofline": {"legendre_synth": roof(st_syn["legendre_synth"][0]),
                                "legendre_anal": roof(st_ana["legendre_anal"][0]),
-                               "work": "7 flops per (l, m, ring-pair) step, nominal full triangle S = %d" % S},
+                               "work": "2 FP64 FMA (4 flops) of the recurrence per (l, m, ring-pair) step, nominal full triangle S = %d" % S},
              "input": inp}
         if grid == sht.GRID_GAUSS_LEGENDRE:
             d = (back - alm).abs().max().item() / alm.abs().pow(2).mean().sqrt().item()

@@ -71,7 +71,8 @@ static const char *const kStageNames[SHT_NSTAGES] = {"sht legendre_synth", "sht 
 StageEvents::StageEvents(const Plan &pl, int st, cudaStream_t str) : p(pl), stage(st), s(str)
 {
     nvtxRangePushA(kStageNames[st]);
-    if (p.timing) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;  // events of a captured launch have no time
+    if (p.timing && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
         a = pool_event(p);
         b = pool_event(p);
         if (a && b) cudaEventRecord(a, s);
