@@ -79,21 +79,25 @@ sht_status sht_plan_create(sht_plan_t *out, sht_grid grid, int nrings,
 
 /*
  * Arithmetic of the transforms:
- *   SHT_MODE_FP64        (default) every step in FP64.
- *   SHT_MODE_SPLIT_BF16  the precision form.  The lambda recurrence stays in FP64.  The sums of
- *                        eq. (matrix_vec) run on the tensor cores: the sum over l of the synthesis
- *                        and the sum over rings of the analysis, both operands cut into seven
- *                        balanced 7-bit digits, digit products accumulated in FP32 and combined in
- *                        FP64 or double-float.  The ring DFTs run in double-float on the FP32 pipe.
+ *   SHT_MODE_FP64        (default) every step to FP64 rounding.  From lmax 192 on the sums of
+ *                        eq. (matrix_vec), over l in the synthesis and over rings in the analysis,
+ *                        run on the tensor cores: both operands are cut into eight balanced base-256
+ *                        digits (62 bits) in fp16, digit products are summed exactly, as integers,
+ *                        and rounded once to FP64.  Values that digits cannot carry (not finite,
+ *                        near the ends of the exponent range) send their columns to FP64 sums.  A
+ *                        map's result does not depend on the maps beside it.  Processes up to 16
+ *                        maps per pass over the recurrence.
+ *   SHT_MODE_SPLIT_BF16  the precision form: the same Legendre steps whatever lmax, and the ring
+ *                        DFTs in double-float on the FP32 pipe.
  *                        SHT_TUNE_PREC_ANAL and SHT_TUNE_PREC_RING select other kernels.  Relative
- *                        error against the exact transform <= 1e-9 of the output RMS.  Processes up
- *                        to 16 maps per pass over the recurrence.  Only the first 256 ring slots
+ *                        error against the exact transform <= 1e-9 of the output RMS.  Only the
+ *                        first 256 ring slots
  *                        (after north/south pairing, ordered from the poles) may lie within
  *                        sin(theta) < 0.03 of a pole; a grid with more polar slots (HEALPix
  *                        Nside >~ 7000) returns SHT_EUNSUPPORTED and stays in its old mode.
- * Switching to SHT_MODE_SPLIT_BF16 the first time runs one FP64 pass of the recurrence to
- * measure the scale of its values per (m, block of 128 ring slots) (synchronous; about the cost
- * of one single-map synthesis).  SHT_EINVAL for an unknown mode.
+ * The creation of a plan with lmax >= 192, or else the first switch to SHT_MODE_SPLIT_BF16, runs
+ * one FP64 pass of the recurrence to measure the scale of its values per (m, block of 128 ring
+ * slots) (synchronous; about the cost of one single-map synthesis).  SHT_EINVAL for an unknown mode.
  */
 typedef enum { SHT_MODE_FP64 = 0, SHT_MODE_SPLIT_BF16 = 1 } sht_mode;
 sht_status sht_plan_set_mode(sht_plan_t plan, int mode);
@@ -127,7 +131,7 @@ sht_status sht_plan_set_mlist(sht_plan_t plan, const int *ms, int n);
  * Work accounting (host call, synchronous): the (l, m, ring-slot) recurrence steps of one pass,
  * *total = nalm * slots, and *live, those from the first 32-l chunk of each (m, block of 128
  * slots) in which some lambda is above the 2^-256 dropping threshold of the rescaling scheme
- * (steps before it contribute exactly zero and the precision-form kernels skip their sums).
+ * (steps before it contribute exactly zero and the tensor-core kernels skip them).
  * Needs the tables made by the first switch to SHT_MODE_SPLIT_BF16; SHT_EINVAL before that.
  */
 sht_status sht_plan_live_steps(sht_plan_t plan, int64_t *live, int64_t *total);
@@ -185,10 +189,12 @@ sht_status sht_map2alm_ws(sht_plan_t plan, const double *map, void *alm, int nma
  *   analysis   E_lm = -(2a_lm + 2a'_lm)/2, B_lm = i (2a_lm - 2a'_lm)/2 with
  *              2a_lm = sum_r w_r sum_j (Q + iU) conj(2Y_lm), 2a'_lm = sum_r w_r sum_j (Q - iU) conj((-2)Y_lm).
  * Layouts: alm complex128 [nmaps][2][nalm] (E then B, m-major triangle as above); map double
- * [nmaps][2][npix] (Q then U).  Arithmetic is FP64 for the Legendre step whatever the plan's mode
- * (the ring DFTs follow the mode, as in the scalar transforms); no Reinsch form on polar rings.
+ * [nmaps][2][npix] (Q then U).  Arithmetic is that of SHT_MODE_FP64 for the Legendre step whatever
+ * the plan's mode (the ring DFTs follow the mode, as in the scalar transforms), on the tensor cores
+ * from lmax 192 on; no Reinsch form on polar rings.
  * The first spin call on a plan builds its spin recurrence tables on the host and copies them to
- * the device (synchronous; 32 nalm bytes): make it before any stream capture.  Scratch grows on
+ * the device (synchronous; 32 nalm bytes, from lmax 192 on with the tables of the tensor-core
+ * kernels): make it before any stream capture.  Scratch grows on
  * demand to sht_spin_workspace_bytes(plan, nmaps).  Stream ordering and errors as sht_alm2map.
  */
 sht_status sht_alm2map_spin(sht_plan_t plan, int spin, const void *alm, double *map, int nmaps, void *stream);
@@ -225,8 +231,9 @@ sht_status sht_plan_reserve(sht_plan_t plan, int nmaps);
  * design.  Each knob bounds how many maps, or ring slots per thread, one
  * kernel launch takes.  Synthesis results are identical for every setting,
  * and the precision-form analysis is too (each map's sums keep their order).
- * The FP64 analysis order of the ring sums changes with the slots per thread,
- * so its results change within rounding.  The defaults are the settings
+ * The order of the ring sums in the plain FP64 analysis changes with the slots
+ * per thread, so its results change within rounding; knobs 0 to 2 have no effect
+ * where the tensor-core kernels run (lmax >= 192).  The defaults are the settings
  * measured best on GB300 at lmax = 4096.  The scratch a call needs follows the
  * setting (sht_workspace_bytes); after a change, call sht_plan_reserve again
  * if calls must not allocate.  Host calls; SHT_EINVAL for a null plan, an
@@ -264,7 +271,8 @@ int sht_plan_tuning(sht_plan_t plan, int knob); /* the knob's value; -1 for a nu
  * ring scratch and queue counters (allocated at creation, and again when a knob changes).
  * sht_batch_run enqueues only stream work on `stream` (a memset of the counters and the
  * launches), so it can be captured in a CUDA graph.  Results equal the one-plan calls bit for bit
- * (same kernels, same summation order), whatever the knobs.
+ * (same kernels, same summation order), whatever the knobs.  The Legendre steps of plans with
+ * lmax >= 192 are launched one plan after another on the tensor-core kernels, beside the queue.
  */
 typedef struct sht_batch_s *sht_batch_t;
 typedef enum {
@@ -300,11 +308,11 @@ sht_status sht_geom_gauss_legendre(int nrings, int64_t nphi, int64_t *nphi_out, 
  * enabled, every stage of every transform call is bracketed by CUDA events
  * recorded on the call's stream.  Stage ids (SHT_NSTAGES of them): 0 Legendre
  * synthesis, 1 ring synthesis, 2 ring analysis, 3 Legendre analysis, 4 ring-block
- * reduction of the FP64 analysis; 5 and 6 time one kernel alone, the main
- * tensor-core kernel of the precision-form synthesis (inside stage 0) and of the
- * precision-form analysis (inside stage 3), so that a roofline can divide by that
+ * reduction of the plain FP64 analysis (none with one block); 5 and 6 time one
+ * kernel alone, the main tensor-core kernel of the synthesis (inside stage 0) and
+ * of the analysis (inside stage 3), so that a roofline can divide by that
  * kernel's own time.  sht_plan_stage_times waits for the recorded events, adds
- * their durations to the running totals, and writes the totals
+ * their durations to the running totals (a captured launch has none), and writes the totals
  * (ms[SHT_NSTAGES], launches[SHT_NSTAGES]); reset != 0 zeroes the totals afterwards.
  */
 enum {
@@ -332,10 +340,12 @@ sht_status sht_fp64_fma_tflops(double *tflops);
  * counterpart; this is a library service).  Same arguments, layouts, stream
  * ordering and arithmetic as sht_alm2map (the plan's mode: the FP64 path, or
  * the precision form's kernels on a SHT_MODE_SPLIT_BF16 plan), but the call
- * allocates nothing: its scratch (the Delta intermediate, then either the
- * precision form's digit tiles or the ring-FFT buffers) is a 64 MiB static
- * device array, sht_noalloc_scratch_bytes(), that every GPU loading this
- * library holds until the process exits.  Calls whose scratch
+ * allocates nothing: its scratch (the Delta intermediate, then either digit
+ * tiles or the ring-FFT buffers) is a 64 MiB static device array,
+ * sht_noalloc_scratch_bytes(), that every GPU loading this library holds until
+ * the process exits.  The tensor-core kernels of an FP64 plan take the room
+ * that is left for their digit tiles, in slabs of whole m, and leave the call
+ * to the plain FP64 kernels when not one m fits.  Calls whose scratch
  * (16 nmaps nrings (mmax+1) bytes, rounded up to 256, plus the larger of one
  * ring-FFT buffer of 48 * max ring length bytes and, in the precision form,
  * the digit tiles of c_lm a_lm) exceeds it return SHT_EINVAL with the sizes

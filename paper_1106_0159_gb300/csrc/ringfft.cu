@@ -1024,8 +1024,8 @@ __global__ void phase_table_kernel(const double *phi0, int nrings, int mmax, dou
 
 // Whether a prime p runs as a direct radix: about p + 7 real operations per point and part against
 // Bluestein's two power-of-two transforms of length M >= 2 p - 1 (3.5 per point and factor of two) with
-// its chirps and filter.  Holds for every p <= 127 and, where 2 p - 1 lies just above a power of two
-// (so that M is nearly 4 p), up to about 280.
+// its chirps and filter.  Holds for every p <= 113 and, where 2 p - 1 lies above a power of two (so
+// that M is nearly 4 p), for 131 <= p <= 181 and 257 <= p <= 271.
 bool direct_radix(int p)
 {
     if (p > 1021) return false;
@@ -1161,7 +1161,9 @@ bool ring_df(const Plan &p) { return p.mode == SHT_MODE_SPLIT_BF16 && p.tune[SHT
 // Shared-memory DFTs: always with knob value 1; with the default 2 for the FP64 DFTs only.  The
 // double-float DFTs are bound by the latency of their FP32 arithmetic, not by the scratch traffic, and
 // ran faster through the global scratch at two CTAs per SM than in shared memory at one (lmax 4096,
-// HEALPix 2048, 16 maps: 45 / 38 ms against 54 / 43 ms for synthesis / analysis).
+// HEALPix 2048, 16 maps: 31.1 / 28.0 ms against 35.4 / 31.1 ms for synthesis / analysis; HEALPix 338, 5
+// maps: 365 / 343 us against 413 / 372).  FP64, global against shared: 810 / 791 us against 748 / 722 at
+// HEALPix 338, 633 / 617 against 629 / 614 at 512 (2 maps), 80.7 / 78.8 ms against 82.6 / 79.6 at 2048.
 bool ring_sm(const Plan &p)
 {
     const int k = p.tune[SHT_TUNE_RING_SMEM];

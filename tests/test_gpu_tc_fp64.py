@@ -160,7 +160,7 @@ def test_spin_transforms_against_oracle(n, L, M, nmaps):
         assert np.array_equal(t[1:], s[1:]) and np.isnan(t[0]).any()
 
 
-# rings of direct prime radices (7 .. 127 and, above, those cheaper than Bluestein's form), of Bluestein
+# rings of direct prime radices (7 .. 113 and, above, those cheaper than Bluestein's form), of Bluestein
 # primes, products, squares, and lengths shorter than the threads that share their folding
 @pytest.mark.parametrize("smem", [1, 0])
 @pytest.mark.parametrize("mode", [0, 1])
