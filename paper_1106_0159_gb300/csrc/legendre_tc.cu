@@ -60,18 +60,28 @@ struct TcTile {
     static constexpr int B_TILE = N2 * 16 * 2;                // bytes of one [N2 x 16] stack
     static constexpr int NSTK = TC_S / 2;                     // stacks per parity
     // accumulator blocks per parity: classes 0 .. 7, and where there is room one that takes the second
-    // halves of the class-7 stacks (incomplete, not read); at N = 32 those MMAs take half a stack
-    static constexpr int NCLS = N == 32 ? TC_S : TC_S + 1;
+    // halves of the class-7 stacks (incomplete, not read); else those MMAs take half a stack
+    static constexpr int NCLS = N == 8 ? TC_S + 1 : TC_S;
+    // Up to 8 maps two CTAs share an SM, each with one stage of y values and tiles: while one waits for
+    // its stage or for tensor memory the other's recurrence has the FP64 pipe, and where both run the
+    // pipe is never short of a warp.  16 maps take all of tensor memory: one CTA, two stages.  Whole
+    // synthesis, one CTA of two stages against two of one: 18.48 -> 17.02 ms (lmax 2048, 1 map), 1.34 ->
+    // 1.25 ms (Gauss-Legendre, lmax 750, 5 maps), 6.33 -> 5.15 ms (spin 2, lmax 1024, 1 map).
+    static constexpr int NCTA = N == 32 ? 1 : 2;
+    static constexpr int NST = N == 32 ? 2 : 1;               // stages
+    static constexpr int CP = N == 32 ? 8 : 4;                // columns of one epilogue step
+    static constexpr int G = N == 32 ? 8 : 4;                 // recurrence steps of one group
     static constexpr int B_CHUNK = 2 * NSTK * B_TILE;         // a_lm digits of one chunk
     static constexpr int A_BYTES = 2 * TC_S * TC_ATILE;       // y digits of one chunk
     static constexpr int Y_BYTES = TC_CH * TC_T * 8;          // one stage of y values
-    static constexpr int OFF_B = 2 * A_BYTES;
-    static constexpr int OFF_Y = OFF_B + 2 * B_CHUNK;
-    static constexpr int OFF_A = OFF_Y + 2 * Y_BYTES;         // the recurrence warps' coefficients
+    static constexpr int OFF_B = NST * A_BYTES;
+    static constexpr int OFF_Y = OFF_B + NST * B_CHUNK;
+    static constexpr int OFF_A = OFF_Y + NST * Y_BYTES;         // the recurrence warps' coefficients
     static constexpr int OFF_BAR = OFF_A + TC_ABUF;
     static constexpr int SMEM = OFF_BAR + 64;
-    static constexpr int TMEM_COLS = N == 8 ? 256 : 512;      // 2 NCLS N, a power of two
-    static_assert(SMEM > 114 * 1024 && SMEM <= 227 * 1024, "one CTA per SM");
+    static constexpr int TMEM_COLS = N == 32 ? 512 : 256;     // 2 NCLS N, a power of two
+    static_assert(2 * NCLS * N <= TMEM_COLS && NCTA * TMEM_COLS <= 512, "tensor memory");
+    static_assert((NCTA + 1) * SMEM > 228 * 1024 && NCTA * (SMEM + 1024) <= 228 * 1024, "NCTA CTAs per SM, no more");
 };
 
 size_t chunk_bytes(int N) { return (size_t)N * 512; }
@@ -302,18 +312,18 @@ __global__ void __launch_bounds__(TC_T) tc_tables_kernel(TcArgs A, int *Ey_out, 
 
 // Warp groups per CTA (one m, 128 slots, 416 threads):
 //   recurrence warps 0-3 (recurrence_warps): thread r runs the FP64 recurrence of slot r and
-//     writes each chunk's 32 values to a double-buffered y stage in shared memory;
+//     writes each chunk's 32 values to one of NST y stages in shared memory;
 //   split warps 4-11: thread (par, r) cuts the 16 values of parity par of slot r into digits and
-//     stores row r of the parity's A tiles (double-buffered); all of them copy the chunk's a_lm
+//     stores row r of the parity's A tiles (NST sets); all of them copy the chunk's a_lm
 //     digit tiles and arrive on the stage's full mbarrier; at the end they read tensor memory,
-//     warps 4-7 the even groups of 8 columns and warps 8-11 the odd ones;
+//     warps 4-7 the even groups of CP columns and warps 8-11 the odd ones;
 //   warp 12: waits on the full mbarrier, and one elected lane issues the chunk's MMAs
 //     (warp-uniform descriptors) and commits them to the stage's done mbarrier.
 // Stages: the y buffer is handed over with named barriers (FULL: recurrence arrives, split
 // waits; EMPTY: split arrives, recurrence waits, only where a later chunk reuses the stage);
 // the A/B tiles of a stage are rewritten after the done mbarrier of the MMAs that read them.
 template <int N, bool SPIN>
-__global__ void __launch_bounds__(TC_NT + 32, 1) tc_synth_kernel(TcArgs A)
+__global__ void __launch_bounds__(TC_NT + 32, TcTile<N>::NCTA) tc_synth_kernel(TcArgs A)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
     using W = TcTile<N>;
@@ -376,11 +386,11 @@ __global__ void __launch_bounds__(TC_NT + 32, 1) tc_synth_kernel(TcArgs A)
     bool ok = true;
     if (rec) {
         if (SPIN)
-            recurrence_warps<REC_SPIN, false, TC_T, 8>(A, m, blk, r, active, base, nch, cfirst, ybuf, abuf);
+            recurrence_warps<REC_SPIN, false, TC_T, W::G, W::NST>(A, m, blk, r, active, base, nch, cfirst, ybuf, abuf);
         else if (polar_block(A, m, blk))
-            recurrence_warps<REC_REIN, false, TC_T, 8>(A, m, blk, r, active, base, nch, cfirst, ybuf, abuf);
+            recurrence_warps<REC_REIN, false, TC_T, W::G, W::NST>(A, m, blk, r, active, base, nch, cfirst, ybuf, abuf);
         else
-            recurrence_warps<REC_Y, false, TC_T, 8>(A, m, blk, r, active, base, nch, cfirst, ybuf, abuf);
+            recurrence_warps<REC_Y, false, TC_T, W::G, W::NST>(A, m, blk, r, active, base, nch, cfirst, ybuf, abuf);
     } else if (issuer) {
         // ------------------------------------------------ MMA issue (one lane of the last warp)
         // per chunk: wait until the stage's tiles are written, issue its 2 x 20 MMAs (per parity eo,
@@ -390,8 +400,8 @@ __global__ void __launch_bounds__(TC_NT + 32, 1) tc_synth_kernel(TcArgs A)
         const uint64_t dB0 = umma_desc(smem_u32(sB), (W::N2 / 8) * 128, 128);
         const uint32_t issue = elect_one();
         for (int q = 0; q < nlive; ++q) {
-            const int st = q & 1;
-            if (ok && !mbar_wait(&full[st], (uint32_t)((q >> 1) & 1))) ok = false;
+            const int st = q & (W::NST - 1);
+            if (ok && !mbar_wait(&full[st], (uint32_t)((q >> (W::NST - 1)) & 1))) ok = false;
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;");
@@ -423,7 +433,7 @@ __global__ void __launch_bounds__(TC_NT + 32, 1) tc_synth_kernel(TcArgs A)
         constexpr int BTOT = W::B_CHUNK / 16;            // uint4 of one chunk's B tiles
         constexpr int BV = (BTOT + NS - 1) / NS;
         for (int q = 0; q < nlive; ++q) {
-            const int st = q & 1;
+            const int st = q & (W::NST - 1);
             unsigned char *a_st = sA + st * W::A_BYTES;
             unsigned char *b_st = sB + st * W::B_CHUNK;
             uint4 breg[BV];
@@ -442,10 +452,10 @@ __global__ void __launch_bounds__(TC_NT + 32, 1) tc_synth_kernel(TcArgs A)
                     const uint2 f1 = digit_fields(yb[(16 * h + 4 * p + 2 + par) * TC_T + r], Ey);
                     digit_pairs(f0, f1, pk[p]);
                 }
-                if (h == 1 && q + 2 < nlive) bar_arrive(BAR_EMPTY + st, TC_NT);  // y stage read
-                // the MMAs of chunk q - 2 read this stage's tiles: wait (bounded) before rewriting them
+                if (h == 1 && q + W::NST < nlive) bar_arrive(BAR_EMPTY + st, TC_NT);  // y stage read
+                // the MMAs of chunk q - NST read this stage's tiles: wait (bounded) before rewriting them
                 // (after the first half is cut, which only reads the y stage)
-                if (h == 0 && q >= 2 && ok && !mbar_wait(&mbar[st], (uint32_t)(((q >> 1) - 1) & 1))) ok = false;
+                if (h == 0 && q >= W::NST && ok && !mbar_wait(&mbar[st], (uint32_t)(((q >> (W::NST - 1)) - 1) & 1))) ok = false;
                 // k-group h of this parity's A tiles: core matrix (slot/8, h), row slot%8
                 const int off = ((h * 16) + (r >> 3)) * 128 + (r & 7) * 16;
 #pragma unroll
@@ -460,7 +470,7 @@ __global__ void __launch_bounds__(TC_NT + 32, 1) tc_synth_kernel(TcArgs A)
             mbar_arrive(&full[st]);
         }
         // the last commits cover every MMA issued: wait (bounded) before TMEM is read
-        if (ok && !mbar_wait(&mbar[(nlive - 1) & 1], (uint32_t)(((nlive - 1) >> 1) & 1))) ok = false;
+        if (ok && !mbar_wait(&mbar[(nlive - 1) & (W::NST - 1)], (uint32_t)(((nlive - 1) >> (W::NST - 1)) & 1))) ok = false;
         ok = bar_red_and(BAR_SPLIT, NS, ok);
         asm volatile("tcgen05.fence::after_thread_sync;");
         if (ok) {
@@ -468,28 +478,34 @@ __global__ void __launch_bounds__(TC_NT + 32, 1) tc_synth_kernel(TcArgs A)
             // class sums are integers: classes 0-3 add up to hi, 4-7 to lo (units of class 3 and class 7),
             // Delta_N = E + O and Delta_S = E - O are formed on them and rounded once to FP64, all on the
             // integer pipe: the FP64 pipe of this SM has no other CTA's work to do meanwhile.
+            constexpr int CP = W::CP;
             const int lw = warp & 3;  // this warp may read lanes 32 lw .. 32 lw + 31
             const int rn = active ? A.slotN[slot] : -1, rs = active ? A.slotS[slot] : -1;
             const int64_t mstride = A.mmax + 1;
 #pragma unroll 1
-            for (int cg = par; cg < N / 8; cg += 2) {  // 8 columns: 4 maps
-                if (4 * cg >= A.nmaps) break;
-                long long hi[2][8], lo[2][8];
+            for (int cg = par; cg < N / CP; cg += 2) {  // CP columns: CP / 2 maps
+                if (CP / 2 * cg >= A.nmaps) break;
+                long long hi[2][CP], lo[2][CP];
 #pragma unroll
                 for (int eo = 0; eo < 2; ++eo) {
-                    uint32_t v[TC_S][8];
+                    uint32_t v[TC_S][CP];
 #pragma unroll
                     for (int cls = 0; cls < TC_S; ++cls) {
                         const uint32_t addr =
-                            tmem + ((uint32_t)(lw * 32) << 16) + (uint32_t)((eo * W::NCLS + cls) * N + 8 * cg);
-                        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                                     : "=r"(v[cls][0]), "=r"(v[cls][1]), "=r"(v[cls][2]), "=r"(v[cls][3]),
-                                       "=r"(v[cls][4]), "=r"(v[cls][5]), "=r"(v[cls][6]), "=r"(v[cls][7])
-                                     : "r"(addr));
+                            tmem + ((uint32_t)(lw * 32) << 16) + (uint32_t)((eo * W::NCLS + cls) * N + CP * cg);
+                        if constexpr (CP == 8)
+                            asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                                         : "=r"(v[cls][0]), "=r"(v[cls][1]), "=r"(v[cls][2]), "=r"(v[cls][3]),
+                                           "=r"(v[cls][4]), "=r"(v[cls][5]), "=r"(v[cls][6]), "=r"(v[cls][7])
+                                         : "r"(addr));
+                        else
+                            asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                                         : "=r"(v[cls][0]), "=r"(v[cls][1]), "=r"(v[cls][2]), "=r"(v[cls][3])
+                                         : "r"(addr));
                     }
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                    for (int t = 0; t < 8; ++t) {
+                    for (int t = 0; t < CP; ++t) {
                         long long h = class_sum(__uint_as_float(v[0][t]));
                         h = h * 256 + class_sum(__uint_as_float(v[1][t]));
                         h = h * 256 + class_sum(__uint_as_float(v[2][t]));
@@ -501,15 +517,15 @@ __global__ void __launch_bounds__(TC_NT + 32, 1) tc_synth_kernel(TcArgs A)
                     }
                 }
 #pragma unroll
-                for (int gg = 0; gg < 4; ++gg) {
-                    const int g = 4 * cg + gg;  // map
+                for (int gg = 0; gg < CP / 2; ++gg) {
+                    const int g = CP / 2 * cg + gg;  // map
                     if (g >= A.nmaps) break;
                     const bool own = !SPIN || ((g & 1) == 0) == (A.sig > 0);
                     double vn[2], vs[2];
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
                         const int t = 2 * gg + c;
-                        const int e = Ey + A.Ea[m * N + 8 * cg + t] - 36;  // class 3: 2^(-6 - 6 - 24)
+                        const int e = Ey + A.Ea[m * N + CP * cg + t] - 36;  // class 3: 2^(-6 - 6 - 24)
                         if (own) vn[c] = pair_to_double(hi[0][t] + hi[1][t], lo[0][t] + lo[1][t], e);
                         if (!SPIN || !own) vs[c] = pair_to_double(hi[0][t] - hi[1][t], lo[0][t] - lo[1][t], e);
                     }

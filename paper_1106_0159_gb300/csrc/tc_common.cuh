@@ -277,7 +277,7 @@ __device__ __forceinline__ double rein_step(double be, double rh, double b0, dou
 
 // The recurrence warps (threads 0-127, thread r = slot r of the block) of the tensor-core kernels:
 // from the plan-time checkpoint at chunk cfirst (earlier chunks hold only dropped values) they run
-// the recurrence and write each chunk's 32 values (0 where dropped) to y stage q & 1, laid out
+// the recurrence and write each chunk's 32 values (0 where dropped) to y stage q & (NST - 1), laid out
 // [32 rows][YS doubles].  Row of step j: j, or with PAR the 16 even steps first.  Coefficients come
 // from a register of lane j (warp shuffle), loaded one chunk ahead.  Stages are handed over with
 // named barriers over all TC_NT threads: FULL (arrive here, the split warps wait) and EMPTY (the
@@ -299,7 +299,9 @@ __device__ __forceinline__ int y_row(int j)
     return PAR ? (j & 1) * (TC_CH / 2) + (j >> 1) : j;
 }
 
-template <int KIND, bool PAR, int YS, int G>
+//
+// NST y stages (2 or 1).
+template <int KIND, bool PAR, int YS, int G, int NST = 2>
 __device__ __forceinline__ void recurrence_warps(const TcArgs &A, int m, int blk, int r, bool active, int64_t base,
                                                  int nch, int cfirst, double *ybuf, double *abuf)
 {
@@ -321,8 +323,8 @@ __device__ __forceinline__ void recurrence_warps(const TcArgs &A, int m, int blk
     for (; c < nch && (REIN || __any_sync(0xffffffffu, k < 0)); ++c) {
         const RecCoef nxt = load_coef<KIND>(A, base, m, lb + TC_CH * (c + 1) + lane);
         const int q = c - cfirst;
-        double *yb = ybuf + (size_t)(q & 1) * TC_CH * YS + r;
-        if (q >= 2) bar_sync(BAR_EMPTY + (q & 1), TC_NT);  // the split warps read chunk q - 2
+        double *yb = ybuf + (size_t)(q & (NST - 1)) * TC_CH * YS + r;
+        if (q >= NST) bar_sync(BAR_EMPTY + (q & (NST - 1)), TC_NT);  // the split warps read chunk q - NST
         bool drop = false;
 #pragma unroll 1
         for (int j0 = 0; j0 < TC_CH; j0 += 4) {
@@ -359,7 +361,7 @@ __device__ __forceinline__ void recurrence_warps(const TcArgs &A, int m, int blk
                 k += 1;
             }
         }
-        bar_arrive(BAR_FULL + (q & 1), TC_NT);
+        bar_arrive(BAR_FULL + (q & (NST - 1)), TC_NT);
         cur = nxt;
     }
     if (REIN || c >= nch) return;
@@ -390,7 +392,7 @@ __device__ __forceinline__ void recurrence_warps(const TcArgs &A, int m, int blk
     for (const int c0 = c; c < nch; ++c) {
         const RecCoef nxt = load_coef<KIND>(A, base, m, lb + TC_CH * (c + 1) + lane);
         const int q = c - cfirst;
-        double *yb = ybuf + (size_t)(q & 1) * TC_CH * YS + r;
+        double *yb = ybuf + (size_t)(q & (NST - 1)) * TC_CH * YS + r;
 #pragma unroll
         for (int j0 = 0; j0 < TC_CH; j0 += G) {
             // coefficients that are all read make room for the next ones: a chunk's 32, or (spin) 16 pairs
@@ -432,8 +434,8 @@ __device__ __forceinline__ void recurrence_warps(const TcArgs &A, int m, int blk
                 if (store) pp[y_row<PAR>(((j0 - G) & 31) + j) * YS] = pv[j];  // steps j0 - G .. j0 - 1
             }
             if (j0 == 0) {
-                if (c > c0) bar_arrive(BAR_FULL + ((q - 1) & 1), TC_NT);
-                if (q >= 2) bar_sync(BAR_EMPTY + (q & 1), TC_NT);  // the split warps read chunk q - 2
+                if (c > c0) bar_arrive(BAR_FULL + ((q - 1) & (NST - 1)), TC_NT);
+                if (q >= NST) bar_sync(BAR_EMPTY + (q & (NST - 1)), TC_NT);  // the split warps read chunk q - NST
                 pp = yb;
             }
 #pragma unroll
@@ -448,5 +450,5 @@ __device__ __forceinline__ void recurrence_warps(const TcArgs &A, int m, int blk
     }
 #pragma unroll
     for (int j = 0; j < G; ++j) pp[y_row<PAR>(TC_CH - G + j) * YS] = pv[j];
-    bar_arrive(BAR_FULL + ((nch - 1 - cfirst) & 1), TC_NT);
+    bar_arrive(BAR_FULL + ((nch - 1 - cfirst) & (NST - 1)), TC_NT);
 }
