@@ -95,9 +95,11 @@ __device__ __forceinline__ void tmem_st4(uint32_t addr, uint32_t a, uint32_t b, 
 
 // CTA: one m, 128 slots, 672 threads in four roles.
 //   warps 0-3   recurrence (recurrence_warps, double-buffered y stage of 32 l, even steps first);
-//   warps 4-11  split: stage X = Sigma | D of the block in shared memory, cut it into tensor memory
-//               once, then cut each chunk's y values into one of two tile sets and arrive on its full
-//               barrier;
+//   warps 4-19  first stage X = Sigma | D of the block in shared memory and cut it into tensor memory,
+//               while the recurrence fills its two stages (whole analysis, with the recurrence waiting
+//               for X cut by warps 4-11 alone against this: 23.59 -> 22.67 ms at lmax 2048, 1 map,
+//               179.9 -> 173.0 at 4096, 4 maps, 200.6 -> 193.3 with 16); then
+//   warps 4-11  split: cut each chunk's y values into one of two tile sets and arrive on its full barrier;
 //   warps 12-19 epilogue, two per tensor-memory lane quarter (8 of the row's 16 columns each): wait for
 //               each region, read it, release it, add the class sums of the top and bottom halves (lane
 //               quarters 0, 1 and 2, 3) through shared memory and write the block's partial a_lm / c_lm;
@@ -165,9 +167,109 @@ __global__ void __launch_bounds__(TA_NT, 1) tc_anal_kernel(TcArgs A)
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = *tslot;
 
+    if (splitw || epi) {
+        // ------------------------------------------------ X into tensor memory, beside the first chunks of y
+        {
+            // rows 32 s + 2 g + c (s: Sigma, D; map g; c: re, im) of slot r: this thread's maps are
+            // hh, hh + 4, ... (uniform per warp); the rows of absent maps are zero
+            const int hh = sp >> 7;
+            const int rn = active ? A.slotN[slot] : -1, rs = active ? A.slotS[slot] : -1;
+            const int64_t mstride = A.mmax + 1, dstride = (int64_t)A.nrings * mstride;
+            double *xr = xs + r * TA_XROW;
+            const bool bn = rn >= 0 && SHT_CHK(rn < A.nrings), bs = rs >= 0 && SHT_CHK(rs < A.nrings);
+            const double2 *dN = A.delta + (int64_t)(bn ? rn : 0) * mstride + m;
+            const double2 *dS = A.delta + (int64_t)(bs ? rs : 0) * mstride + m;
+            const double2 zero = make_double2(0.0, 0.0);
+            if (SPIN) {
+                // column pair 2 h + c of polarised map h (this thread: h = hh, hh + 4, ...): Dq +- i Du of the
+                // northern ring for the pass's own sign c (0: +), of the southern ring for the other
+#pragma unroll 1
+                for (int h = hh; h < TA_MAPS / 2; h += 4) {
+                    const bool have = 2 * h < nm;
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        const bool own = (c == 0) == (A.sig > 0);
+                        const double2 *d = (own ? dN : dS) + 2 * h * dstride;
+                        const bool in = have && (own ? bn : bs);
+                        const double2 q = in ? d[0] : zero, w = in ? d[dstride] : zero;
+                        const double re = c == 0 ? q.x - w.y : q.x + w.y, im = c == 0 ? q.y + w.x : q.y - w.x;
+                        const bool neg = !own && m == 1;  // (-1)^(l+m) of the even rows, l - max(m, 2) even
+                        double *x = xr + 2 * (2 * h + c);
+                        x[0] = neg ? -re : re;
+                        x[1] = neg ? -im : im;
+                        x[32] = own || neg ? re : -re;
+                        x[33] = own || neg ? im : -im;
+                    }
+                }
+            } else {
+                // rolled, one map ahead: unrolled over the 8 maps the loop was slower (its code is run once per
+                // CTA: instruction fetch), 202.9 -> 200.5 ms for the whole analysis at lmax 4096, 16 maps
+                double2 n = bn && hh < nm ? dN[hh * dstride] : zero, s = bs && hh < nm ? dS[hh * dstride] : zero;
+#pragma unroll 1
+                for (int g = hh; g < TA_MAPS; g += 4) {
+                    const bool more = g + 4 < nm;
+                    const double2 n1 = bn && more ? dN[(g + 4) * dstride] : zero, s1 = bs && more ? dS[(g + 4) * dstride] : zero;
+                    double *x = xr + 2 * g;
+                    if (g < nm) {
+                        x[0] = n.x + s.x;
+                        x[1] = n.y + s.y;
+                        x[32] = n.x - s.x;
+                        x[33] = n.y - s.y;
+                    } else {
+                        x[0] = x[1] = x[32] = x[33] = 0.0;
+                    }
+                    n = n1;
+                    s = s1;
+                }
+            }
+        }
+        bar_sync(BAR_STAGED, 2 * TC_T + TA_NEPI);  // X staged
+        {
+            // lane quarter qd holds rows 32 (qd & 1) .. + 31: the even digits of each stack in quarters
+            // 0, 1 and the odd ones in 2, 3.  Four warps each take 32 slots.
+            const int qd = warp & 3, kh = (warp - 4) >> 2;
+            const int row = 32 * (qd & 1) + lane;
+            const double *xc = xs + (32 * kh) * TA_XROW + row;
+            if (qd < 2) {  // row exponents and rows the digits cannot carry
+                int mx = 0;
+                bool odd = false;
+#pragma unroll 4
+                for (int k = 0; k < 32; ++k) {
+                    const double v = xc[k * TA_XROW];
+                    const int ex = dexp(v);
+                    mx = max(mx, ex);
+                    odd |= ex == 0 && (((uint32_t)__double2hiint(v) << 1) | (uint32_t)__double2loint(v)) != 0u;
+                }
+                if (mx) atomicMax(&sEx[row], mx);
+                if (odd || mx > TC_EHUGE) A.fix[m * 16 + (lane >> 1)] = 1;
+            }
+            bar_sync(BAR_STAGED, 2 * TC_T + TA_NEPI);  // row exponents complete
+            const int e = sEx[row];
+            if (kh == 0 && qd < 2 && e && e < TC_ETINY) A.fix[m * 16 + (lane >> 1)] = 1;
+            const int E = e ? e - 1022 : TC_EZERO;
+            const uint32_t at = tmem + ((uint32_t)(32 * qd) << 16) + (uint32_t)(TA_XCOL + 2 * kh * 8);
+#pragma unroll 1
+            for (int p0 = 0; p0 < 16; p0 += 4) {  // 4 slot pairs = 4 columns of K-step 2 kh + p0 / 8
+                uint32_t w[4][4];
+#pragma unroll
+                for (int p = 0; p < 4; ++p) {
+                    const uint2 f0 = digit_fields(xc[(2 * (p0 + p)) * TA_XROW], E);
+                    const uint2 f1 = digit_fields(xc[(2 * (p0 + p) + 1) * TA_XROW], E);
+                    uint32_t d[TC_S];
+                    digit_pairs(f0, f1, d);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) w[i][p] = qd < 2 ? d[2 * i] : d[2 * i + 1];
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) tmem_st4(at + (uint32_t)(i * TA_KS * 8 + p0), w[i][0], w[i][1], w[i][2], w[i][3]);
+            }
+            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;");
+    }
+
     bool ok = true;
     if (rec) {
-        bar_sync(BAR_STAGED, TC_NT);  // X staged: its additions need the FP64 pipe first
         if (SPIN)
             recurrence_warps<REC_SPIN, true, TA_YS, 4>(A, m, blk, r, active, base, nch, cfirst, ybuf, abuf);
         else if (polar_block(A, m, blk))
@@ -209,107 +311,9 @@ __global__ void __launch_bounds__(TA_NT, 1) tc_anal_kernel(TcArgs A)
         }
         if (lane == 0 && !ok) atomicOr(A.status, 1);
     } else if (splitw) {
-        // ------------------------------------------------ X into tensor memory, then the y tiles
+        // ------------------------------------------------ the y tiles
         const int Ey = A.Ey[m * A.nblk + blk];
-        {
-            // rows 32 s + 2 g + c (s: Sigma, D; map g; c: re, im) of slot r: this thread's maps are
-            // hh, hh + 2, ... (uniform per warp); the rows of absent maps are zero
-            const int hh = sp >> 7;
-            const int rn = active ? A.slotN[slot] : -1, rs = active ? A.slotS[slot] : -1;
-            const int64_t mstride = A.mmax + 1, dstride = (int64_t)A.nrings * mstride;
-            double *xr = xs + r * TA_XROW;
-            const bool bn = rn >= 0 && SHT_CHK(rn < A.nrings), bs = rs >= 0 && SHT_CHK(rs < A.nrings);
-            const double2 *dN = A.delta + (int64_t)(bn ? rn : 0) * mstride + m;
-            const double2 *dS = A.delta + (int64_t)(bs ? rs : 0) * mstride + m;
-            const double2 zero = make_double2(0.0, 0.0);
-            if (SPIN) {
-                // column pair 2 h + c of polarised map h (this thread: h = hh, hh + 2, ...): Dq +- i Du of the
-                // northern ring for the pass's own sign c (0: +), of the southern ring for the other
-#pragma unroll 1
-                for (int h = hh; h < TA_MAPS / 2; h += 2) {
-                    const bool have = 2 * h < nm;
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-                        const bool own = (c == 0) == (A.sig > 0);
-                        const double2 *d = (own ? dN : dS) + 2 * h * dstride;
-                        const bool in = have && (own ? bn : bs);
-                        const double2 q = in ? d[0] : zero, w = in ? d[dstride] : zero;
-                        const double re = c == 0 ? q.x - w.y : q.x + w.y, im = c == 0 ? q.y + w.x : q.y - w.x;
-                        const bool neg = !own && m == 1;  // (-1)^(l+m) of the even rows, l - max(m, 2) even
-                        double *x = xr + 2 * (2 * h + c);
-                        x[0] = neg ? -re : re;
-                        x[1] = neg ? -im : im;
-                        x[32] = own || neg ? re : -re;
-                        x[33] = own || neg ? im : -im;
-                    }
-                }
-            } else {
-                // rolled, one map ahead: unrolled over the 8 maps the loop was slower (its code is run once per
-                // CTA: instruction fetch), 202.9 -> 200.5 ms for the whole analysis at lmax 4096, 16 maps
-                double2 n = bn && hh < nm ? dN[hh * dstride] : zero, s = bs && hh < nm ? dS[hh * dstride] : zero;
-#pragma unroll 1
-                for (int g = hh; g < TA_MAPS; g += 2) {
-                    const bool more = g + 2 < nm;
-                    const double2 n1 = bn && more ? dN[(g + 2) * dstride] : zero, s1 = bs && more ? dS[(g + 2) * dstride] : zero;
-                    double *x = xr + 2 * g;
-                    if (g < nm) {
-                        x[0] = n.x + s.x;
-                        x[1] = n.y + s.y;
-                        x[32] = n.x - s.x;
-                        x[33] = n.y - s.y;
-                    } else {
-                        x[0] = x[1] = x[32] = x[33] = 0.0;
-                    }
-                    n = n1;
-                    s = s1;
-                }
-            }
-        }
-        bar_sync(BAR_STAGED, TC_NT);  // X staged; the recurrence starts
-        {
-            // lane quarter qd holds rows 32 (qd & 1) .. + 31: the even digits of each stack in quarters
-            // 0, 1 and the odd ones in 2, 3.  Warps 4-7 take slots 0-63, warps 8-11 slots 64-127.
-            const int qd = warp & 3, kh = (warp - 4) >> 2;
-            const int row = 32 * (qd & 1) + lane;
-            const double *xc = xs + (64 * kh) * TA_XROW + row;
-            if (qd < 2) {  // row exponents and rows the digits cannot carry
-                int mx = 0;
-                bool odd = false;
-#pragma unroll 4
-                for (int k = 0; k < 64; ++k) {
-                    const double v = xc[k * TA_XROW];
-                    const int ex = dexp(v);
-                    mx = max(mx, ex);
-                    odd |= ex == 0 && (((uint32_t)__double2hiint(v) << 1) | (uint32_t)__double2loint(v)) != 0u;
-                }
-                if (mx) atomicMax(&sEx[row], mx);
-                if (odd || mx > TC_EHUGE) A.fix[m * 16 + (lane >> 1)] = 1;
-            }
-            bar_sync(BAR_SPLIT, 2 * TC_T);  // row exponents complete
-            const int e = sEx[row];
-            if (kh == 0 && qd < 2 && e && e < TC_ETINY) A.fix[m * 16 + (lane >> 1)] = 1;
-            const int E = e ? e - 1022 : TC_EZERO;
-            const uint32_t at = tmem + ((uint32_t)(32 * qd) << 16) + (uint32_t)(TA_XCOL + 4 * kh * 8);
-#pragma unroll 1
-            for (int p0 = 0; p0 < 32; p0 += 4) {  // 4 slot pairs = 4 columns of K-step 4 kh + p0 / 8
-                uint32_t w[4][4];
-#pragma unroll
-                for (int p = 0; p < 4; ++p) {
-                    const uint2 f0 = digit_fields(xc[(2 * (p0 + p)) * TA_XROW], E);
-                    const uint2 f1 = digit_fields(xc[(2 * (p0 + p) + 1) * TA_XROW], E);
-                    uint32_t d[TC_S];
-                    digit_pairs(f0, f1, d);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) w[i][p] = qd < 2 ? d[2 * i] : d[2 * i + 1];
-                }
-#pragma unroll
-                for (int i = 0; i < 4; ++i) tmem_st4(at + (uint32_t)(i * TA_KS * 8 + p0), w[i][0], w[i][1], w[i][2], w[i][3]);
-            }
-            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-        }
-        asm volatile("tcgen05.fence::before_thread_sync;");
         bar_sync(BAR_PREP, 2 * TC_T + TA_NEPI + 32);  // X in tensor memory, its staging area free
-
         // this thread cuts row n of the y stage (l - l0 = 2 (n % 16) + n / 16) for the 8-slot groups
         // sg and sg + 8: its 8 values of a digit are one 16-byte core-matrix row
         const int w8 = warp - 4;
