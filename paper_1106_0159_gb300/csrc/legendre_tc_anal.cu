@@ -93,6 +93,18 @@ __device__ __forceinline__ void tmem_st4(uint32_t addr, uint32_t a, uint32_t b, 
                  : "memory");
 }
 
+// The sums of classes 0 .. 7 of one column as one integer in units of 2^-3 of class 5, rounded to FP64
+__device__ __forceinline__ double classes_to_double(const float (&v)[8], int e)
+{
+    int S[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) S[c] = class_sum(v[c]);
+    const long long H = (long long)S[0] * 65536 + (S[1] * 256 + S[2]);              // class 2
+    const long long M = (long long)S[3] * 65536 + ((long long)S[4] * 256 + S[5]);  // class 5
+    const long long Z = (long long)S[6] * 256 + S[7];                             // class 7
+    return i64_to_double(H * (1ll << 27) + M * 8 + ((Z + 4096) >> 13), e);
+}
+
 // CTA: one m, 128 slots, 672 threads in four roles.
 //   warps 0-3   recurrence (recurrence_warps, double-buffered y stage of 32 l, even steps first);
 //   warps 4-19  first stage X = Sigma | D of the block in shared memory and cut it into tensor memory,
@@ -354,10 +366,15 @@ __global__ void __launch_bounds__(TA_NT, 1) tc_anal_kernel(TcArgs A)
         // the 8 columns of this warp the top lane finishes 4 and the bottom lane of the same row the other
         // 4: each hands the other its sums of those, and the eight class sums of a column become one
         // integer in units of 2^-3 of class 5 (2^-55 of 2^(E_y + E_x)), rounded once to FP64.
+        // Up to 8 (4) maps only lanes 0-15 (0-7) hold rows: they leave their own sums beside those handed
+        // over, and all lanes take a share of the columns, W / 8 each (whole analysis, against every lane
+        // finishing 4: 22.67 -> 22.02 ms at lmax 2048, 1 map, 173.0 -> 168.4 at 4096, 4 maps).
         const int qd = warp & 3, es = qd & 1, hc = (warp - 12) >> 2;
         const bool top = qd < 2;
-        const int erow = 32 * es + lane;
-        const int eg = lane >> 1, ec = lane & 1;
+        const int W = nm <= 4 ? 8 : nm <= 8 ? 16 : 32;
+        const int rr = lane & (W - 1);          // this lane finishes columns of row 32 es + rr
+        const int erow = 32 * es + rr;
+        const int eg = rr >> 1, ec = rr & 1;
         const int t0 = 4 * hc + (top ? 0 : 8);  // this lane finishes columns t0 .. t0 + 3
         bar_sync(BAR_PREP, 2 * TC_T + TA_NEPI + 32);  // row exponents complete
         const int ex = sEx[erow];
@@ -391,17 +408,21 @@ __global__ void __launch_bounds__(TA_NT, 1) tc_anal_kernel(TcArgs A)
                 const float4 fr = make_float4(__uint_as_float(orr[0]), __uint_as_float(orr[1]), __uint_as_float(orr[2]),
                                               __uint_as_float(orr[3]));
                 if (top) {
-                    mine[(2 * t) * TA_NEPI] = fl;
-                    mine[(2 * t + 1) * TA_NEPI] = fr;
+                    if (lane < W) {
+                        mine[(2 * t) * TA_NEPI] = fl;
+                        mine[(2 * t + 1) * TA_NEPI] = fr;
+                    }
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         v[t][0][j] = __uint_as_float(l[j]);
                         v[t][1][j] = __uint_as_float(r[j]);
                     }
                 } else {
-                    if (t == 0) mine[0] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    mine[(2 * t + 1) * TA_NEPI] = fl;
-                    if (t + 1 < TA_REG) mine[(2 * t + 2) * TA_NEPI] = fr;
+                    if (lane < W) {
+                        if (t == 0) mine[0] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        mine[(2 * t + 1) * TA_NEPI] = fl;
+                        if (t + 1 < TA_REG) mine[(2 * t + 2) * TA_NEPI] = fr;
+                    }
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         if (t == 0) v[0][0][j] = 0.f;
@@ -410,8 +431,27 @@ __global__ void __launch_bounds__(TA_NT, 1) tc_anal_kernel(TcArgs A)
                     }
                 }
             }
+            if (lane < W && W < 32) {
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const float *w = v[c >> 1][c & 1];
+                    mine[c * TA_NEPI + W] = make_float4(w[0], w[1], w[2], w[3]);
+                }
+            }
             ok = bar_red_and(BAR_EPI + 1, TA_NEPI, ok);  // the sums are handed over; the warps agree
-            if (ok) {
+            if (ok && W < 32) {
+                const float *po = (const float *)(other - lane + rr), *pm = (const float *)(mine - lane + W + rr);
+#pragma unroll 1
+                for (int j = lane / W * (W / 8), i = 0; i < W / 8; ++i, ++j) {
+                    float f[8];
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) f[c] = pm[4 * c * TA_NEPI + j] + po[4 * c * TA_NEPI + j];
+                    const double d = classes_to_double(f, e);
+                    const int l = l1 + TC_CH * q + 2 * j;
+                    if (eg < nm && l <= L && SHT_CHK(base + (l - m) >= A.idx0 && base + (l - m) < A.idx0 + A.nalm_part))
+                        dst[(int64_t)(4 * j) * nm] = d;
+                }
+            } else if (ok) {
 #pragma unroll
                 for (int t = 0; t < TA_REG; ++t)
 #pragma unroll
@@ -424,13 +464,10 @@ __global__ void __launch_bounds__(TA_NT, 1) tc_anal_kernel(TcArgs A)
                     }
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    int S[8];
+                    float f[8];
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) S[c] = class_sum(v[c >> 1][c & 1][j]);
-                    const long long H = (long long)S[0] * 65536 + (S[1] * 256 + S[2]);              // class 2
-                    const long long M = (long long)S[3] * 65536 + ((long long)S[4] * 256 + S[5]);  // class 5
-                    const long long Z = (long long)S[6] * 256 + S[7];                             // class 7
-                    const double d = i64_to_double(H * (1ll << 27) + M * 8 + ((Z + 4096) >> 13), e);
+                    for (int c = 0; c < 8; ++c) f[c] = v[c >> 1][c & 1][j];
+                    const double d = classes_to_double(f, e);
                     const int l = l1 + TC_CH * q + 2 * j;
                     if (eg < nm && l <= L && SHT_CHK(base + (l - m) >= A.idx0 && base + (l - m) < A.idx0 + A.nalm_part))
                         dst[(int64_t)(4 * j) * nm] = d;
