@@ -74,16 +74,16 @@ def parse():
     return ap.parse_args()
 
 
-MODES = {"split": "precision form: FP64 recurrence, tensor-core (tcgen05, split-bf16, 7 digits) synthesis "
+MODES = {"split": "precision form: FP64 recurrence, tensor-core (tcgen05, 8 base-256 fp16 digits) synthesis "
                   "sum, %s analysis sum",
-         "fp64": "plain FP64"}
+         "fp64": "FP64"}
 
 
 def mode_desc(a, mode=None):
     mode = mode or a.mode
     if mode != "split":
         return MODES[mode]
-    return MODES[mode] % ("tensor-core (split-bf16)" if a.prec_anal == "tc" else "double-float (FP32 pipe)")
+    return MODES[mode] % ("tensor-core (the same digits)" if a.prec_anal == "tc" else "double-float (FP32 pipe)")
 
 
 def workload_name(a):
@@ -594,8 +594,8 @@ def ours_arm(a, rank, world, local_rank):
             "metric": METRIC, "value": value, "unit": "maps/s", "n_gpus": world, "steps": a.steps,
             "warmup": a.warmup, "ms_per_step": total_ms / a.steps, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None,
-            "dtype": ("f64 recurrence; synthesis: bf16 digits (tcgen05, f32 accum, f64 combination); analysis: "
-                      + ("bf16 digits (tcgen05)" if a.prec_anal == "tc" else "double-float (f32 pairs)"))
+            "dtype": ("f64 recurrence; synthesis: fp16 digits (tcgen05, exact f32 class sums, integer combination); analysis: "
+                      + ("fp16 digits (tcgen05)" if a.prec_anal == "tc" else "double-float (f32 pairs)"))
                      if a.mode == "split" else "f64",
             "data": DATA,
             "config": workload_config(a),

@@ -28,8 +28,8 @@
 //      the chunk's stage and copy in the a_lm digit tiles (prepared by tc_split_b_kernel);
 //   3. one lane of the issuing warp issues the 2 x 20 MMAs (M = 128, N2 columns, K = 16) and
 //      commits them to the stage's mbarrier.
-// y values and tiles are double-buffered, so the recurrence of chunk c + 1 runs while chunk c is
-// cut and multiplied.  The B operand stacks two a_lm digits along N: stack b/2 = [B_b | B_(b+1)],
+// y values and tiles are double-buffered (16 maps), or a second CTA has the SM meanwhile (up to 8), so
+// recurrence runs while a chunk is cut and multiplied.  The B operand stacks two a_lm digits along N: stack b/2 = [B_b | B_(b+1)],
 // so one MMA A_a x stack adds class a + b to accumulator block a + b and class a + b + 1 to block
 // a + b + 1 (20 MMAs per parity and chunk instead of 36).
 //
@@ -38,9 +38,11 @@
 // pair is two complex columns E + iB, E - iB, and two passes, one per sign of the recurrence, give
 // P+- everywhere: the column of the pass's own sign on the northern rings (E + O), the other on the
 // southern ones (E - O).  spin_combine_kernel then forms Q and U.  4 FP64 instructions per step and
-// ring pair for up to 8 maps, where the FP64 kernels take 6 + 8 per map.
+// ring pair for up to 8 maps, where the FP64 kernels take 6 + 8 per map (lmax 1024, 1 map: whole synthesis
+// 20.7 -> 5.15 ms; analysis of 2 maps 32.5 -> 7.62 ms).
 //
-// What bounds it: the FP64 recurrence, 64 FP64 instructions per warp and chunk = 4096 SM cycles.
+// What bounds it: the FP64 recurrence, 64 FP64 instructions per warp and chunk = 4096 SM cycles, and the
+// other roles' instructions that delay it (about 6.1K cycles a chunk at lmax 4096, 16 maps: 124 ms).
 #include "sht_internal.h"
 
 #include <algorithm>

@@ -277,7 +277,7 @@ __device__ __forceinline__ double rein_step(double be, double rh, double b0, dou
 
 // The recurrence warps (threads 0-127, thread r = slot r of the block) of the tensor-core kernels:
 // from the plan-time checkpoint at chunk cfirst (earlier chunks hold only dropped values) they run
-// the recurrence and write each chunk's 32 values (0 where dropped) to y stage q & (NST - 1), laid out
+// the recurrence and write each chunk's 32 values (0 where dropped) to one of NST (2 or 1) y stages, laid out
 // [32 rows][YS doubles].  Row of step j: j, or with PAR the 16 even steps first.  Coefficients come
 // from a register of lane j (warp shuffle), loaded one chunk ahead.  Stages are handed over with
 // named barriers over all TC_NT threads: FULL (arrive here, the split warps wait) and EMPTY (the
@@ -299,8 +299,6 @@ __device__ __forceinline__ int y_row(int j)
     return PAR ? (j & 1) * (TC_CH / 2) + (j >> 1) : j;
 }
 
-//
-// NST y stages (2 or 1).
 template <int KIND, bool PAR, int YS, int G, int NST = 2>
 __device__ __forceinline__ void recurrence_warps(const TcArgs &A, int m, int blk, int r, bool active, int64_t base,
                                                  int nch, int cfirst, double *ybuf, double *abuf)
