@@ -55,8 +55,8 @@ namespace {
 constexpr int TC_ATILE = TC_T * 16 * 2;      // bytes of one [128 x 16] fp16 tile
 constexpr size_t TC_SLAB_BYTES = size_t(2) << 30;  // a_lm digits held at a time (whole m)
 
-// N columns (2 per map): 8, 16 or 32
-template <int N>
+// N columns (2 per map): 8, 16 or 32; NC CTAs per SM
+template <int N, int NC = 1>
 struct TcTile {
     static constexpr int N2 = 2 * N;                          // columns of one B stack
     static constexpr int B_TILE = N2 * 16 * 2;                // bytes of one [N2 x 16] stack
@@ -64,15 +64,14 @@ struct TcTile {
     // accumulator blocks per parity: classes 0 .. 7, and where there is room one that takes the second
     // halves of the class-7 stacks (incomplete, not read); else those MMAs take half a stack
     static constexpr int NCLS = N == 8 ? TC_S + 1 : TC_S;
-    // Up to 8 maps two CTAs share an SM, each with one stage of y values and tiles: while one waits for
+    // Up to 8 maps two CTAs can share an SM (launch_slab), each with one stage of y values and tiles: while one waits for
     // its stage or for tensor memory the other's recurrence has the FP64 pipe, and where both run the
     // pipe is never short of a warp.  16 maps take all of tensor memory: one CTA, two stages.  Whole
     // synthesis, one CTA of two stages against two of one: 18.48 -> 17.02 ms (lmax 2048, 1 map), 1.34 ->
     // 1.25 ms (Gauss-Legendre, lmax 750, 5 maps), 6.33 -> 5.15 ms (spin 2, lmax 1024, 1 map).
-    static constexpr int NCTA = N == 32 ? 1 : 2;
-    static constexpr int NST = N == 32 ? 2 : 1;               // stages
-    static constexpr int CP = N == 32 ? 8 : 4;                // columns of one epilogue step
-    static constexpr int G = N == 32 ? 8 : 4;                 // recurrence steps of one group
+    static constexpr int NST = NC == 1 ? 2 : 1;               // stages
+    static constexpr int CP = NC == 1 ? 8 : 4;                // columns of one epilogue step
+    static constexpr int G = NC == 1 ? 8 : 4;                 // recurrence steps of one group
     static constexpr int B_CHUNK = 2 * NSTK * B_TILE;         // a_lm digits of one chunk
     static constexpr int A_BYTES = 2 * TC_S * TC_ATILE;       // y digits of one chunk
     static constexpr int Y_BYTES = TC_CH * TC_T * 8;          // one stage of y values
@@ -82,8 +81,8 @@ struct TcTile {
     static constexpr int OFF_BAR = OFF_A + TC_ABUF;
     static constexpr int SMEM = OFF_BAR + 64;
     static constexpr int TMEM_COLS = N == 32 ? 512 : 256;     // 2 NCLS N, a power of two
-    static_assert(2 * NCLS * N <= TMEM_COLS && NCTA * TMEM_COLS <= 512, "tensor memory");
-    static_assert((NCTA + 1) * SMEM > 228 * 1024 && NCTA * (SMEM + 1024) <= 228 * 1024, "NCTA CTAs per SM, no more");
+    static_assert(2 * NCLS * N <= TMEM_COLS && NC * TMEM_COLS <= 512, "tensor memory");
+    static_assert((NC + 1) * SMEM > 228 * 1024 && NC * (SMEM + 1024) <= 228 * 1024, "NC CTAs per SM, no more");
 };
 
 size_t chunk_bytes(int N) { return (size_t)N * 512; }
@@ -324,11 +323,11 @@ __global__ void __launch_bounds__(TC_T) tc_tables_kernel(TcArgs A, int *Ey_out, 
 // Stages: the y buffer is handed over with named barriers (FULL: recurrence arrives, split
 // waits; EMPTY: split arrives, recurrence waits, only where a later chunk reuses the stage);
 // the A/B tiles of a stage are rewritten after the done mbarrier of the MMAs that read them.
-template <int N, bool SPIN>
-__global__ void __launch_bounds__(TC_NT + 32, TcTile<N>::NCTA) tc_synth_kernel(TcArgs A)
+template <int N, int NC, bool SPIN>
+__global__ void __launch_bounds__(TC_NT + 32, NC) tc_synth_kernel(TcArgs A)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
-    using W = TcTile<N>;
+    using W = TcTile<N, NC>;
     unsigned char *sA = smem;                               // [stage][parity][digit][128 x 16] fp16
     unsigned char *sB = smem + W::OFF_B;                    // [stage][parity][stack][N2 x 16] fp16
     double *ybuf = (double *)(smem + W::OFF_Y);             // [stage][32 l][128 slots]
@@ -564,14 +563,31 @@ __global__ void spin_combine_kernel(double2 *__restrict__ delta, int64_t n, int 
     }
 }
 
+template <int N, int NC>
+cudaError_t set_synth_smem(cudaFuncAttribute a)
+{
+    cudaError_t e = cudaFuncSetAttribute(tc_synth_kernel<N, NC, false>, a, TcTile<N, NC>::SMEM);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(tc_synth_kernel<N, NC, true>, a, TcTile<N, NC>::SMEM);
+}
+
 template <int N, bool SPIN>
 cudaError_t launch_slab(const Plan &p, const TcArgs &A, int count_m, int64_t nchunks, cudaStream_t st)
 {
+    constexpr int NC2 = N == 32 ? 1 : 2;
+    const unsigned ctas = (unsigned)(count_m * A.nblk);
+    // Two CTAs per SM once there are enough of them.  With few, the time is that of the longest chain, a polar
+    // block's Reinsch steps at low m, and a lone CTA with two stages runs it faster.  One map, one against two,
+    // us: 386 CTAs (lmax 192) 73 / 92, 514 (256) 100 / 116, 963 (320) 174 / 149, 6152 (768) 1242 / 1085.  The
+    // spin recurrence has no such blocks, whole synthesis: 193 CTAs 108 / 113, 386 158 / 133, 514 223 / 193.
+    const bool two = NC2 == 2 && ctas >= (SPIN ? 2u : 5u) * 152u;
     tc_scale_kernel<N, SPIN><<<count_m, 256, 0, st>>>(A);
     tc_split_b_kernel<N, SPIN><<<(unsigned)nchunks, 4 * N, 0, st>>>(A);  // one thread per (parity, k half, column)
     if (!SPIN) {
         StageEvents ev(p, SHT_STAGE_TC_SYNTH_KERNEL, st);
-        tc_synth_kernel<N, false><<<(unsigned)(count_m * A.nblk), TC_NT + 32, TcTile<N>::SMEM, st>>>(A);
+        if (two)
+            tc_synth_kernel<N, NC2, false><<<ctas, TC_NT + 32, TcTile<N, NC2>::SMEM, st>>>(A);
+        else
+            tc_synth_kernel<N, 1, false><<<ctas, TC_NT + 32, TcTile<N>::SMEM, st>>>(A);
         p.launches[SHT_STAGE_TC_SYNTH_KERNEL] += 1;
         ev.done();
     } else {  // both signs of the recurrence on the same columns
@@ -579,7 +595,10 @@ cudaError_t launch_slab(const Plan &p, const TcArgs &A, int count_m, int64_t nch
         TcArgs B = A;
         for (int sig = 1; sig >= -1; sig -= 2) {
             B.sig = sig;
-            tc_synth_kernel<N, true><<<(unsigned)(count_m * A.nblk), TC_NT + 32, TcTile<N>::SMEM, st>>>(B);
+            if (two)
+                tc_synth_kernel<N, NC2, true><<<ctas, TC_NT + 32, TcTile<N, NC2>::SMEM, st>>>(B);
+            else
+                tc_synth_kernel<N, 1, true><<<ctas, TC_NT + 32, TcTile<N>::SMEM, st>>>(B);
             B.Ey += 2 * tables;
             B.first += 2 * tables;
             B.ck_y += tables * TC_T;
@@ -628,12 +647,11 @@ size_t exponent_bytes(const Plan &p) { return (size_t)(p.mmax + 1) * (32 + 16) *
 cudaError_t configure_tc_kernels()
 {
     const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaError_t e = cudaFuncSetAttribute(tc_synth_kernel<32, false>, a, TcTile<32>::SMEM);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_synth_kernel<16, false>, a, TcTile<16>::SMEM);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_synth_kernel<8, false>, a, TcTile<8>::SMEM);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_synth_kernel<32, true>, a, TcTile<32>::SMEM);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_synth_kernel<16, true>, a, TcTile<16>::SMEM);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_synth_kernel<8, true>, a, TcTile<8>::SMEM);
+    cudaError_t e = set_synth_smem<32, 1>(a);
+    if (e == cudaSuccess) e = set_synth_smem<16, 1>(a);
+    if (e == cudaSuccess) e = set_synth_smem<16, 2>(a);
+    if (e == cudaSuccess) e = set_synth_smem<8, 1>(a);
+    if (e == cudaSuccess) e = set_synth_smem<8, 2>(a);
     if (e == cudaSuccess) e = configure_tc_anal_kernel();
     return e;
 }
@@ -697,8 +715,8 @@ cudaError_t build_tc_spin_tables(Plan &p)
 // The results do not depend on how maps are grouped into calls, so the rule looks at the plan only.
 // Legendre synthesis / analysis of HEALPix plans (lmax = 2 Nside), plain kernels against these, us:
 //     lmax 128: 1 map 35 / 61, 58 / 61    4 maps 62 / 173, 62 / 64      16 maps 247 / 677, 71 / 67
-//     lmax 192: 1 map 78 / 132, 74 / 92   4 maps 151 / 404, 77 / 94     16 maps 603 / 1598, 95 / 106
-//     lmax 1024: 1 map 3435 / 4598, 2623 / 3456                         16 maps 31679 / 55869, 3039 / 4165
+//     lmax 192: 1 map 77 / 132, 73 / 87   4 maps 151 / 403, 77 / 88     16 maps 601 / 1598, 95 / 97
+//     lmax 1024: 1 map 3419 / 4599, 2322 / 3185                         16 maps 31672 / 55868, 3040 / 3861
 // so that from lmax 192 on no number of maps loses.
 bool tc_fp64_plan(const Plan &p) { return p.lmax >= 192; }
 

@@ -41,9 +41,11 @@ def rings(n, seed=1, nphi=24):
     return np.full(n, nphi, np.int64), th, rng.uniform(0, 6, n), rng.uniform(0.5, 2.0, n) / n
 
 
-# slots 1 block less one, full, one over; l ranges of a chunk edge (l - m + 1 = 32 k, +- 1); mmax < lmax
+# slots 1 block less one, full, one over; l ranges of a chunk edge (l - m + 1 = 32 k, +- 1); mmax < lmax; the
+# last two have enough blocks for the synthesis form of two CTAs per SM
 @pytest.mark.parametrize("n,L,M,nmaps", [(127, 192, 192, 1), (128, 223, 31, 4), (129, 224, 192, 5),
-                                         (257, 222, 60, 9), (40, 255, 255, 16), (130, 193, 0, 17)])
+                                         (257, 222, 60, 9), (40, 255, 255, 16), (130, 193, 0, 17),
+                                         (513, 197, 197, 1), (520, 200, 200, 7)])
 def test_legendre_steps_against_oracle(n, L, M, nmaps):
     geom = rings(n, seed=n)
     p = _plan(geom, L, M)
