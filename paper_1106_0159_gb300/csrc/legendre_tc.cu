@@ -11,10 +11,19 @@
 // of |y| over the block and all l, once per plan) and one per (m, map column)
 // for c_lm a_lm.  The products of digit pairs with i + j <= 7 are summed by
 // tcgen05.mma, one accumulator block per class i + j, so every block adds
-// numbers of one scale: class 0 stays below 2^12 l terms (2^23 at lmax 4096),
-// and the sums are exact in FP32.  (The tensor core aligns a small addend to
-// the accumulator and truncates it, so classes must not share one.)  The
-// epilogue adds the classes as integers and rounds once to FP64.  Eight digits
+// numbers of one scale.  (The tensor core aligns a small addend to the
+// accumulator and truncates it, so classes must not share one.)
+//
+// The sums are exact in FP32 for any operands, by carries (carry_classes below).  A class k >= 1 grows
+// by at most k 2^14 per l term (|d_0| <= 64, |d_s| <= 128), so that 146 terms of one parity keep even
+// class 7 below 2^24; digits need not look random (on the equator y_l = -y_(l-2), a zonal source there
+// makes c_l a_l constant too, and class 5 reached 3.5 times 2^24 at lmax 4096: Delta_0 off by 2e-11).
+// So every 9 chunks (144 terms) each class hands the multiple of 256 in its sum to the class above
+// and keeps a remainder of at most 128.  Class 0 takes the carries: it stays within half a unit of the
+// whole sum, below 2^12 per term while |y| < 2^Ey and |c a| < 2^Ea, which is 2^24 at 4096 terms; from lmax
+// 8190 on E_a is one higher for every further 8190 (tc_scale_kernel).
+//
+// The epilogue adds the classes as integers and rounds once to FP64.  Eight digits
 // and not seven: with one scale over all l, the y of a polar block (which
 // grows like sqrt(l)) against a red spectrum (which falls like 1 / l) leave the
 // low l, where the signal is, several bits below the scale; with seven digits
@@ -109,9 +118,9 @@ __device__ __forceinline__ double c_factor(const TcArgs &A, int64_t ix)
     return SPIN ? A.tab[ix].w : A.cfac[ix];
 }
 
-// E_a[m][n] with |c_lm a_lm| < 2^E_a for all l (from exponent fields, no FP64 work), and the columns
-// the digits cannot carry: a value that is not finite or subnormal, or a maximum near the ends of the
-// FP64 range.
+// E_a[m][n] with |c_lm a_lm| < 2^E_a 2^-(lmax / 8190) for all l (from exponent fields, no FP64 work), and
+// the columns the digits cannot carry: a value that is not finite or subnormal, or a maximum near the
+// ends of the FP64 range.
 template <int N, bool SPIN>
 __global__ void tc_scale_kernel(TcArgs A)
 {
@@ -153,7 +162,8 @@ __global__ void tc_scale_kernel(TcArgs A)
     __syncthreads();
     if (threadIdx.x < N) {
         const int e = s_max[threadIdx.x];
-        A.Ea[m * N + threadIdx.x] = e ? e - 2044 : TC_EZERO;
+        // L / 8190 more: |d_0| halves where a parity has over 4096 terms, so that class 0 stays below 2^24
+        A.Ea[m * N + threadIdx.x] = e ? e - 2044 + L / 8190 : TC_EZERO;
         if (e && (e < 1023 + TC_ETINY || e > 1023 + TC_EHUGE)) s_fix[threadIdx.x >> 1] = 1;
     }
     __syncthreads();
@@ -310,6 +320,66 @@ __global__ void __launch_bounds__(TC_T) tc_tables_kernel(TcArgs A, int *Ey_out, 
 }
 
 // ---------------------------------------------------------------- the synthesis kernel
+
+// Chunks between two carries: 9 x 16 terms of one parity, 144 x 7 x 2^14 + 128 < 2^24.
+constexpr int TC_CARRY = 9;
+static_assert(TC_CARRY * (TC_CH / 2) * (TC_S - 1) * (1 << 14) + 128 < (1 << 24), "class sums exact in FP32");
+
+// two FP32 operations in one instruction (they delay the FP64 chain half as often)
+__device__ __forceinline__ uint64_t f32x2(float x) { return 0x100000001ull * __float_as_uint(x); }
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// Carries between the accumulator blocks of one parity (8 blocks of N columns, the first at `acc`; this
+// warp's 32 lanes), columns below ncols: from class 7 up, a sum S = 256 q + r with |r| <= 128 keeps r and q
+// moves to the class above.  An accumulator holds S 2^-18, so q is rounded by an addition at ulp 2^-18;
+// every step is exact.  No MMA may be in flight.  What it costs are its issue slots beside the recurrence:
+// whole synthesis at lmax 4096, 16 maps 157.4 -> 158.6 ms, with plain FP32 operations 162.5, and with 4
+// columns after every chunk instead of all of them after 9 no less (162.7).
+template <int N>
+__device__ __forceinline__ void carry_classes(uint32_t acc, int ncols)
+{
+#pragma unroll 1
+    for (int c = 0; c < N && c < ncols; c += 4) {
+        uint32_t v[TC_S][4];
+#pragma unroll
+        for (int k = 0; k < TC_S; ++k)
+            asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                         : "=r"(v[k][0]), "=r"(v[k][1]), "=r"(v[k][2]), "=r"(v[k][3])
+                         : "r"(acc + (uint32_t)(k * N + c)));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int t = 0; t < 4; t += 2) {
+            uint64_t up = 0;
+#pragma unroll
+            for (int k = TC_S - 1; k >= 0; --k) {
+                uint64_t x = add2((uint64_t)v[k][t + 1] << 32 | v[k][t], up);
+                if (k) {
+                    up = add2(fma2(x, f32x2(0x1p-8f), f32x2(48.f)), f32x2(-48.f));  // |x| < 2^6: 48 + x / 256 has ulp 2^-18
+                    x = fma2(up, f32x2(-256.f), x);
+                }
+                v[k][t] = (uint32_t)x;
+                v[k][t + 1] = (uint32_t)(x >> 32);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < TC_S; ++k)
+            asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(acc + (uint32_t)(k * N + c)),
+                         "r"(v[k][0]), "r"(v[k][1]), "r"(v[k][2]), "r"(v[k][3])
+                         : "memory");
+    }
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
 
 // Warp groups per CTA (one m, 128 slots, 416 threads):
 //   recurrence warps 0-3 (recurrence_warps): thread r runs the FP64 recurrence of slot r and
@@ -468,6 +538,15 @@ __global__ void __launch_bounds__(TC_NT + 32, NC) tc_synth_kernel(TcArgs A)
             for (int i = 0; i < BV; ++i)
                 if (i * NS + sp < BTOT) ((uint4 *)b_st)[i * NS + sp] = breg[i];
             asm volatile("fence.proxy.async.shared::cta;");
+            if (q && q % TC_CARRY == 0) {
+                // carries of this parity, between the MMAs of chunk q - 1 (one stage: waited for above) and those
+                // of chunk q, which start once every split thread has arrived
+                if (W::NST == 2 && ok && !mbar_wait(&mbar[st ^ 1], (uint32_t)(((q - 1) >> 1) & 1))) ok = false;
+                ok = __all_sync(0xffffffffu, ok);  // tcgen05.ld and st are warp-wide
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                if (ok) carry_classes<N>(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(par * W::NCLS * N), 2 * A.nmaps);
+                asm volatile("tcgen05.fence::before_thread_sync;");
+            }
             mbar_arrive(&full[st]);
         }
         // the last commits cover every MMA issued: wait (bounded) before TMEM is read
