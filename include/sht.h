@@ -84,7 +84,8 @@ sht_status sht_plan_create(sht_plan_t *out, sht_grid grid, int nrings,
  *                        run on the tensor cores: both operands are cut into eight balanced base-256
  *                        digits (62 bits) in fp16, digit products are summed exactly, as integers,
  *                        and rounded once to FP64.  Values that digits cannot carry (not finite,
- *                        near the ends of the exponent range) send their columns to FP64 sums.  A
+ *                        near the upper end of the exponent range; in the analysis a ring set that
+ *                        is tiny throughout) send their columns to FP64 sums.  A
  *                        map's result does not depend on the maps beside it.  Processes up to 16
  *                        maps per pass over the recurrence.
  *   SHT_MODE_SPLIT_BF16  the precision form: the same Legendre steps whatever lmax, and the ring

@@ -495,9 +495,10 @@ __global__ void reduce_blocks_kernel(const double2 *__restrict__ partial, const 
 // ---------------------------------------------------------------- columns left by the tensor-core kernels
 //
 // The tensor-core kernels cut their operands into digits below one exponent, which cannot carry a
-// value that is not finite, subnormal or near the ends of the FP64 range.  They mark such (m, map)
-// columns in fix[m][16], and these kernels redo them with the sums above; without marks (every
-// ordinary input) each CTA reads its 16 marks and ends.
+// value that is not finite or a column near the upper end of the FP64 range (analysis: the lower end
+// too).  They mark such (m, map) columns in fix[m][16], and these kernels redo them with the sums
+// above, one CTA per m (slow: every mark must be rare); without marks (every ordinary input) each
+// CTA reads its 16 marks and ends.
 
 __global__ void __launch_bounds__(SYN_T) legendre_synth_fix_kernel(SynArgs A, const int *__restrict__ fix, int nmaps)
 {

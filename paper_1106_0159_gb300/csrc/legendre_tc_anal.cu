@@ -253,8 +253,9 @@ __global__ void __launch_bounds__(TA_NT, 1) tc_anal_kernel(TcArgs A)
                     mx = max(mx, ex);
                     odd |= ex == 0 && (((uint32_t)__double2hiint(v) << 1) | (uint32_t)__double2loint(v)) != 0u;
                 }
+                if (odd) mx = max(mx, 1);  // subnormal values mark a row that holds nothing larger
                 if (mx) atomicMax(&sEx[row], mx);
-                if (odd || mx > TC_EHUGE) A.fix[m * 16 + (lane >> 1)] = 1;
+                if (mx > TC_EHUGE) A.fix[m * 16 + (lane >> 1)] = 1;
             }
             bar_sync(BAR_STAGED, 2 * TC_T + TA_NEPI);  // row exponents complete
             const int e = sEx[row];

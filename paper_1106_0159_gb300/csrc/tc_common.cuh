@@ -24,8 +24,15 @@ constexpr int TC_B = 62;                 // bits kept below 2^E
 constexpr int TC_CH = 32;                // l per chunk: 16 even + 16 odd l - m
 constexpr long long WAIT_POLLS = 1ll << 26;
 constexpr int TC_EZERO = 3000;           // scale exponent of an all-zero column or row: every digit 0
-constexpr int TC_ETINY = 100, TC_EHUGE = 1990;  // a column whose maximum has a biased exponent outside
-                                         // these is left to the plain FP64 sums
+constexpr int TC_ETINY = 100, TC_EHUGE = 1990;  // a column whose maximum has a biased exponent above EHUGE
+                                         // (analysis: or below ETINY) is left to the plain FP64 sums
+
+// exponent field of v, 1 if v is a nonzero subnormal (0 for zero only)
+__device__ __forceinline__ int dexp_nonzero(double v)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(v) << 1, lo = (uint32_t)__double2loint(v);
+    return max((int)(hi >> 21), (hi | lo) != 0u ? 1 : 0);
+}
 
 // v 2^(B - E) truncated to an integer F, plus 128 in every 8-bit field: byte s (from the top) of
 // the result is d_s + 128.  Integer pipe only (a conversion would take an FP64 issue slot).
@@ -70,7 +77,9 @@ __device__ __forceinline__ void digit_pairs(uint2 a, uint2 b, uint32_t out[TC_S]
 __device__ __forceinline__ int class_sum(float acc) { return __float2int_rn(acc * 262144.0f); }
 
 // T 2^e rounded to nearest (ties away), integer pipe only and without branches, so that several of
-// them overlap; a result below the normal range is 0 (the exponents used here cannot exceed it)
+// them overlap; a result below the normal range is 0, or with SUB a subnormal (the exponents used here
+// cannot exceed the range)
+template <bool SUB = false>
 __device__ __forceinline__ double i64_to_double(long long T, int e)
 {
     const long long s = T >> 63;
@@ -78,8 +87,15 @@ __device__ __forceinline__ double i64_to_double(long long T, int e)
     const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a;
     const int lz = ah ? __clz((int)ah) : 32 + __clz((int)al);
     a <<= (lz & 63);                                       // leading one at bit 63
-    const unsigned long long mant = (a >> 11) + ((a >> 10) & 1ull);  // may carry into 2^53
     const int ex = 1023 + 63 - lz + e;                     // biased exponent of the leading one
+    if constexpr (SUB) {
+        const int d = max(1 - ex, 0);                      // bits lost below the normal range
+        a >>= 10 + min(d, 53);
+        const unsigned long long mant = (a >> 1) + (a & 1ull);
+        const unsigned long long r = (((unsigned long long)(uint32_t)(ex + d - 1) << 52) + mant) | ((unsigned long long)s << 63);
+        return __longlong_as_double((long long)((T != 0 && d <= 53) ? r : 0ull));
+    }
+    const unsigned long long mant = (a >> 11) + ((a >> 10) & 1ull);  // may carry into 2^53
     const unsigned long long r = (((unsigned long long)(uint32_t)(ex - 1) << 52) + mant) | ((unsigned long long)s << 63);
     return __longlong_as_double((long long)((T != 0 && ex > 0) ? r : 0ull));
 }
@@ -92,7 +108,7 @@ __device__ __forceinline__ double pair_to_double(long long hi, long long lo, int
     const long long r = lo & 0xFFFFFFFFll;
     const long long m = hi < 0 ? -hi : hi;
     const int sh = m < (1ll << 30) ? 32 : m < (1ll << 38) ? 24 : m < (1ll << 44) ? 18 : 11;
-    return i64_to_double(hi * (1ll << sh) + (r >> (32 - sh)), e - sh);
+    return i64_to_double<true>(hi * (1ll << sh) + (r >> (32 - sh)), e - sh);
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }

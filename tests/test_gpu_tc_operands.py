@@ -57,3 +57,49 @@ def test_coherent_operands(L, ms):
         w = np.zeros((1, oracle.nalm(L, W)), np.complex128)
         w[0, :a.shape[1]] = a[0]
         assert np.array_equal(host(_plan(RINGS, L, W).legendre_synth(dev(w)))[0, :, :M + 1], d[0])
+
+
+def test_subnormal_values_beside_ordinary_ones():
+    """Coefficients of a strongly smoothed spectrum pass through the subnormal range.  Beside a column's
+    ordinary values they are below 2^-99 of its scale: the results are those with zeros there, bit for bit,
+    which the plain sums are not."""
+    L, n = 260, 140
+    rng = np.random.default_rng(5)
+    geom = (np.full(n, 8, np.int64), np.sort(rng.uniform(0.2, 2.9, n)), np.zeros(n), np.ones(n))
+    p = _plan(geom, L)
+    lv, mv = inputs.lm_arrays(L, L)
+    a = inputs.uniform_alm(L, L, seed=6, nmaps=6) * np.exp(-0.5 * (lv * 0.15) ** 2)
+    tiny = (np.abs(a.real) < 2.0 ** -1022) & (np.abs(a.imag) < 2.0 ** -1022)
+    assert (tiny & (a != 0.0) & (mv < 200)).any(axis=1).all()
+    z = np.where(tiny, 0.0, a)
+    d, e = host(p.legendre_synth(dev(a))), host(p.legendre_synth(dev(z)))
+    assert np.array_equal(d[:, :, :200], e[:, :, :200])
+    t = inputs.uniform_alm(L, L, seed=8, nmaps=6).reshape(3, 2, -1)
+    t[:, :, lv == 255] = 0.0
+    w = host(p.alm2map_spin(dev(t)))
+    t[:, :, (lv == 255) & (mv < 250)] = 1e-310 * (1.0 + 1j)
+    assert np.array_equal(host(p.alm2map_spin(dev(t))), w)
+    x = inputs.random_delta(n, L, seed=7, nmaps=6)
+    x[:, ::7] = 0.0
+    b = host(p.legendre_anal(dev(x)))
+    x[:, ::7, 1:] = 3e-309 * (1.0 - 1j)
+    assert np.array_equal(host(p.legendre_anal(dev(x))), b)
+    assert p.device_status() == 0
+
+
+@pytest.mark.parametrize("scale", [2.0 ** -950, 2.0 ** -1010, 2.0 ** -1030])
+def test_columns_near_the_lower_end_of_the_range(scale):
+    """Coefficients that are all tiny, some or all of them subnormal: the FP64 bar on Delta, plus for results
+    below the normal range one rounding to a multiple of 2^-1074 and that of each input (the scaled
+    oracle's inputs are the stored ones, so only the result's counts)."""
+    L, M, n = 200, 30, 60
+    rng = np.random.default_rng(15)
+    geom = (np.full(n, 8, np.int64), np.sort(rng.uniform(0.2, 2.9, n)), np.zeros(n), np.ones(n))
+    p = _plan(geom, L, M)
+    a = inputs.uniform_alm(L, M, seed=16, nmaps=2) * scale
+    d = host(p.legendre_synth(dev(a)))
+    for g in (0, 1):
+        ref = oracle.delta_synth(geom, a[g] * 2.0 ** 900, L, M)
+        bar = 1e-11 * np.sqrt(np.mean(np.abs(ref) ** 2)) + 2.0 ** (900 - 1074)
+        got = d[g] * 2.0 ** 900
+        assert np.max(np.abs(got.real - ref.real)) <= bar and np.max(np.abs(got.imag - ref.imag)) <= bar
