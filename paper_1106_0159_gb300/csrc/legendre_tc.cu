@@ -128,6 +128,7 @@ __global__ void tc_scale_kernel(TcArgs A)
     __shared__ int s_max[N];
     __shared__ int s_fix[N / 2];
     const int m = A.m0 + blockIdx.x;
+    if (A.mflag && !A.mflag[m]) return;  // an m this plan does not compute: nothing reads its digits
     const int L = A.lmax;
     const int64_t base = (int64_t)m * (2 * L + 3 - m) / 2;
     if (threadIdx.x < N) s_max[threadIdx.x] = 0;
@@ -187,6 +188,7 @@ __global__ void tc_split_b_kernel(TcArgs A)
 {
     const int64_t chunk = A.chunk0 + blockIdx.x;
     const int m = A.chunk_m[chunk];
+    if (A.mflag && !A.mflag[m]) return;
     const int c = (int)(chunk - A.chunk_base[m]);
     const int L = A.lmax;
     const int64_t base = (int64_t)m * (2 * L + 3 - m) / 2;

@@ -103,3 +103,22 @@ def test_columns_near_the_lower_end_of_the_range(scale):
         bar = 1e-11 * np.sqrt(np.mean(np.abs(ref) ** 2)) + 2.0 ** (900 - 1074)
         got = d[g] * 2.0 ** 900
         assert np.max(np.abs(got.real - ref.real)) <= bar and np.max(np.abs(got.imag - ref.imag)) <= bar
+
+
+def test_an_m_list_cuts_the_coefficients_of_its_m_only():
+    """A plan with an m list (one rank's share) reads and cuts no other m's coefficients: the rest of its scratch
+    stays as it was."""
+    L = 500
+    p = _plan((np.full(8, 16, np.int64), np.linspace(0.4, 2.7, 8), np.zeros(8), np.ones(8)), L)
+    a = dev(inputs.uniform_alm(L, L, seed=31))
+    s = p.scratch(1)
+    full = p.alm2map_ws(a, s).clone()
+    p.set_mlist([0, 3])
+    s.fill_(0xA5)
+    got = p.alm2map_ws(a, s)
+    assert float((s == 0xA5).double().mean()) > 0.9
+    b = a.clone()
+    b[:, oracle.alm_index(L, 4, 4):] = 0.0
+    b[:, oracle.alm_index(L, 1, 1):oracle.alm_index(L, 3, 3)] = 0.0
+    p.set_mlist()
+    assert torch.equal(p.alm2map(b), got) and not torch.equal(got, full)
