@@ -98,7 +98,9 @@ sht_status sht_plan_create(sht_plan_t *out, sht_grid grid, int nrings,
  *                        Nside >~ 7000) returns SHT_EUNSUPPORTED and stays in its old mode.
  * The creation of a plan with lmax >= 192, or else the first switch to SHT_MODE_SPLIT_BF16, runs
  * one FP64 pass of the recurrence to measure the scale of its values per (m, block of 128 ring
- * slots) (synchronous; about the cost of one single-map synthesis).  SHT_EINVAL for an unknown mode.
+ * slots) (synchronous; about the cost of one single-map synthesis).  These tables take 20 bytes per m
+ * and ring slot; where there is no device memory for them, the plan is created all the same and its FP64
+ * mode runs the plain FP64 kernels.  SHT_EINVAL for an unknown mode.
  */
 typedef enum { SHT_MODE_FP64 = 0, SHT_MODE_SPLIT_BF16 = 1 } sht_mode;
 sht_status sht_plan_set_mode(sht_plan_t plan, int mode);
@@ -195,7 +197,8 @@ sht_status sht_map2alm_ws(sht_plan_t plan, const double *map, void *alm, int nma
  * from lmax 192 on; no Reinsch form on polar rings.
  * The first spin call on a plan builds its spin recurrence tables on the host and copies them to
  * the device (synchronous; 32 nalm bytes, from lmax 192 on with the tables of the tensor-core
- * kernels): make it before any stream capture.  Scratch grows on
+ * kernels, 40 bytes per m and ring slot, without which the plain kernels run): make it before any
+ * stream capture.  Scratch grows on
  * demand to sht_spin_workspace_bytes(plan, nmaps).  Stream ordering and errors as sht_alm2map.
  */
 sht_status sht_alm2map_spin(sht_plan_t plan, int spin, const void *alm, double *map, int nmaps, void *stream);

@@ -121,7 +121,9 @@ struct Plan {
     int *d_sp_Ey = nullptr;             // spin 2 on the tensor cores: as d_tc_Ey, d_tc_ck_*, for the signs + and -
     double2 *d_sp_ck_y = nullptr;
     int *d_sp_ck_k = nullptr;
-    bool tc64 = false;                  // the FP64 mode's Legendre steps take the tensor-core kernels (tc_fp64_plan)
+    bool tc64 = false;                  // the FP64 mode's Legendre steps take the tensor-core kernels (tc_fp64_plan,
+                                        // and there was memory for their tables)
+    bool spin_plain = false;            // there was no memory for the spin tables of the tensor-core kernels
     bool split_ready = false;           // the plan has been switched to the precision form once
     bool polar_first_slot = false;      // slot 0 runs the Reinsch form (sin(theta) < 0.03)
 

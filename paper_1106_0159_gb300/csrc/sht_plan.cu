@@ -685,9 +685,14 @@ sht_status sht_plan_create(sht_plan_t *out, sht_grid grid, int nrings, const int
         e = sht::build_fft_tables(p);
     }
     if (e == cudaSuccess && sht::tc_fp64_plan(p)) {
+        // without memory for these tables the plan runs its Legendre steps on the plain FP64 kernels
         where = "tensor-core tables";
         e = sht::build_tc_tables(p);
         p.tc64 = e == cudaSuccess;
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            e = cudaSuccess;
+        }
     }
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -791,6 +796,8 @@ sht_status sht_map2alm(sht_plan_t plan, const double *map, void *alm, int nmaps,
 }
 
 // Spin-2 transforms (see the header and spin.cu).
+static bool spin_tc(const Plan &p) { return sht::tc_fp64_plan(p) && !p.spin_plain; }
+
 static sht_status spin_prepare(Plan &p, int spin)
 {
     if (p.n_mlist > 0) {
@@ -802,7 +809,14 @@ static sht_status spin_prepare(Plan &p, int spin)
         return SHT_EUNSUPPORTED;
     }
     cudaError_t e = sht::build_spin_tables(p);
-    if (e == cudaSuccess && sht::tc_fp64_plan(p)) e = sht::build_tc_spin_tables(p);
+    if (e == cudaSuccess && spin_tc(p)) {
+        e = sht::build_tc_spin_tables(p);
+        if (e == cudaErrorMemoryAllocation) {  // no room for them: the plain kernels, from now on
+            cudaGetLastError();
+            p.spin_plain = true;
+            e = cudaSuccess;
+        }
+    }
     if (e != cudaSuccess) return cuda_fail(p, e, "spin tables");
     return SHT_OK;
 }
@@ -813,9 +827,9 @@ size_t sht_spin_workspace_bytes(sht_plan_t plan, int nmaps)
     const Plan &p = plan->p;
     return align256(delta_bytes(p, 2 * nmaps)) +
            std::max(align256(sht::ring_scratch_bytes(p)),
-                    sht::tc_fp64_plan(p) ? std::max(align256(sht::tc_workspace_bytes(p, 2 * nmaps)),
-                                                    align256(sht::tc_anal_partial_bytes(p, 2 * nmaps)))
-                                         : align256(sht::spin_partial_bytes(p, std::min(nmaps, 2))));
+                    spin_tc(p) ? std::max(align256(sht::tc_workspace_bytes(p, 2 * nmaps)),
+                                          align256(sht::tc_anal_partial_bytes(p, 2 * nmaps)))
+                               : align256(sht::spin_partial_bytes(p, std::min(nmaps, 2))));
 }
 
 sht_status sht_alm2map_spin(sht_plan_t plan, int spin, const void *alm, double *map, int nmaps, void *stream)
@@ -833,7 +847,7 @@ sht_status sht_alm2map_spin(sht_plan_t plan, int spin, const void *alm, double *
     {
         StageScope sc(p, SHT_STAGE_LEGENDRE_SYNTH, s);
         int n = 0;
-        cudaError_t e = sht::tc_fp64_plan(p)
+        cudaError_t e = spin_tc(p)
                             ? sht::launch_spin_synth_tc(p, (const double2 *)alm, delta, scratch,
                                                         sht::tc_workspace_bytes(p, 2 * nmaps), nmaps, s, &n)
                             : sht::launch_spin_synth(p, (const double2 *)alm, delta, nmaps, s, &n);
@@ -860,8 +874,8 @@ sht_status sht_map2alm_spin(sht_plan_t plan, int spin, const double *map, void *
     if (st != SHT_OK) return st;
     StageScope sc(p, SHT_STAGE_LEGENDRE_ANAL, s);
     int n = 0;
-    cudaError_t e = sht::tc_fp64_plan(p) ? sht::launch_spin_anal_tc(p, delta, (double2 *)alm, scratch, nmaps, s, &n)
-                                         : sht::launch_spin_anal(p, delta, (double2 *)alm, scratch, nmaps, s, &n);
+    cudaError_t e = spin_tc(p) ? sht::launch_spin_anal_tc(p, delta, (double2 *)alm, scratch, nmaps, s, &n)
+                               : sht::launch_spin_anal(p, delta, (double2 *)alm, scratch, nmaps, s, &n);
     p.launches[SHT_STAGE_LEGENDRE_ANAL] += n;
     if (e != cudaSuccess) return cuda_fail(p, e, "spin legendre_anal");
     sc.done();
