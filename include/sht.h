@@ -346,7 +346,8 @@ sht_status sht_fp64_fma_tflops(double *tflops);
  * the precision form's kernels on a SHT_MODE_SPLIT_BF16 plan), but the call
  * allocates nothing: its scratch (the Delta intermediate, then either digit
  * tiles or the ring-FFT buffers) is a 64 MiB static device array,
- * sht_noalloc_scratch_bytes(), that every GPU loading this library holds until
+ * sht_noalloc_scratch_bytes() (8 KiB more for folding short rings, which the
+ * limit below leaves out), that every GPU loading this library holds until
  * the process exits.  The tensor-core kernels of an FP64 plan take the room
  * that is left for their digit tiles, in slabs of whole m, and leave the call
  * to the plain FP64 kernels when not one m fits.  Calls whose scratch

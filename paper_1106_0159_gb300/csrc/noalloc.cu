@@ -9,7 +9,7 @@
 // __device__ array instead of the plan's workspace.  It runs the plan's own
 // arithmetic (sht_plan_set_mode), with the same kernels as sht_alm2map.
 //
-// The array is 64 MiB and exists on every GPU on which this library's module
+// The array is 64 MiB (and 8 KiB for short rings) and exists on every GPU on which this library's module
 // is loaded, for the life of the process.  Host code may not pass the
 // array's symbol to a kernel (on the host it only names a stand-in object);
 // its device address is looked up with cudaGetSymbolAddress once per device,
@@ -25,7 +25,11 @@ namespace {
 constexpr size_t NOALLOC_SCRATCH_BYTES = size_t(64) << 20;
 constexpr int NOALLOC_MAX_DEVICES = 64;
 
-__device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH_BYTES];
+// The rule for the calls that fit counts the DFT buffers only.  Folding short rings takes more than
+// those, so the array has room for it beyond the size that the rule sees.
+constexpr size_t NOALLOC_FOLD_BYTES = (3 * ((sht::RING_FOLD + 2) / 3) * sizeof(double2) + 255) & ~size_t(255);
+
+__device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH_BYTES + NOALLOC_FOLD_BYTES];
 
 std::mutex g_noalloc_mu;
 void *g_noalloc_addr[NOALLOC_MAX_DEVICES] = {};
@@ -71,7 +75,7 @@ extern "C" sht_status sht_alm2map_noalloc(sht_plan_t plan, const void *alm, doub
     const size_t tc = prec ? (size_t)p.tc_total_chunks * (std::min(nmaps, p.tune[SHT_TUNE_TC_MAPS]) > 8 ? 16384 : 8192) +
                                  (size_t)(p.mmax + 1) * 32 * sizeof(int) + 256
                            : 0;
-    const size_t need = delta + std::max(per_cta, tc);
+    const size_t need = delta + std::max((size_t)3 * p.dft_maxlen * sizeof(double2), tc);
     if (need > NOALLOC_SCRATCH_BYTES) {
         p.last_error = "sht_alm2map_noalloc: " + std::to_string(nmaps) + " map(s) need " + std::to_string(need) +
                        " bytes of scratch; the static scratch holds " + std::to_string(NOALLOC_SCRATCH_BYTES) +
@@ -79,7 +83,7 @@ extern "C" sht_status sht_alm2map_noalloc(sht_plan_t plan, const void *alm, doub
         return SHT_EINVAL;
     }
     int grid = sht::ring_grid(p);
-    const size_t fit = (NOALLOC_SCRATCH_BYTES - delta) / per_cta;
+    const size_t fit = (NOALLOC_SCRATCH_BYTES + NOALLOC_FOLD_BYTES - delta) / per_cta;  // >= 1
     if ((size_t)grid > fit) grid = (int)fit;
     void *base = nullptr;
     cudaError_t e = scratch_address(&base);

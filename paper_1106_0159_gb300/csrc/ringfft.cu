@@ -40,7 +40,7 @@ constexpr int FFT_T = RING_T;
 // for two): 1024 at 64 registers each (lmax 4096, HEALPix 2048, 16 maps: synthesis / analysis
 // 42.4 / 38.0 ms, against 46.4 / 38.8 with 512 threads at 128 registers); the FP64 ones keep 512.
 constexpr int RING_DF_WIDE_T = 1024;
-constexpr int FOLD_T = 512;  // threads (and scratch entries) that share the folding of a short ring
+constexpr int FOLD_T = RING_FOLD;
 static_assert(FOLD_T <= FFT_T && FOLD_T <= RING_DF_WIDE_T, "every ring kernel has FOLD_T threads");
 
 #include "check.cuh"
@@ -1484,6 +1484,7 @@ cudaError_t build_fft_tables(Plan &p)
     }
     p.nitems = (int)items.size();
     p.nlens = (int)p.lens.size();
+    p.dft_maxlen = maxlen;
     maxlen = std::max(maxlen, (FOLD_T + 2) / 3);  // three buffers hold FOLD_T entries
     p.fft_maxlen = maxlen;
     p.fft_tab_len = off;

@@ -22,6 +22,9 @@ cudaError_t dev_malloc(T **ptr, size_t bytes)
     return dev_malloc((void **)ptr, bytes);
 }
 
+// threads (and scratch entries) that share the folding of a short ring (ringfft.cu)
+constexpr int RING_FOLD = 512;
+
 // Runs f(0) .. f(n - 1) on the host's cores (at most 16 threads, fewer when they cannot be had); the
 // plan tables of each m are independent.  f must not throw.
 void host_parallel(int n, const std::function<void(int)> &f);
@@ -100,7 +103,9 @@ struct Plan {
     float4 *d_fft_tab_df = nullptr;     // double-float copies for the precision form (built by set_mode)
     float4 *d_phase_df = nullptr;
     int64_t fft_tab_len = 0;
-    int fft_maxlen = 0;         // per-CTA scratch length (complex entries, per buffer)
+    int fft_maxlen = 0;         // per-CTA scratch length (complex entries, per buffer): the longest DFT's, and
+                                // RING_FOLD entries in the three buffers together
+    int dft_maxlen = 0;         // the longest DFT's alone
     int *d_fft_perm = nullptr;  // spectrum positions of the shared-memory DFTs
     int ring_smem = 0;          // dynamic shared memory of the ring kernels (bytes), 0: none fit
     int ring_occ = 1;           // ring CTAs resident per SM with that shared memory
