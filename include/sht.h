@@ -104,6 +104,8 @@ sht_status sht_plan_create(sht_plan_t *out, sht_grid grid, int nrings,
  */
 typedef enum { SHT_MODE_FP64 = 0, SHT_MODE_SPLIT_BF16 = 1 } sht_mode;
 sht_status sht_plan_set_mode(sht_plan_t plan, int mode);
+/* 1 if the plan's FP64 mode runs its (scalar) Legendre steps on the tensor cores, else 0; -1 for null */
+int sht_plan_fp64_tensor(sht_plan_t plan);
 int        sht_plan_mode(sht_plan_t plan);
 
 /*
@@ -248,7 +250,8 @@ typedef enum {
     SHT_TUNE_ANAL_MAPS = 1,  /* FP64 analysis: maps per launch, 1 or 2 (default 2) */
     SHT_TUNE_ANAL_SLOTS = 2, /* FP64 analysis: ring slots per thread, 1 or 4 (default 4, or 1 below 512 slots) */
     SHT_TUNE_DF_MAPS = 3,    /* precision-form analysis: maps per launch, 4, 8 or 16 (default 8) */
-    SHT_TUNE_TC_MAPS = 4,    /* precision-form synthesis: maps per tensor-core launch, 8 or 16 (default 16) */
+    SHT_TUNE_TC_MAPS = 4,    /* tensor-core synthesis (precision form, and FP64 plans from lmax 192 on):
+                                maps per launch, 8 or 16 (default 16) */
     SHT_TUNE_PREC_ANAL = 5,  /* precision-form analysis kernel: 0 double-float FP32, 1 tensor cores (default) */
     SHT_TUNE_PREC_RING = 6,  /* precision-form ring DFTs: 1 double-float FP32 (default), 0 FP64 */
     SHT_TUNE_RING_SMEM = 7,  /* ring DFTs: 1 in shared memory where the ring fits, 0 all through the

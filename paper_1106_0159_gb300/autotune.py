@@ -1,9 +1,9 @@
 """Autotuner for a plan's launch-tuning knobs (sht_plan_set_tuning).
 
 For a key (grid, band limits, maps per call, mode, direction) it times every combination of the
-knobs that the direction and mode use, one transform each (after a warm-up), with CUDA events on
-the call's stream, keeps the fastest and caches it (in memory, and in a JSON file when a path is
-given).  Every combination gives the same synthesis results and analysis results within rounding
+knobs that the plan's direction and kernels read, one transform each (after a warm-up), with CUDA
+events on the call's stream, keeps the fastest and caches it (in memory, and in a JSON file when a
+path is given); a transform with nothing to choose is timed once, for the record.  Every combination gives the same synthesis results and analysis results within rounding
 (the FP64 ring sums change order with the slots per thread), so tuning only moves time.
 
 The timer is injectable so that the search and the cache can be tested without a GPU.
@@ -20,22 +20,27 @@ from . import sht
 ALM2MAP, MAP2ALM = "alm2map", "map2alm"
 
 
-def knobs_for(direction: str, mode: int) -> List[int]:
-    """The knobs a transform of this direction and mode reads."""
+def knobs_for(direction: str, mode: int, tensor: Optional[bool] = None) -> List[int]:
+    """The knobs a transform of this direction and mode reads.  tensor: whether an FP64 plan's Legendre
+    steps run on the tensor cores (Plan.fp64_tensor); None lists the knobs of the mode's kernels
+    without looking at a plan, the plain ones' in the precision form too."""
+    if direction not in (ALM2MAP, MAP2ALM):
+        raise ValueError("unknown direction %r" % (direction,))
+    split = mode == sht.MODE_SPLIT_BF16
     if direction == ALM2MAP:
-        # precision form: tensor-core groups, and the FP64 kernel on polar slot blocks
-        return [sht.TUNE_TC_MAPS, sht.TUNE_SYNTH_MAPS] if mode == sht.MODE_SPLIT_BF16 else [sht.TUNE_SYNTH_MAPS]
-    if direction == MAP2ALM:
-        # precision form: tensor-core or double-float kernel (the latter's maps per launch)
-        return [sht.TUNE_PREC_ANAL, sht.TUNE_DF_MAPS] if mode == sht.MODE_SPLIT_BF16 else [sht.TUNE_ANAL_MAPS, sht.TUNE_ANAL_SLOTS]
-    raise ValueError("unknown direction %r" % (direction,))
+        if tensor is None:
+            return [sht.TUNE_TC_MAPS, sht.TUNE_SYNTH_MAPS] if split else [sht.TUNE_SYNTH_MAPS]
+        return [sht.TUNE_TC_MAPS] if split or tensor else [sht.TUNE_SYNTH_MAPS]
+    if split:  # tensor-core or double-float kernel (the latter's maps per launch)
+        return [sht.TUNE_PREC_ANAL, sht.TUNE_DF_MAPS]
+    return [] if tensor else [sht.TUNE_ANAL_MAPS, sht.TUNE_ANAL_SLOTS]
 
 
-def candidates(direction: str, mode: int, nmaps: int) -> List[Dict[int, int]]:
+def candidates(direction: str, mode: int, nmaps: int, tensor: Optional[bool] = None) -> List[Dict[int, int]]:
     """Knob settings worth timing: values above the call's map count act like the map count, so
     only the smallest of those is kept; the double-float maps per launch matter only when the
     double-float analysis kernel is chosen."""
-    ks = knobs_for(direction, mode)
+    ks = knobs_for(direction, mode, tensor)
     per_knob = []
     for k in ks:
         vals = sorted(sht.TUNE_VALUES[k])
@@ -112,15 +117,17 @@ class Autotuner:
         if not force and key in self.cache:
             self.apply(plan, nmaps, direction)
             return self.cache[key]
-        ks = knobs_for(direction, plan.mode)
+        tensor = bool(getattr(plan, "fp64_tensor", False))
+        ks = knobs_for(direction, plan.mode, tensor)
         default = {k: plan.tuning(k) for k in ks}
         tried: List[Tuple[Dict[int, int], float]] = []
-        for cand in candidates(direction, plan.mode, nmaps):
+        cands = candidates(direction, plan.mode, nmaps, tensor)
+        for cand in cands if len(cands) > 1 else []:  # one candidate: nothing to choose
             self._apply(plan, cand)
             tried.append((cand, float(self.timer(plan, direction, src, dst))))
         self._apply(plan, default)
         default_ms = float(self.timer(plan, direction, src, dst))
-        best, best_ms = min(tried, key=lambda t: t[1])
+        best, best_ms = min(tried + [(default, default_ms)], key=lambda t: t[1])
         if default_ms <= best_ms:
             best, best_ms = default, default_ms
         self._apply(plan, best)
@@ -175,6 +182,9 @@ def tune_batch(batch, direction: str, timer: Callable = batch_timer, cache: Opti
             batch.set_tuning(int(k), int(v))
         return cache[key]
     ks = batch_knobs(direction)
+    if hasattr(batch, "tiles") and batch.tiles(0) == 0:
+        # every plan runs its Legendre steps on the tensor cores, beside the queue
+        ks = [sht.BATCH_RING_CTAS]
     cur = {k: batch.tuning(k) for k in ks}
     default_ms = float(timer(batch))
     best_ms = default_ms

@@ -509,6 +509,7 @@ sht_status sht_plan_set_mode(sht_plan_t plan, int mode)
 }
 
 int sht_plan_mode(sht_plan_t plan) { return plan ? plan->p.mode : -1; }
+int sht_plan_fp64_tensor(sht_plan_t plan) { return plan ? (int)plan->p.tc64 : -1; }
 
 sht_status sht_plan_device_status(sht_plan_t plan, int *status, int clear)
 {

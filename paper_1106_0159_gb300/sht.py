@@ -34,7 +34,7 @@ EXPORTS = (
     "sht_workspace_bytes", "sht_geom_healpix", "sht_geom_gauss_legendre",
     "sht_status_string", "sht_plan_last_error", "sht_plan_set_stage_timing", "sht_plan_stage_times",
     "sht_fp64_fma_tflops", "sht_alm2map_noalloc", "sht_noalloc_scratch_bytes",
-    "sht_plan_set_mode", "sht_plan_mode", "sht_plan_device_status", "sht_plan_reserve",
+    "sht_plan_set_mode", "sht_plan_mode", "sht_plan_fp64_tensor", "sht_plan_device_status", "sht_plan_reserve",
     "sht_plan_set_tuning", "sht_plan_tuning", "sht_plan_selftest_timeout", "sht_alm2map_ws", "sht_map2alm_ws",
     "sht_plan_live_steps", "sht_alm2map_spin", "sht_map2alm_spin", "sht_spin_workspace_bytes",
     "sht_plan_set_mlist", "sht_debug_fail_allocations_after",
@@ -99,6 +99,7 @@ def load():
             "sht_noalloc_scratch_bytes": (S, []),
             "sht_plan_set_mode": (I, [P, I]),
             "sht_plan_mode": (I, [P]),
+            "sht_plan_fp64_tensor": (I, [P]),
             "sht_plan_live_steps": (I, [P, P, P]),
             "sht_alm2map_spin": (I, [P, I, P, P, I, P]),
             "sht_map2alm_spin": (I, [P, I, P, P, I, P]),
@@ -241,6 +242,11 @@ class Plan:
     @property
     def mode(self) -> int:
         return int(load().sht_plan_mode(self._h))
+
+    @property
+    def fp64_tensor(self) -> bool:
+        """Whether the FP64 mode runs its Legendre steps on the tensor cores (from lmax 192 on)."""
+        return load().sht_plan_fp64_tensor(self._h) == 1
 
     def device_status(self, clear: bool = True) -> int:
         """The plan's device status word (bit 0: a bounded device wait gave up); waits for the device."""
@@ -434,7 +440,8 @@ BATCH_ALM2MAP, BATCH_MAP2ALM = 0, 1
 
 
 class Batch:
-    """Many transforms of one direction as one persistent launch per stage (sht_batch_*).
+    """Many transforms of one direction as one persistent launch per stage (sht_batch_*); the Legendre
+    steps of plans with fp64_tensor are one launch per plan instead.
 
     jobs: list of (plan, src, dst) with the tensors of plan.alm2map / plan.map2alm (device,
     contiguous, kept by the batch: write new inputs into src in place between runs)."""
