@@ -739,10 +739,10 @@ def o1_leg(lmax=64, nside=32):
 
 def batch_leg(a, rep, local_rank):
     """The batched form: `--batch-maps` maps, each with lmax drawn from {512, 1024, 2048} (HEALPix
-    nside = lmax/2) and alm2map or map2alm with probability 1/2.  Plain FP64: one persistent launch
-    per stage and direction (tiles of all plans from one longest-first queue; the two directions on
-    two streams of one CUDA graph), batch knobs autotuned first.  Beside it, and for the precision
-    form, a CUDA graph of one library call per (lmax, direction) with the per-call knobs autotuned.
+    nside = lmax/2) and alm2map or map2alm with probability 1/2.  FP64: the library's batched form per
+    direction (at these sizes one Legendre launch per plan, and one persistent ring launch over the
+    units of all plans, longest first; the two directions on two streams of one CUDA graph), batch
+    knobs autotuned first.  Beside it, and for the precision form, a CUDA graph of one library call per (lmax, direction) with the per-call knobs autotuned.
     Replays and eager calls are timed with CUDA events, `--steps` times each after one warm-up."""
     import functools
 
@@ -817,8 +817,8 @@ def batch_leg(a, rep, local_rank):
                          for j, r in zip(jobs, recs)}}
         del b
         if mode == sht.MODE_FP64:
-            # the persistent form: one launch per stage and direction, tiles of every plan from one
-            # queue, longest first; the batch knobs (tile shapes, persistent grids) tuned first
+            # the batched form: one persistent ring launch per direction over the units of every plan,
+            # longest first, beside one tensor-core Legendre launch per plan; its knobs tuned first
             pb = batch.PersistentBatch(jobs)
             t0 = time.perf_counter()
             cache = {}
@@ -833,8 +833,8 @@ def batch_leg(a, rep, local_rank):
                         "persistent_tuned": {d: {"knobs": r["knobs"], "ms": r["ms"], "default_ms": r["default_ms"]}
                                              for d, r in ptuned.items()},
                         "tiles": {d: {"legendre": bb.tiles(0), "ring": bb.tiles(1)} for d, bb in pb.batches},
-                        "form": "persistent: one launch per stage and direction, longest-first tile queue, both "
-                                "directions on two streams of one CUDA graph"})
+                        "form": "batched: one tensor-core Legendre launch per plan and one persistent longest-first "
+                                "ring launch per direction, both directions on two streams of one CUDA graph"})
             pb.close()
         else:
             res.update({"maps_per_s": res["graph_of_calls_maps_per_s"],

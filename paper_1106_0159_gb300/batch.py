@@ -1,11 +1,14 @@
 """A fixed batch of transforms (several plans, band limits, directions and map counts) run as
 one CUDA graph.
 
-Two forms.  PersistentBatch (plain FP64 plans): every transform of one direction is one library
+Two forms.  PersistentBatch (plans in the FP64 mode): every transform of one direction is one library
 batch (sht_batch_*): one persistent launch per stage whose CTAs take (transform, map group, m,
 slot block) tiles of all plans from one device queue, longest l-range first, and (transform, ring
 pair, map) DFT units longest first; the alm2map batch and the map2alm batch run on two streams
 inside one graph, so the ring stage of one direction overlaps the Legendre stage of the other.
+Plans whose Legendre steps run on the tensor cores (from lmax 192 on) have only their ring units in
+the queue: their Legendre steps are one launch per plan, one plan after another, so that a batch of
+such plans is no faster than a GraphBatch of them.
 GraphBatch (any mode): one library call per job, as below.
 
 Each job is one library call (sht_alm2map or sht_map2alm) with device buffers that stay put.
@@ -116,7 +119,7 @@ class GraphBatch:
 
 
 class PersistentBatch:
-    """All jobs of one direction in one sht batch (plain FP64 plans); the two directions on two
+    """All jobs of one direction in one sht batch (plans in the FP64 mode); the two directions on two
     streams of one CUDA graph.  Same interface as GraphBatch."""
 
     def __init__(self, jobs: List[Job], nstreams: int = 2):
