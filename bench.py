@@ -287,6 +287,22 @@ def traffic_from_profiles(kernel_key):
     return rec.get("bytes_per_launch")
 
 
+def plain_legendre_figures(stages, steps, nmaps, triangle, fp64_peak_tflops, live_share):
+    """Roofline of the plain FP64 Legendre kernels (plans below lmax 192), from the per-stage CUDA-event
+    times {name: (ms over `steps` round trips, launches)}: the longer of the two stages, nominal 3 flops
+    per (l, m, ring-pair) step of `triangle` for each launch's recurrence and 4 per step and map for the
+    sums; steps whose lambda is dropped are skipped, so the fraction can exceed 1."""
+    key = max(("legendre_synth", "legendre_anal"), key=lambda k: stages[k][0])
+    ms, launches = stages[key]
+    achieved = triangle * (3.0 * launches + 4.0 * nmaps * steps) / (ms * 1e-3) / 1e12
+    return {"bound": "alu", "pipe": "fp64", "kernel": key + "_kernel", "achieved": achieved, "peak": fp64_peak_tflops,
+            "unit": "TFLOP/s", "frac": achieved / fp64_peak_tflops, "traffic": traffic_from_profiles(key + "_kernel"),
+            "peak_source": "derived: 2 FP64 FMA/clk/SM x SMs x maximum SM clock x 2 flop",
+            "work": "per (l, m, ring-pair) step of the full triangle 3 flops a launch (recurrence) and 4 a map (sums)",
+            "time": "the Legendre stage (all its launches)", "live_share": live_share,
+            "frac_of_executed": achieved / fp64_peak_tflops * live_share}
+
+
 def ring_stage_figures(stages, steps, nmaps, nrings, mmax, npix, nphi, hbm_peak_gbs, fp64_peak_tflops,
                        double_float=False, traffic_lookup=None):
     """Ring stages (eqs. Delta2map and almfftdef), one launch per call and direction, from the
@@ -413,11 +429,13 @@ def ours_arm(a, rank, world, local_rank):
 
     def tc_roofline(run, steps):
         # the tensor-core kernels, each timed alone by its own CUDA events on the call's stream
-        # (stage ids tc_synth_kernel / tc_anal_kernel: no digit split, no block reduction); both modes
-        # run them at this size
+        # (stage ids tc_synth_kernel / tc_anal_kernel: no digit split, no block reduction); below lmax
+        # 192 the FP64 mode runs the plain kernels instead
         st = run["stages"]
         ka_ms, ka_n = st["tc_anal_kernel"]
         ks_ms, ks_n = st["tc_synth_kernel"]
+        if ka_n == 0 and ks_n == 0:
+            return plain_legendre_figures(st, steps, B, S, peak_tf, live_share)
         anal = ka_ms >= ks_ms
         ms, nl = (ka_ms, ka_n) if anal else (ks_ms, ks_n)
         key = "tc_anal_kernel" if anal else "tc_synth_kernel"
@@ -742,7 +760,8 @@ def batch_leg(a, rep, local_rank):
     nside = lmax/2) and alm2map or map2alm with probability 1/2.  FP64: the library's batched form per
     direction (at these sizes one Legendre launch per plan, and one persistent ring launch over the
     units of all plans, longest first; the two directions on two streams of one CUDA graph), batch
-    knobs autotuned first.  Beside it, and for the precision form, a CUDA graph of one library call per (lmax, direction) with the per-call knobs autotuned.
+    knobs autotuned first.  Beside it, and for the precision form, a CUDA graph of one library call
+    per (lmax, direction) with the per-call knobs autotuned.
     Replays and eager calls are timed with CUDA events, `--steps` times each after one warm-up."""
     import functools
 
