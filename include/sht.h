@@ -79,15 +79,22 @@ sht_status sht_plan_create(sht_plan_t *out, sht_grid grid, int nrings,
 
 /*
  * Arithmetic of the transforms:
- *   SHT_MODE_FP64        (default) every step to FP64 rounding.  From lmax 192 on the sums of
- *                        eq. (matrix_vec), over l in the synthesis and over rings in the analysis,
- *                        run on the tensor cores: both operands are cut into eight balanced base-256
- *                        digits (62 bits) in fp16, digit products are summed exactly, as integers,
- *                        and rounded once to FP64.  Values that digits cannot carry (not finite,
- *                        near the upper end of the exponent range; in the analysis a ring set that
- *                        is tiny throughout) send their columns to FP64 sums.  A
- *                        map's result does not depend on the maps beside it.  Processes up to 16
- *                        maps per pass over the recurrence.
+ *   SHT_MODE_FP64        (default) FP64 arithmetic.  From lmax 192 on the sums of eq. (matrix_vec),
+ *                        over l in the synthesis and over rings in the analysis, run on the tensor
+ *                        cores: both operands are cut into eight balanced base-256 digits in fp16,
+ *                        digit products are summed exactly, as integers, and rounded once to FP64.
+ *                        The digits hold 62 bits below one power of two per m and ring (lambda over
+ *                        all l), per m and map (the coefficients c_lm a_lm; 61 bits from lmax 8190
+ *                        on, 60 from 16380) and per m, map and 128 ring slots (the ring sums, each
+ *                        weighted by the largest lambda of its slot).  A term is off by at most
+ *                        2^-56 of the largest product such a set could form, where an FP64 product is
+ *                        off by 2^-53 of itself: errors are bounded against the sum's largest terms,
+ *                        not against each value that lies far below the others of its set (more than
+ *                        2^9 for a coefficient: high l of a steep spectrum).
+ *                        Values that digits cannot carry (not finite, near the upper end of the
+ *                        exponent range; in the analysis a ring set that is tiny throughout) send
+ *                        their columns to FP64 sums.  A map's result does not depend on the maps
+ *                        beside it.  Processes up to 16 maps per pass over the recurrence.
  *   SHT_MODE_SPLIT_BF16  the precision form: the same Legendre steps whatever lmax, and the ring
  *                        DFTs in double-float on the FP32 pipe.
  *                        SHT_TUNE_PREC_ANAL and SHT_TUNE_PREC_RING select other kernels.  Relative

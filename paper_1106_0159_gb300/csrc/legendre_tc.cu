@@ -7,9 +7,8 @@
 // E (even) and O (odd) so that Delta_N = E + O, Delta_S = E - O.
 //
 // Both operands are cut into eight base-256 digits (tc_common.cuh), with one
-// scale exponent per (m, slot block) for y = lambda / c (the measured maximum
-// of |y| over the block and all l, once per plan) and one per (m, map column)
-// for c_lm a_lm.  The products of digit pairs with i + j <= 7 are summed by
+// scale exponent per (m, slot) for y = lambda / c (the measured maximum of |y|
+// over all l, once per plan) and one per (m, map column) for c_lm a_lm.  The products of digit pairs with i + j <= 7 are summed by
 // tcgen05.mma, one accumulator block per class i + j, so every block adds
 // numbers of one scale.  (The tensor core aligns a small addend to the
 // accumulator and truncates it, so classes must not share one.)
@@ -230,7 +229,7 @@ __global__ void tc_split_b_kernel(TcArgs A)
 // ---------------------------------------------------------------- plan tables
 
 // Per (m, slot block): E with |y| < 2^E over the kept values of the block's slots and all l (-1000
-// when every value is dropped), the first chunk of 32 l in which any slot keeps a value (every
+// when every value is dropped), how far each slot's own exponent lies below it, the first chunk of 32 l in which any slot keeps a value (every
 // earlier chunk contributes exactly zero), and the recurrence state (y1, y2, k) of every slot at the
 // start of that chunk, where the tensor-core kernels begin (at lmax 4096 on HEALPix about a quarter
 // of the steps lie before it).  Same recurrence, operation for operation, as recurrence_warps, so
@@ -303,8 +302,9 @@ __device__ __forceinline__ void tables_body(const TcArgs &A, int m, int blk, int
         if (active && live && dead) atomicMin(s_first, c);
     }
     atomicMax(s_max, active ? mx : 0);
+    __syncthreads();
     ck_y[ci] = make_double2(c1, c2);
-    ck_k[ci] = ckk;
+    ck_k[ci] = slot_state(ckk, min(*s_max - mx, 255));
 }
 
 template <bool SPIN>
@@ -512,7 +512,7 @@ __global__ void __launch_bounds__(TC_NT + 32, NC) tc_synth_kernel(TcArgs A)
     } else {
         // ------------------------------------------------ split group
         const int64_t chunk0 = A.chunk_base[m] - A.chunk0;
-        const int Ey = A.Ey[m * A.nblk + blk];
+        const int Ey = A.Ey[m * A.nblk + blk] - state_d(A.ck_k[(int64_t)(m * A.nblk + blk) * TC_T + r]);  // of this slot
         constexpr int NS = TC_NT - TC_T;                 // split threads
         constexpr int BTOT = W::B_CHUNK / 16;            // uint4 of one chunk's B tiles
         constexpr int BV = (BTOT + NS - 1) / NS;

@@ -10,8 +10,8 @@
 // the other half is computed and dropped.  One launch serves 16 maps with one pass of the FP64
 // recurrence.
 //
-// Digits (tc_common.cuh): eight of y, with the plan's exponent per (m, block), and eight of X, with
-// an exponent per (m, block, row) measured in the CTA.  An MMA of 64 rows costs as much as one of
+// Digits (tc_common.cuh): eight of y 2^d and eight of X 2^-d, with the plan's exponent per (m, block) and
+// shift d per slot for y and an exponent per (m, block, row) measured in the CTA for X.  An MMA of 64 rows costs as much as one of
 // 128, so each MMA stacks two digits on both sides: A = [X_a ; X_(a+1)] (rows 0-63, 64-127) and
 // B = [Y_b | Y_(b+1)] (columns 0-31, 32-63), a and b even.  Its four quadrants collect
 // the classes a + b, a + b + 1 (two) and a + b + 2 in the accumulator region of t = a + b (0, 2, 4, 6).
@@ -79,6 +79,17 @@ __device__ __forceinline__ void umma_f16_ts_by(uint32_t issue, uint32_t tmem_d, 
         "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
         " @q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(tmem_d),
         "r"(tmem_a), "l"(b), "r"(idesc), "r"(acc), "r"(issue));
+}
+
+// v 2^-d, d <= 255, integer pipe only; a value that would leave the normal range becomes the smallest
+// subnormal, which marks a row that holds nothing larger; what is not finite stays
+__device__ __forceinline__ double shift_down(double v, int d)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    const int ex = (int)((hi >> 20) & 0x7ffu);
+    if (ex > d && ex < 0x7ff) return __hiloint2double((int)(hi - ((uint32_t)d << 20)), (int)lo);
+    if (ex == 0x7ff || ((hi << 1) | lo) == 0u) return v;
+    return __hiloint2double(0, 1);
 }
 
 __device__ __forceinline__ void tmem_ld4(uint32_t addr, uint32_t v[4])
@@ -189,6 +200,7 @@ __global__ void __launch_bounds__(TA_NT, 1) tc_anal_kernel(TcArgs A)
             const int rn = active ? A.slotN[slot] : -1, rs = active ? A.slotS[slot] : -1;
             const int64_t mstride = A.mmax + 1, dstride = (int64_t)A.nrings * mstride;
             double *xr = xs + r * TA_XROW;
+            const int sd = state_d(A.ck_k[(int64_t)(m * A.nblk + blk) * TC_T + r]);  // this slot's d
             const bool bn = rn >= 0 && SHT_CHK(rn < A.nrings), bs = rs >= 0 && SHT_CHK(rs < A.nrings);
             const double2 *dN = A.delta + (int64_t)(bn ? rn : 0) * mstride + m;
             const double2 *dS = A.delta + (int64_t)(bs ? rs : 0) * mstride + m;
@@ -207,11 +219,12 @@ __global__ void __launch_bounds__(TA_NT, 1) tc_anal_kernel(TcArgs A)
                         const double2 q = in ? d[0] : zero, w = in ? d[dstride] : zero;
                         const double re = c == 0 ? q.x - w.y : q.x + w.y, im = c == 0 ? q.y + w.x : q.y - w.x;
                         const bool neg = !own && m == 1;  // (-1)^(l+m) of the even rows, l - max(m, 2) even
+                        const double xre = shift_down(re, sd), xim = shift_down(im, sd);
                         double *x = xr + 2 * (2 * h + c);
-                        x[0] = neg ? -re : re;
-                        x[1] = neg ? -im : im;
-                        x[32] = own || neg ? re : -re;
-                        x[33] = own || neg ? im : -im;
+                        x[0] = neg ? -xre : xre;
+                        x[1] = neg ? -xim : xim;
+                        x[32] = own || neg ? xre : -xre;
+                        x[33] = own || neg ? xim : -xim;
                     }
                 }
             } else {
@@ -224,10 +237,10 @@ __global__ void __launch_bounds__(TA_NT, 1) tc_anal_kernel(TcArgs A)
                     const double2 n1 = bn && more ? dN[(g + 4) * dstride] : zero, s1 = bs && more ? dS[(g + 4) * dstride] : zero;
                     double *x = xr + 2 * g;
                     if (g < nm) {
-                        x[0] = n.x + s.x;
-                        x[1] = n.y + s.y;
-                        x[32] = n.x - s.x;
-                        x[33] = n.y - s.y;
+                        x[0] = shift_down(n.x + s.x, sd);
+                        x[1] = shift_down(n.y + s.y, sd);
+                        x[32] = shift_down(n.x - s.x, sd);
+                        x[33] = shift_down(n.y - s.y, sd);
                     } else {
                         x[0] = x[1] = x[32] = x[33] = 0.0;
                     }
@@ -332,6 +345,17 @@ __global__ void __launch_bounds__(TA_NT, 1) tc_anal_kernel(TcArgs A)
         // sg and sg + 8: its 8 values of a digit are one 16-byte core-matrix row
         const int w8 = warp - 4;
         const int n = (lane & 7) + 8 * (w8 & 3), sg0 = (lane >> 3) + 4 * (w8 >> 2);
+        // d of its 16 slots, a byte each
+        uint32_t sd[4];
+        {
+            const int *ck = A.ck_k + (int64_t)(m * A.nblk + blk) * TC_T + 8 * sg0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                sd[i] = 0;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) sd[i] |= (uint32_t)state_d(ck[64 * (i >> 1) + 4 * (i & 1) + j]) << (8 * j);
+            }
+        }
         for (int q = 0; q < nlive; ++q) {
             const int st = q & 1;
             bar_sync(BAR_FULL + st, TC_NT);  // y of chunk q is in its stage
@@ -340,11 +364,13 @@ __global__ void __launch_bounds__(TA_NT, 1) tc_anal_kernel(TcArgs A)
 #pragma unroll 1
             for (int i = 0; i < 2; ++i) {
                 const int sg = sg0 + 8 * i;
+                const uint32_t da = i ? sd[2] : sd[0], db = i ? sd[3] : sd[1];
                 uint32_t pk[4][TC_S];
 #pragma unroll
                 for (int p = 0; p < 4; ++p) {
                     const double2 v = *reinterpret_cast<const double2 *>(yb + 8 * sg + 2 * p);
-                    digit_pairs(digit_fields(v.x, Ey), digit_fields(v.y, Ey), pk[p]);
+                    const uint32_t w = (p < 2 ? da : db) >> (16 * (p & 1));
+                    digit_pairs(digit_fields(v.x, Ey - (int)(w & 255u)), digit_fields(v.y, Ey - (int)((w >> 8) & 255u)), pk[p]);
                 }
                 if (i == 1 && q + 2 < nlive) bar_arrive(BAR_EMPTY + st, TC_NT);  // y stage read
                 // the MMAs of chunk q - 2 read this tile set: wait (bounded) before rewriting it

@@ -117,7 +117,7 @@ struct Plan {
     int *d_tc_chunk_m = nullptr;        // [tc_total_chunks]
     int *d_tc_Ey = nullptr;             // [2][mmax + 1][slot blocks]: scale exponent of y = lambda / c, first live chunk
     double2 *d_tc_ck_y = nullptr;       // [mmax + 1][slot blocks][128] recurrence state at the first live chunk
-    int *d_tc_ck_k = nullptr;           // its rescaling exponents
+    int *d_tc_ck_k = nullptr;           // its rescaling exponents and the slots' scales (slot_state)
     int *d_status = nullptr;            // device status word (bounded waits that gave up)
     int *d_mflag = nullptr;             // [mmax + 1] m computed by the FP64 Legendre steps (null: all)
     int n_mlist = 0;                    // number of listed m (0: all)

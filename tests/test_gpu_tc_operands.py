@@ -122,3 +122,48 @@ def test_an_m_list_cuts_the_coefficients_of_its_m_only():
     b[:, oracle.alm_index(L, 1, 1):oracle.alm_index(L, 3, 3)] = 0.0
     p.set_mlist()
     assert torch.equal(p.alm2map(b), got) and not torch.equal(got, full)
+
+
+# Slots far below their block's scale, and what is bright on them.  The plain FP64 sums lose nothing to
+# the other slots of a block; bar 1e-11, the FP64 bar of the parity tests, against each column's own RMS
+# (analysis) and against each ring's own sum of |a_lm lambda_lm| (synthesis; above the dropping threshold).
+SLOTS, BAND = 150, 256
+
+
+def _slots_geom():
+    th = np.concatenate([[0.025, 0.03], np.linspace(0.05, 0.5 * np.pi - 0.01, SLOTS - 2)])
+    return np.full(SLOTS, 8, np.int64), th, np.zeros(SLOTS), np.ones(SLOTS)
+
+
+@pytest.mark.parametrize("nmaps", [1, 7, 16])
+def test_a_bright_polar_ring_leaves_the_other_columns_alone(nmaps):
+    geom, ms = _slots_geom(), [0, 1, 20, 60, 150, 250]
+    p = _plan(geom, BAND)
+    x = inputs.random_delta(SLOTS, BAND, seed=41, nmaps=nmaps)
+    x[:, 0] *= 1e9
+    x[:, 1] *= 1e6
+    b = host(p.legendre_anal(dev(x)))
+    for g in {0, nmaps - 1}:
+        ref = oracle.legendre_anal(geom, x[g].T[ms].copy(), BAND, np.array(ms))
+        for m, r in zip(ms, ref):
+            i = oracle.alm_index(BAND, m, m)
+            assert np.max(np.abs(b[g, i:i + BAND - m + 1] - r)) <= 1e-11 * np.sqrt(np.mean(np.abs(r) ** 2)), (g, m)
+
+
+@pytest.mark.parametrize("nmaps", [1, 16])
+def test_every_ring_keeps_its_own_precision(nmaps):
+    geom = _slots_geom()
+    p = _plan(geom, BAND)
+    a = inputs.uniform_alm(BAND, BAND, seed=43, nmaps=nmaps)
+    d = host(p.legendre_synth(dev(a)))
+    ref = oracle.delta_synth(geom, a[-1], BAND, BAND)
+    seen = 0
+    for m in (0, 5, 30, 80, 160, 250):
+        i = oracle.alm_index(BAND, m, m)
+        am = np.abs(a[-1, i:i + BAND - m + 1])
+        for r in range(0, SLOTS, 3):
+            tot = float(np.sum(am * np.abs(oracle.lambda_lm(float(geom[1][r]), BAND, m))))
+            if tot > 1e-50:
+                assert abs(d[-1, r, m] - ref[r, m]) <= 1e-11 * tot, (m, r)
+                seen += tot < 1e-12
+    assert seen > 10  # rings far below the others of their block
