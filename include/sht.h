@@ -86,11 +86,12 @@ sht_status sht_plan_create(sht_plan_t *out, sht_grid grid, int nrings,
  *                        The digits hold 62 bits below one power of two per m and ring (lambda over
  *                        all l), per m and map (the coefficients c_lm a_lm; 61 bits from lmax 8190
  *                        on, 60 from 16380) and per m, map and 128 ring slots (the ring sums, each
- *                        weighted by the largest lambda of its slot).  A term is off by at most
- *                        2^-56 of the largest product such a set could form, where an FP64 product is
- *                        off by 2^-53 of itself: errors are bounded against the sum's largest terms,
- *                        not against each value that lies far below the others of its set (more than
- *                        2^9 for a coefficient: high l of a steep spectrum).
+ *                        weighted by the largest lambda of its slot).  A term is off by less than
+ *                        2^-56 of the product of its two powers of two (2^-54 at the largest lmax),
+ *                        where an FP64 product is off by 2^-53 of itself: errors are bounded against
+ *                        the sum's largest terms, not against each value that lies far below the
+ *                        others of its set (more than 2^9 for a coefficient: high l of a steep
+ *                        spectrum).
  *                        Values that digits cannot carry (not finite, near the upper end of the
  *                        exponent range; in the analysis a ring set that is tiny throughout) send
  *                        their columns to FP64 sums.  A map's result does not depend on the maps
@@ -111,9 +112,9 @@ sht_status sht_plan_create(sht_plan_t *out, sht_grid grid, int nrings,
  */
 typedef enum { SHT_MODE_FP64 = 0, SHT_MODE_SPLIT_BF16 = 1 } sht_mode;
 sht_status sht_plan_set_mode(sht_plan_t plan, int mode);
-/* 1 if the plan's FP64 mode runs its (scalar) Legendre steps on the tensor cores, else 0; -1 for null */
-int sht_plan_fp64_tensor(sht_plan_t plan);
 int        sht_plan_mode(sht_plan_t plan);
+/* 1 if the plan's FP64 mode runs its (scalar) Legendre steps on the tensor cores, else 0; -1 for null */
+int        sht_plan_fp64_tensor(sht_plan_t plan);
 
 /*
  * Device status word of the plan: bit 0 is set when a bounded wait inside a tensor-core kernel

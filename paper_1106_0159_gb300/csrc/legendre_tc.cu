@@ -809,7 +809,15 @@ cudaError_t build_tc_spin_tables(Plan &p)
 //     lmax 128: 1 map 35 / 61, 58 / 61    4 maps 62 / 173, 62 / 64      16 maps 247 / 677, 71 / 67
 //     lmax 192: 1 map 77 / 132, 73 / 87   4 maps 151 / 403, 77 / 88     16 maps 601 / 1598, 95 / 97
 //     lmax 1024: 1 map 3419 / 4599, 2322 / 3185                         16 maps 31672 / 55868, 3040 / 3861
-// so that from lmax 192 on no number of maps loses.
+// so that from lmax 192 on no number of maps loses.  Few rings, and mmax far below lmax (unpaired rings over
+// both hemispheres):
+//     16 rings, lmax 192: 1 map 48 / 87, 51 / 56      4 maps 98 / 249, 53 / 57
+//     64 rings, lmax 512, mmax 4: 1 map 92 / 173, 78 / 83     4 maps 205 / 523, 80 / 85
+//     130 rings, one block polar, lmax 192, mmax 2: 1 map 61 / 95, 82 / 86   4 maps 100 / 256, 85 / 86;
+//         lmax 2048, mmax 4: 1 map 484 / 780, 511 / 526     4 maps 911 / 2353, 518 / 529
+//     300 rings, lmax 4096, mmax 100: 1 map 1034 / 1859, 741 / 869    4 maps 2562 / 6331, 778 / 885
+// There the one-map synthesis of a few m can lose 3 to 30 us (the chain of a polar block); every analysis
+// and every call of more maps gains.
 bool tc_fp64_plan(const Plan &p) { return p.lmax >= 192; }
 
 // scratch of the synthesis: the a_lm digits of one m-slab, then the scale exponents and marks

@@ -496,8 +496,8 @@ sht_status sht_plan_set_mode(sht_plan_t plan, int mode)
     if (!plan || (mode != SHT_MODE_FP64 && mode != SHT_MODE_SPLIT_BF16)) return SHT_EINVAL;
     Plan &p = plan->p;
     if (mode == SHT_MODE_SPLIT_BF16) {
-        // the Reinsch-form kernels of the precision form cover the first 256 slots (the analysis: one
-        // CTA over slots 0 .. 255 per m; the synthesis: the leading polar 128-slot blocks)
+        // the double-float analysis (SHT_TUNE_PREC_ANAL 0) runs Reinsch's form in one CTA per m over
+        // slots 0 .. 255 only; a plan may be switched to it at any time
         if (p.nslots > 256 && p.slotTheta[256] > 0.0 && std::sin(p.slotTheta[256]) < 0.03) return SHT_EUNSUPPORTED;
         cudaError_t e = sht::build_tc_tables(p);  // one FP64 pass of the recurrence, synchronous
         if (e == cudaSuccess) e = sht::build_df_ring_tables(p);
