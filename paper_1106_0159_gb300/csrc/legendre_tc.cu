@@ -47,10 +47,10 @@
 // P+- everywhere: the column of the pass's own sign on the northern rings (E + O), the other on the
 // southern ones (E - O).  spin_combine_kernel then forms Q and U.  4 FP64 instructions per step and
 // ring pair for up to 8 maps, where the FP64 kernels take 6 + 8 per map (lmax 1024, 1 map: whole synthesis
-// 20.7 -> 5.15 ms; analysis of 2 maps 32.5 -> 7.62 ms).
+// 20.7 -> 5.19 ms; analysis of 2 maps 32.5 -> 7.64 ms).
 //
 // What bounds it: the FP64 recurrence, 64 FP64 instructions per warp and chunk = 4096 SM cycles, and the
-// other roles' instructions that delay it (about 6.1K cycles a chunk at lmax 4096, 16 maps: 124 ms).
+// other roles' instructions that delay it (about 6.2K cycles a chunk at lmax 4096, 16 maps: 126 ms).
 #include "sht_internal.h"
 
 #include <algorithm>
