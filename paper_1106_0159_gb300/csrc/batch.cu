@@ -83,8 +83,10 @@ sht_status prepare(sht_batch_s &b)
     for (size_t j = 0; j < nj; ++j) {
         const sht::Plan &p = *b.plans[j];
         (p.tc64 ? b.tc : b.queued).push_back(j);
+        // enough for 16 maps a launch whatever the plan's knob: it may be set after the batch is made
         if (p.tc64)
-            b.tc_bytes = std::max(b.tc_bytes, al256(b.direction == 0 ? sht::tc_workspace_bytes(p, b.nmaps[j])
+            b.tc_bytes = std::max(b.tc_bytes, al256(b.direction == 0 ? std::max(sht::tc_workspace_bytes(p, b.nmaps[j]),
+                                                                                sht::tc_workspace_least(p, b.nmaps[j], 16))
                                                                      : sht::tc_anal_partial_bytes(p, b.nmaps[j])));
     }
     const int k = b.tune[SHT_BATCH_ANAL_SLOTS];

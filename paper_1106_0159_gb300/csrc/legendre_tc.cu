@@ -830,10 +830,10 @@ size_t tc_workspace_bytes(const Plan &p, int nmaps)
     return std::max(std::min(all, TC_SLAB_BYTES), one) + exponent_bytes(p) + 256;
 }
 
-// the least scratch the synthesis can run in (one m at a time)
-size_t tc_workspace_least(const Plan &p, int nmaps)
+// the least scratch the synthesis can run in (one m at a time); maps: per launch, 0 for the plan's knob
+size_t tc_workspace_least(const Plan &p, int nmaps, int maps)
 {
-    const int N = group_columns(std::min(nmaps, p.tune[SHT_TUNE_TC_MAPS]));
+    const int N = group_columns(std::min(nmaps, maps ? maps : p.tune[SHT_TUNE_TC_MAPS]));
     return (size_t)((p.lmax + TC_CH) / TC_CH) * chunk_bytes(N) + exponent_bytes(p) + 256;
 }
 

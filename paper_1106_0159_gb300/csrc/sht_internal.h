@@ -200,7 +200,7 @@ cudaError_t build_tc_tables(Plan &p);
 bool tc_fp64_plan(const Plan &p);                // the rule for Plan::tc64
 int64_t tc_chunks_below(const Plan &p, int m);   // 32-l chunks of all m' < m
 size_t tc_workspace_bytes(const Plan &p, int nmaps);
-size_t tc_workspace_least(const Plan &p, int nmaps);
+size_t tc_workspace_least(const Plan &p, int nmaps, int maps = 0);
 cudaError_t launch_legendre_synth_tc(const Plan &p, const double2 *alm, double2 *delta, void *scratch,
                                      size_t scratch_bytes, int nmaps, cudaStream_t st, int *nlaunch);
 cudaError_t launch_legendre_anal_tc(const Plan &p, const double2 *delta, double2 *alm, void *partial, int nmaps,

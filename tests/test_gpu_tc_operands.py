@@ -167,3 +167,21 @@ def test_every_ring_keeps_its_own_precision(nmaps):
                 assert abs(d[-1, r, m] - ref[r, m]) <= 1e-11 * tot, (m, r)
                 seen += tot < 1e-12
     assert seen > 10  # rings far below the others of their block
+
+
+def test_a_batch_follows_its_plans_knobs():
+    """The maps per launch set on a plan after the batch was made: the batch's own scratch serves both settings."""
+    from paper_1106_0159_gb300 import sht
+    p = _plan(RINGS, 400, 0)
+    a = dev(inputs.uniform_alm(400, 0, seed=51, nmaps=12))
+    want = p.alm2map(a)
+    p.set_tuning(sht.TUNE_TC_MAPS, 8)
+    out = torch.zeros_like(want)
+    b = sht.Batch(sht.BATCH_ALM2MAP, [(p, a, out)])
+    for maps in (16, 8):
+        p.set_tuning(sht.TUNE_TC_MAPS, maps)
+        out.zero_()
+        b.run()
+        torch.cuda.synchronize()
+        assert torch.equal(out, want)
+    b.close()
