@@ -89,12 +89,14 @@ sht_status sht_plan_create(sht_plan_t *out, sht_grid grid, int nrings,
  *                        weighted by the largest lambda of its slot).  A term is off by less than
  *                        2^-56 of the product of its two powers of two (2^-54 at the largest lmax),
  *                        where an FP64 product is off by 2^-53 of itself: errors are bounded against
- *                        the sum's largest terms, not against each value that lies far below the
+ *                        the largest terms of a map, not against each value that lies far below the
  *                        others of its set (more than 2^9 for a coefficient: high l of a steep
  *                        spectrum).
- *                        Values that digits cannot carry (not finite, near the upper end of the
- *                        exponent range; in the analysis a ring set that is tiny throughout) send
- *                        their columns to FP64 sums.  A map's result does not depend on the maps
+ *                        Columns that digits cannot carry go to FP64 sums: those with values that are
+ *                        not finite or near the upper end of the exponent range; in the analysis also
+ *                        a ring set that is tiny throughout, in the synthesis one whose terms all lie
+ *                        more than 2^9 below the product of its powers of two and are the map's
+ *                        largest (a single low l at high m on a polar cap).  A map's result does not depend on the maps
  *                        beside it.  Processes up to 16 maps per pass over the recurrence.
  *   SHT_MODE_SPLIT_BF16  the precision form: the same Legendre steps whatever lmax, and the ring
  *                        DFTs in double-float on the FP32 pipe.
@@ -107,7 +109,7 @@ sht_status sht_plan_create(sht_plan_t *out, sht_grid grid, int nrings,
  * The creation of a plan with lmax >= 192, or else the first switch to SHT_MODE_SPLIT_BF16, runs
  * one FP64 pass of the recurrence to measure the scale of its values per (m, block of 128 ring
  * slots) (synchronous; about the cost of one single-map synthesis).  These tables take 20 bytes per m
- * and ring slot; where there is no device memory for them, the plan is created all the same and its FP64
+ * and ring slot and 2 per coefficient; where there is no device memory for them, the plan is created all the same and its FP64
  * mode runs the plain FP64 kernels.  SHT_EINVAL for an unknown mode.
  */
 typedef enum { SHT_MODE_FP64 = 0, SHT_MODE_SPLIT_BF16 = 1 } sht_mode;

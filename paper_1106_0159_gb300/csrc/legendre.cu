@@ -496,11 +496,13 @@ __global__ void reduce_blocks_kernel(const double2 *__restrict__ partial, const 
 //
 // The tensor-core kernels cut their operands into digits below one exponent, which cannot carry a
 // value that is not finite or a column near the upper end of the FP64 range (analysis: the lower end
-// too).  They mark such (m, map) columns in fix[m][16], and these kernels redo them with the sums
+// too), nor, in the synthesis, a column whose terms all lie far below its scales (synth_marked).  They
+// mark such (m, map) columns, the analysis in fix[m][16], and these kernels redo them with the sums
 // above, one CTA per m (slow: every mark must be rare); without marks (every ordinary input) each
-// CTA reads its 16 marks and ends.
+// CTA reads its marks and ends.
 
-__global__ void __launch_bounds__(SYN_T) legendre_synth_fix_kernel(SynArgs A, const int *__restrict__ fix, int nmaps)
+__global__ void __launch_bounds__(SYN_T) legendre_synth_fix_kernel(SynArgs A, const int *__restrict__ reach,
+                                                                   const int *__restrict__ size, int nmaps)
 {
     __shared__ Coef C;
     __shared__ double2 s_a[1][CHL];
@@ -508,7 +510,7 @@ __global__ void __launch_bounds__(SYN_T) legendre_synth_fix_kernel(SynArgs A, co
     if (A.mflag && !A.mflag[m]) return;
     const int64_t dstride = (int64_t)A.nrings * (A.mmax + 1);
     for (int g = 0; g < nmaps; ++g) {
-        if (!fix[m * 16 + g]) continue;
+        if (!synth_marked<1>(reach, size, A.mflag, A.mmax, m, g)) continue;
         SynArgs B = A;
         B.alm += (int64_t)g * A.nalm;
         B.delta += (int64_t)g * dstride;
@@ -767,8 +769,8 @@ cudaError_t launch_legendre_anal(const Plan &p, const double2 *delta, double2 *p
     return cudaSuccess;
 }
 
-cudaError_t launch_legendre_synth_fix(const Plan &p, const double2 *alm, double2 *delta, const int *fix, int nmaps,
-                                      cudaStream_t st)
+cudaError_t launch_legendre_synth_fix(const Plan &p, const double2 *alm, double2 *delta, const int *reach,
+                                      const int *size, int nmaps, cudaStream_t st)
 {
     SynArgs A{};
     A.alm = alm;
@@ -788,7 +790,7 @@ cudaError_t launch_legendre_synth_fix(const Plan &p, const double2 *alm, double2
     A.mmax = p.mmax;
     A.nrings = p.nrings;
     A.nalm = p.nalm;
-    legendre_synth_fix_kernel<<<(unsigned)(p.mmax + 1), SYN_T, 0, st>>>(A, fix, nmaps);
+    legendre_synth_fix_kernel<<<(unsigned)(p.mmax + 1), SYN_T, 0, st>>>(A, reach, size, nmaps);
     return cudaGetLastError();
 }
 

@@ -119,27 +119,31 @@ __device__ __forceinline__ double c_factor(const TcArgs &A, int64_t ix)
 }
 
 // E_a[m][n] with |c_lm a_lm| < 2^E_a 2^-(lmax / 8190) for all l (from exponent fields, no FP64 work), and
-// the columns the digits cannot carry: a value that is not finite or a maximum near the upper end of the
-// FP64 range.  Subnormal values count as one of exponent field 1.
+// per map the exponents that decide which columns the digits cannot carry (synth_marked): a value that
+// is not finite or a maximum near the upper end of the FP64 range is one of them.  Subnormal values count
+// as one of exponent field 1.
 template <int N, bool SPIN>
 __global__ void tc_scale_kernel(TcArgs A)
 {
-    __shared__ int s_max[N];
+    __shared__ int s_max[N], s_size[N / 2], s_y;
     __shared__ int s_fix[N / 2];
     const int m = A.m0 + blockIdx.x;
     if (A.mflag && !A.mflag[m]) return;  // an m this plan does not compute: nothing reads its digits
     const int L = A.lmax;
     const int64_t base = (int64_t)m * (2 * L + 3 - m) / 2;
     if (threadIdx.x < N) s_max[threadIdx.x] = 0;
-    if (threadIdx.x < N / 2) s_fix[threadIdx.x] = 0;
+    if (threadIdx.x < N / 2) s_fix[threadIdx.x] = s_size[threadIdx.x] = 0;
+    if (threadIdx.x == 0) s_y = 0;
     __syncthreads();
-    int mx[N];
+    int mx[N], sz[N / 2];
     unsigned bad = 0;  // maps with a non-finite value
+#pragma unroll
+    for (int g = 0; g < N / 2; ++g) sz[g] = 0;
 #pragma unroll
     for (int n = 0; n < N; ++n) mx[n] = 0;
     for (int l = first_l<SPIN ? REC_SPIN : REC_Y>(m) + threadIdx.x; l <= L; l += blockDim.x) {
         const int64_t ix = base + (l - m);
-        const int ec = dexp(c_factor<SPIN>(A, ix));
+        const int ec = dexp(c_factor<SPIN>(A, ix)), ey = A.Yl[ix];
 #pragma unroll
         for (int g = 0; g < N / 2; ++g) {
             if (g < A.nmaps) {
@@ -148,6 +152,7 @@ __global__ void tc_scale_kernel(TcArgs A)
                 if (er == 0x7ff || ei == 0x7ff) bad |= 1u << g;
                 if (er) mx[2 * g] = max(mx[2 * g], er + ec);
                 if (ei) mx[2 * g + 1] = max(mx[2 * g + 1], ei + ec);
+                if (ey && (er | ei)) sz[g] = max(sz[g], max(er, ei) + ec + ey);
             }
         }
     }
@@ -156,6 +161,14 @@ __global__ void tc_scale_kernel(TcArgs A)
         const int w = (int)__reduce_max_sync(0xffffffffu, (unsigned)mx[n]);
         if ((threadIdx.x & 31) == 0) atomicMax(&s_max[n], w);
     }
+#pragma unroll
+    for (int g = 0; g < N / 2; ++g) {
+        const int w = (int)__reduce_max_sync(0xffffffffu, (unsigned)sz[g]);
+        if ((threadIdx.x & 31) == 0 && w) atomicMax(&s_size[g], w);
+    }
+    for (int pass = 0; pass < (SPIN ? 2 : 1); ++pass)  // the largest |y| of any slot (spin: of both signs)
+        for (int b = threadIdx.x; b < A.nblk; b += blockDim.x)
+            atomicMax(&s_y, A.Ey[(int64_t)pass * 2 * (A.mmax + 1) * A.nblk + m * A.nblk + b] + 1022);
     bad = __reduce_or_sync(0xffffffffu, bad);
     if ((threadIdx.x & 31) == 0)
         for (int g = 0; g < N / 2; ++g)
@@ -168,7 +181,11 @@ __global__ void tc_scale_kernel(TcArgs A)
         if (e > 1023 + TC_EHUGE) s_fix[threadIdx.x >> 1] = 1;
     }
     __syncthreads();
-    if (threadIdx.x < N / 2 && (int)threadIdx.x < A.nmaps) A.fix[m * 16 + threadIdx.x] = s_fix[threadIdx.x];
+    if (threadIdx.x < N / 2 && (int)threadIdx.x < A.nmaps) {
+        const int g = threadIdx.x, e = max(s_max[2 * g], s_max[2 * g + 1]);
+        A.reach[m * 16 + g] = s_fix[g] ? INT_MAX : e ? e + s_y : 0;
+        A.size[m * 16 + g] = s_size[g];
+    }
 }
 
 // digits of c_lm a_lm for one (m, chunk) in the tile layout of the MMA B operand:
@@ -229,11 +246,25 @@ __global__ void tc_split_b_kernel(TcArgs A)
 // ---------------------------------------------------------------- plan tables
 
 // Per (m, slot block): E with |y| < 2^E over the kept values of the block's slots and all l (-1000
-// when every value is dropped), how far each slot's own exponent lies below it, the first chunk of 32 l in which any slot keeps a value (every
-// earlier chunk contributes exactly zero), and the recurrence state (y1, y2, k) of every slot at the
-// start of that chunk, where the tensor-core kernels begin (at lmax 4096 on HEALPix about a quarter
-// of the steps lie before it).  Same recurrence, operation for operation, as recurrence_warps, so
-// that both see the same rescaling steps and the same values.
+// when every value is dropped), how far each slot's own exponent lies below it, the first chunk of
+// 32 l in which any slot keeps a value (every earlier chunk contributes exactly zero), and the
+// recurrence state (y1, y2, k) of every slot at the start of that chunk, where the tensor-core kernels
+// begin (at lmax 4096 on HEALPix about a quarter of the steps lie before it).  Same recurrence, operation
+// for operation, as recurrence_warps, so that both see the same rescaling steps and the same values.
+
+// lambda of the first l at one slot, y0 2^(512 k)
+template <int KIND>
+__device__ __forceinline__ void slot_start(const TcArgs &A, int m, int64_t base, int slot, double u, double &y0, int &k)
+{
+    if (KIND == REC_SPIN) {  // S_m sin^|m-2| times sin^p(theta/2) (+) or sigma cos^p(theta/2) (-): spin.cu
+        sectoral_start(A.s[slot], A.start[m], m >= 2 ? m - 2 : 2 - m, y0, k);
+        const double f = A.sig > 0 ? 0.5 * u : 1.0 - 0.5 * u;
+        y0 *= m >= 2 ? f * f : m == 1 ? (A.sig > 0 ? f : -f) : 1.0;
+    } else {
+        sectoral_start(A.s[slot], A.alpha[base], m, y0, k);
+    }
+}
+
 template <int KIND>
 __device__ __forceinline__ void tables_body(const TcArgs &A, int m, int blk, int *s_max, int *s_first, RecCoef *s_c,
                                             double2 *ck_y, int *ck_k)
@@ -251,13 +282,7 @@ __device__ __forceinline__ void tables_body(const TcArgs &A, int m, int blk, int
     if (active) {
         u = A.u[slot];
         double y0;
-        if (KIND == REC_SPIN) {  // S_m sin^|m-2| times sin^p(theta/2) (+) or sigma cos^p(theta/2) (-): spin.cu
-            sectoral_start(A.s[slot], A.start[m], m >= 2 ? m - 2 : 2 - m, y0, k);
-            const double f = A.sig > 0 ? 0.5 * u : 1.0 - 0.5 * u;
-            y0 *= m >= 2 ? f * f : m == 1 ? (A.sig > 0 ? f : -f) : 1.0;
-        } else {
-            sectoral_start(A.s[slot], A.alpha[base], m, y0, k);
-        }
+        slot_start<KIND>(A, m, base, slot, u, y0, k);
         y2 = KIND == REC_REIN ? y0 : -y0;
     }
     double c1 = y1, c2 = y2;  // state at the start of the first live chunk
@@ -329,6 +354,64 @@ __global__ void __launch_bounds__(TC_T) tc_tables_kernel(TcArgs A, int *Ey_out, 
     if (threadIdx.x == 0) {
         Ey_out[m * A.nblk + blk] = s_max ? s_max - 1022 : -1000;
         first_out[m * A.nblk + blk] = s_first;
+    }
+}
+
+// Exponent field of the largest kept |y_l| per (m, l) of up to 128 slots spread evenly over the grid, the
+// most equatorward one among them; 0 where all are dropped (spin: of both signs of the recurrence).  One
+// CTA per m, the y form or spin's recurrence: only exponents count.  2 bytes per coefficient.
+template <bool SPIN>
+__global__ void __launch_bounds__(TC_T) tc_top_kernel(TcArgs A, uint16_t *__restrict__ Yl)
+{
+    constexpr int KIND = SPIN ? REC_SPIN : REC_Y;
+    __shared__ RecCoef s_c[TC_CH];
+    __shared__ int s_m[TC_CH];
+    const int m = blockIdx.x, tid = threadIdx.x;
+    const bool active = tid < A.nslots;
+    const int slot = A.nslots <= TC_T ? tid : A.nslots - 1 - (int)((int64_t)tid * (A.nslots - 1) / (TC_T - 1));
+    const int L = A.lmax, lb = first_l<KIND>(m);
+    const int64_t base = (int64_t)m * (2 * L + 3 - m) / 2;
+    for (int l = m + tid; l < min(lb, L + 1); l += TC_T) Yl[base + l - m] = 0;
+    for (int pass = 0; pass < (SPIN ? 2 : 1); ++pass) {
+        A.sig = pass == 0 ? 1 : -1;
+        double u = 0.0, y1 = 0.0, y2 = 0.0;
+        int k = 0;
+        if (active) {
+            u = A.u[slot];
+            double y0;
+            slot_start<KIND>(A, m, base, slot, u, y0, k);
+            y2 = -y0;
+        }
+        for (int l0 = lb; l0 <= L; l0 += TC_CH) {
+            __syncthreads();
+            if (tid < TC_CH) {
+                s_c[tid] = load_coef<KIND>(A, base, m, l0 + tid);
+                s_m[tid] = 0;
+            }
+            __syncthreads();
+            for (int h = 0; h < 2; ++h) {
+                const bool scaled = __any_sync(0xffffffffu, k < 0);
+                const bool drop = scaled && k < 0;
+                for (int j = 16 * h; j < 16 * h + 16; ++j) {
+                    const RecCoef C = s_c[j];
+                    const double y = fma(fma(-C.a, u, KIND == REC_SPIN ? C.rh : C.a), y1, -y2);
+                    y2 = y1;
+                    y1 = y;
+                    const unsigned e = __reduce_max_sync(0xffffffffu, (unsigned)(drop || !active ? 0 : dexp(y)));
+                    if ((tid & 31) == 0) atomicMax(&s_m[j], (int)e);
+                }
+                if (drop && max(dexp(y1), dexp(y2)) > RESCALE_THR) {
+                    y1 *= 0x1p-512;
+                    y2 *= 0x1p-512;
+                    k += 1;
+                }
+            }
+            __syncthreads();
+            if (tid < TC_CH && l0 + tid <= L) {
+                uint16_t *o = Yl + base + (l0 - m) + tid;
+                *o = (uint16_t)(pass == 0 ? s_m[tid] : max((int)*o, s_m[tid]));
+            }
+        }
     }
 }
 
@@ -732,7 +815,7 @@ int slab_end(const Plan &p, int m0, int N, size_t cap)
     return lo;
 }
 
-size_t exponent_bytes(const Plan &p) { return (size_t)(p.mmax + 1) * (32 + 16) * sizeof(int); }
+size_t exponent_bytes(const Plan &p) { return (size_t)(p.mmax + 1) * (32 + 2 * 16) * sizeof(int); }
 
 }  // namespace
 
@@ -764,11 +847,11 @@ static cudaError_t build_tables(const Plan &p, bool spin, int **ey_out, double2 
     A.nblk = (p.nslots + TC_T - 1) / TC_T;
     A.lmax = p.lmax;
     A.mmax = p.mmax;
-    int *ey = nullptr;  // per sign [2][mmax + 1][nblk]: y exponents, then first live chunks
+    int *ey = nullptr;  // per sign [2][mmax + 1][nblk]: y exponents, then first live chunks; last uint16 [nalm]
     const size_t n = (size_t)(p.mmax + 1) * A.nblk, ns = spin ? 2 : 1;
     double2 *cky = nullptr;
     int *ckk = nullptr;
-    cudaError_t e = sht::dev_malloc(&ey, sizeof(int) * 2 * n * ns);
+    cudaError_t e = sht::dev_malloc(&ey, sizeof(int) * 2 * n * ns + sizeof(uint16_t) * (size_t)p.nalm);
     if (e == cudaSuccess) e = sht::dev_malloc(&cky, sizeof(double2) * n * TC_T * ns);
     if (e == cudaSuccess) e = sht::dev_malloc(&ckk, sizeof(int) * n * TC_T * ns);
     for (size_t k = 0; k < ns && e == cudaSuccess; ++k) {
@@ -778,6 +861,14 @@ static cudaError_t build_tables(const Plan &p, bool spin, int **ey_out, double2 
             tc_tables_kernel<true><<<(unsigned)n, TC_T>>>(A, ek, ek + n, cky + n * TC_T * k, ckk + n * TC_T * k);
         else
             tc_tables_kernel<false><<<(unsigned)n, TC_T>>>(A, ek, ek + n, cky, ckk);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) {
+        uint16_t *yl = (uint16_t *)(ey + 2 * n * ns);
+        if (spin)
+            tc_top_kernel<true><<<(unsigned)(p.mmax + 1), TC_T>>>(A, yl);
+        else
+            tc_top_kernel<false><<<(unsigned)(p.mmax + 1), TC_T>>>(A, yl);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -857,6 +948,7 @@ static cudaError_t synth_tc(const Plan &p, bool spin, const double2 *alm, double
     A.nblk = (p.nslots + TC_T - 1) / TC_T;
     A.Ey = spin ? p.d_sp_Ey : p.d_tc_Ey;
     A.first = A.Ey + (size_t)(p.mmax + 1) * A.nblk;
+    A.Yl = (const uint16_t *)(A.Ey + (size_t)(spin ? 4 : 2) * (p.mmax + 1) * A.nblk);
     A.ck_y = spin ? p.d_sp_ck_y : p.d_tc_ck_y;
     A.ck_k = spin ? p.d_sp_ck_k : p.d_tc_ck_k;
     A.chunk_base = p.d_tc_chunk_base;
@@ -869,8 +961,9 @@ static cudaError_t synth_tc(const Plan &p, bool spin, const double2 *alm, double
     A.mR = p.mR;
     A.nalm = p.nalm;
     A.mflag = spin ? nullptr : p.d_mflag;
-    A.fix = (int *)scratch;  // [mmax + 1][16], then Ea [mmax + 1][N], then the digits
-    A.Ea = A.fix + (size_t)(p.mmax + 1) * 16;
+    A.reach = (int *)scratch;  // [mmax + 1][16], size the same, then Ea [mmax + 1][N], then the digits
+    A.size = A.reach + (size_t)(p.mmax + 1) * 16;
+    A.Ea = A.size + (size_t)(p.mmax + 1) * 16;
     const size_t head = (exponent_bytes(p) + 255) & ~(size_t)255;
     A.bdig = (uint4 *)((char *)scratch + head);
     const size_t cap = scratch_bytes - head;
@@ -905,9 +998,9 @@ static cudaError_t synth_tc(const Plan &p, bool spin, const double2 *alm, double
             spin_combine_kernel<<<152 * 16, 256, 0, st>>>(A.delta, dstride, nm / 2);
             ++*nlaunch;
             e = cudaGetLastError();
-            if (e == cudaSuccess) e = launch_spin_synth_fix(p, A.alm, A.delta, A.fix, nm / 2, st);
+            if (e == cudaSuccess) e = launch_spin_synth_fix(p, A.alm, A.delta, A.reach, A.size, nm / 2, st);
         } else {
-            e = launch_legendre_synth_fix(p, A.alm, A.delta, A.fix, nm, st);
+            e = launch_legendre_synth_fix(p, A.alm, A.delta, A.reach, A.size, nm, st);
         }
         *nlaunch += 1;
         if (e != cudaSuccess) return e;

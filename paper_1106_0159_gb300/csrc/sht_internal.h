@@ -115,7 +115,8 @@ struct Plan {
     int64_t tc_total_chunks = 0;        // sum over m of ceil((lmax - m + 1) / 32)
     int64_t *d_tc_chunk_base = nullptr; // [mmax + 1]
     int *d_tc_chunk_m = nullptr;        // [tc_total_chunks]
-    int *d_tc_Ey = nullptr;             // [2][mmax + 1][slot blocks]: scale exponent of y = lambda / c, first live chunk
+    int *d_tc_Ey = nullptr;             // [2][mmax + 1][slot blocks]: scale exponent of y = lambda / c, first live
+                                        // chunk; then as uint16 [nalm] the exponent of the largest y_l
     double2 *d_tc_ck_y = nullptr;       // [mmax + 1][slot blocks][128] recurrence state at the first live chunk
     int *d_tc_ck_k = nullptr;           // its rescaling exponents and the slots' scales (slot_state)
     int *d_status = nullptr;            // device status word (bounded waits that gave up)
@@ -207,8 +208,8 @@ cudaError_t launch_legendre_anal_tc(const Plan &p, const double2 *delta, double2
                                     cudaStream_t st, int *nlaunch);
 size_t tc_anal_partial_bytes(const Plan &p, int nmaps);
 cudaError_t configure_tc_anal_kernel();
-cudaError_t launch_legendre_synth_fix(const Plan &p, const double2 *alm, double2 *delta, const int *fix, int nmaps,
-                                      cudaStream_t st);
+cudaError_t launch_legendre_synth_fix(const Plan &p, const double2 *alm, double2 *delta, const int *reach,
+                                      const int *size, int nmaps, cudaStream_t st);
 cudaError_t launch_legendre_anal_fix(const Plan &p, const double2 *delta, double2 *alm, double2 *partial, const int *fix,
                                      int nmaps, int m0, int m1, int64_t idx0, int64_t nalm_part, cudaStream_t st);
 
@@ -217,8 +218,8 @@ cudaError_t launch_spin_synth_tc(const Plan &p, const double2 *alm, double2 *del
                                  int nmaps, cudaStream_t st, int *nlaunch);
 cudaError_t launch_spin_anal_tc(const Plan &p, const double2 *delta, double2 *alm, void *partial, int nmaps,
                                 cudaStream_t st, int *nlaunch);
-cudaError_t launch_spin_synth_fix(const Plan &p, const double2 *alm, double2 *delta, const int *fix, int nmaps,
-                                  cudaStream_t st);
+cudaError_t launch_spin_synth_fix(const Plan &p, const double2 *alm, double2 *delta, const int *reach, const int *size,
+                                  int nmaps, cudaStream_t st);
 cudaError_t launch_spin_anal_fix(const Plan &p, const double2 *delta, double2 *alm, double2 *partial, const int *fix,
                                  int nmaps, int m0, int m1, int64_t idx0, int64_t nalm_part, cudaStream_t st);
 

@@ -201,14 +201,15 @@ __global__ void __launch_bounds__(SP_T) spin_synth_kernel(SpinArgs A)
     spin_synth_body<NM>(A, blockIdx.x / A.nblk, blockIdx.x % A.nblk, s_t, s_e, s_b);
 }
 
-// the maps whose columns the tensor-core kernels left (fix[m][2 g], fix[m][2 g + 1]; see legendre.cu)
-__global__ void __launch_bounds__(SP_T) spin_synth_fix_kernel(SpinArgs A, const int *__restrict__ fix, int nmaps)
+// the maps whose columns 2 g, 2 g + 1 the tensor-core kernels left (see legendre.cu)
+__global__ void __launch_bounds__(SP_T) spin_synth_fix_kernel(SpinArgs A, const int *__restrict__ reach,
+                                                              const int *__restrict__ size, int nmaps)
 {
     __shared__ double4 s_t[SP_CH];
     __shared__ double2 s_e[1][SP_CH], s_b[1][SP_CH];
     const int m = blockIdx.x;
     for (int g = 0; g < nmaps; ++g) {
-        if (!fix[m * 16 + 2 * g] && !fix[m * 16 + 2 * g + 1]) continue;
+        if (!synth_marked<2>(reach, size, nullptr, A.mmax, m, 2 * g)) continue;
         SpinArgs B = A;
         B.alm += (int64_t)g * 2 * A.nalm;
         B.delta += (int64_t)g * 2 * A.nrings * (A.mmax + 1);
@@ -557,14 +558,14 @@ cudaError_t launch_spin_anal(const Plan &p, const double2 *delta, double2 *alm, 
     return cudaSuccess;
 }
 
-cudaError_t launch_spin_synth_fix(const Plan &p, const double2 *alm, double2 *delta, const int *fix, int nmaps,
-                                  cudaStream_t st)
+cudaError_t launch_spin_synth_fix(const Plan &p, const double2 *alm, double2 *delta, const int *reach, const int *size,
+                                  int nmaps, cudaStream_t st)
 {
     SpinArgs A = spin_args(p);
     A.alm = alm;
     A.delta = delta;
     A.nmaps = 1;
-    spin_synth_fix_kernel<<<(unsigned)(p.mmax + 1), SP_T, 0, st>>>(A, fix, nmaps);
+    spin_synth_fix_kernel<<<(unsigned)(p.mmax + 1), SP_T, 0, st>>>(A, reach, size, nmaps);
     return cudaGetLastError();
 }
 

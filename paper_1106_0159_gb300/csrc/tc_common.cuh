@@ -227,7 +227,9 @@ struct TcArgs {
     const double2 *ck_y;     // [mmax+1][nblk][128] recurrence state at chunk first
     const int *ck_k;         // [mmax+1][nblk][128] rescaling exponents k there, with the slot's scale (slot_state)
     int *Ea;                 // synthesis: [mmax+1][N] scale exponent of c a
-    int *fix;                // [mmax+1][16] 1: the map's column of this m is left to the plain FP64 sums
+    int *fix;                // analysis: [mmax+1][16] 1: the map's column of this m is left to the plain FP64 sums
+    int *reach, *size;       // synthesis: [mmax+1][16] each, the same decided from them (synth_marked)
+    const uint16_t *Yl;      // synthesis: [nalm] exponent field of the largest |y_l| of the grid (tc_top_kernel)
     const int64_t *chunk_base;  // [mmax+1] first chunk of each m
     const int *chunk_m;      // [total chunks] m of each chunk
     uint4 *bdig;             // synthesis: [chunks of the slab][B_CHUNK / 16]
